@@ -20,7 +20,9 @@
 // the resampling is fused into this load) and written to the next buffers.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <mutex>
+#include <type_traits>
 #include <unordered_map>
 
 #include "pa_internal.cuh"
@@ -48,13 +50,16 @@ __device__ __forceinline__ uint32_t prmt_sign(uint32_t a, uint32_t b, uint32_t s
     return d;
 }
 
-// Entry i of a decision table in 16-bit lanes (the multi-spin-coded and the
-// packed kernels): E(m) in both halves, m = i - 32 for counts of |m| <= 31
-// kept as byte offsets 4m + 128, else m = i - 128 (word index). With the top
-// byte of the uniform, lane = 128 top + E is below 0x8000 iff the move is
-// accepted, 0x8000 exactly on a tie that the low bits decide.
-__device__ __forceinline__ uint32_t msc_entry(int i, bool pk, const uint32_t *tab, int mmax) {
-    const int m = pk ? i - 32 : i - 128;
+// Entry of m in the packed kernel's decision table: E(m) in both 16-bit
+// halves. Two replicas are decided by one 32-bit multiply-add in 16-bit lanes,
+// lane = 128 top + E(m) with the top byte of the uniform (t8 = T[m] >> 24):
+//   E = 0x8000 - 128 t8:  lane < 0x8000 iff top < t8 (accept),
+//                         lane = 0x8000 iff top = t8 (tie),
+//   + 64 when T[m] has no low bits (a tie rejects), 0x8040 when T[m] = 0,
+//   1 for m <= 0 (always accepted).
+// Every lane stays in [1, 0xFFC0], so lanes never carry into each other; bit
+// 15 of a lane is "reject or tie" and bit 15 of lane - 1 is "reject".
+__device__ __forceinline__ uint32_t pk_entry(int m, const uint32_t *tab, int mmax) {
     uint32_t e = 1u;   // m <= 0: always accepted
     if (m > 0) {
         const uint32_t T = m <= mmax ? tab[m] : 0u;
@@ -347,7 +352,7 @@ __device__ __forceinline__ void pk_decide(const uint32_t *__restrict__ Bsm, cons
     const uint32_t hb = (b & 0xFEFEFEFEu) | (par * 0x01010101u);
     const uint32_t mb = (hb ^ (smask * 0xFFu)) + smask;
     const uint32_t uw = word_of(philox10(make_uint4(vid, c1 >> 2, (uint32_t)a.k, c3), a.key0, a.key1), c1 & 3u);
-    // The four decisions in 16-bit lanes, as in the multi-spin-coded item.
+    // The four decisions in 16-bit lanes (pk_entry).
     const uint32_t e0 = T256[mb & 0xFFu], e1 = T256[(mb >> 8) & 0xFFu];
     const uint32_t e2 = T256[(mb >> 16) & 0xFFu], e3 = T256[mb >> 24];
     const uint32_t slo = __byte_perm(uw, 0u, 0x4140u) * 128u + __byte_perm(e0, e1, 0x5410u);
@@ -436,7 +441,7 @@ __global__ void __launch_bounds__(NTB, MINB) k_sweep_packed(const SweepArgs a) {
     const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31;
     uint2 *Q = Qall + (size_t)(tid >> 5) * PK_QCAP;
     const uint32_t *tab = a.tables + (size_t)a.tidx[a.k] * (a.g.mmax + 1);
-    for (int i = tid; i < 256; i += NT) T256[i] = msc_entry(i, false, tab, a.g.mmax);   // by m + 128
+    for (int i = tid; i < 256; i += NT) T256[i] = pk_entry(i - 128, tab, a.g.mmax);   // by m + 128
     for (int i = tid; i <= a.g.ncol; i += NT) cls[i] = a.g.cls[i];
     for (int i = tid; i < npw; i += NT) Psm[i] = a.g.parity[i];
 
@@ -584,34 +589,38 @@ __global__ void __launch_bounds__(NTB, MINB) k_sweep_packed(const SweepArgs a) {
 
 // ---------------------------------------------------------------------------
 // Multi-spin-coded variant: W[p] holds the spins of 32 replicas (slots
-// 32*blk .. 32*blk+31) at position p, 1 for +1. Replica 4g + q (group g of
-// the Philox call that serves it, word q) sits at bit 8q + g, so that a
-// group's four replicas are one bit of each byte. No fields are kept:
-// an item (p, word) XORs its word with each neighbour's word (and with all
-// ones for a -1 weight), so bit r of d_j is 1 iff the bond (p, j) contributes
-// +1 to m_r = -x_p h_p; a bit-sliced counter over the neighbours (carry-save
-// adders, four bonds per step) gives c_r and m_r = 2 c_r - deg(p). An 8 x 8
-// bit transpose in every byte lane turns the counter planes into one byte per
-// replica, group by group. The uniforms of the group's four replicas have
-// their top bytes in one Philox word (word g & 3 of the call of slots
-// 16 (slot >> 4) ..): byte q belongs to replica 4g + q, the same byte as its
-// count. With |m| <= 31 the count byte holds 4m + 128, which is also the byte
-// offset of the entry of m in a table kept at the start of shared memory, so
-// the lookup needs no address arithmetic (wider counts: m + 128, a word index).
-// An entry holds a 16-bit value E(m) in both halves. Two replicas are decided
-// by one 32-bit multiply-add in 16-bit lanes, lane = 128 top + E(m):
-//   E = 0x8000 - 128 t8 (t8 = T[m] >> 24):  lane < 0x8000 iff top < t8 (accept),
-//                                           lane = 0x8000 iff top = t8 (tie),
-//   + 64 when T[m] has no low bits (a tie rejects), 0x8040 when T[m] = 0,
-//   1 for m <= 0 (always accepted).
-// Every lane stays in [1, 0xFFC0], so lanes never carry into each other; bit
-// 15 of a lane is "reject or tie" and bit 15 of lane - 1 is "reject". A byte
-// permute replicating those sign bits turns the four lanes of a group into
-// byte masks. A tie (probability 1/256 per uncertain attempt) is settled by
-// the low 24 bits of the uniform, drawn only then: the ties of a warp's items
-// are queued and settled by all 32 lanes together before the class barrier
-// (one tail Philox call per lane instead of one per tying lane while the
-// others wait). Accepted replicas flip with one XOR.
+// 32*blk .. 32*blk+31) at position p, 1 for +1. Replica 4g + q (byte q of
+// word g of its Philox calls) sits at bit 8q + g. No fields are kept.
+//
+// An item (p, word) makes 32 attempts with bit-sliced arithmetic from the
+// neighbour words to the decisions; a plane is one word holding one binary
+// digit of a number for each of the 32 replicas.
+//   count     XOR with each neighbour's word (and with all ones for a -1
+//             weight) gives the frustrated-bond bits; carry-save adders count
+//             them. The counter starts at -(deg/2 + 1), so it ends as
+//             e = c - deg/2 - 1 in N-bit two's complement: its top plane says
+//             m <= 0, and m = 2e + 1 (odd degree) or 2e + 2 (even degree).
+//   uniforms  the 32 top bytes of the two Philox calls are turned into eight
+//             planes by an 8 x 8 bit transpose in every byte lane.
+//   decision  the planes of the threshold's top byte are OR-ed together from
+//             the values of m whose T[m] has a non-zero top byte (from none
+//             above beta = 2.8 to about 2.8 / beta); one comparison of eight
+//             planes then gives "below" (accepted) and "equal" (a tie, which
+//             the low 24 bits decide) for all 32 replicas.
+//   energy    m of the accepted replicas is added to bit-sliced accumulators.
+// What it replaces: the counts were transposed to one byte per replica, each
+// group of four replicas was decided by two look-ups in a pair table and two
+// multiply-adds in 16-bit lanes, and the energies went to byte counters
+// flushed after every colour class: about 200 of 560 instructions per item.
+// Bound: the ALU pipe (three-input logic and shifts) and, with few large
+// colour classes' worth of warps per SM, latency. Measured per step of 10
+// sweeps, means over beta 0.2 .. 3.6, R = 16384: G63-shaped (N = 7000) 0.981 ->
+// 0.872 ms, signed torus (N = 10000) 1.030 -> 0.843 ms.
+//
+// A tie (probability 1/256 per uncertain attempt) is queued with its counter
+// planes, and the ties of a warp's items are settled by all 32 lanes together
+// before the class barrier (one tail Philox call per lane). Accepted replicas
+// flip with one XOR.
 __device__ __forceinline__ int msc_bit(int r) {   // bit of replica r = 4g + q in a word
     return 8 * (r & 3) + (r >> 2);
 }
@@ -659,9 +668,9 @@ __device__ __forceinline__ void msc_unpack_rows(const uint32_t (&w4)[4], int8_t 
     }
 }
 
-// Philox4x32-10 for the eight counters (c0, c1_g, c2, c3) of one item, which
-// differ only in word 1: the products of rounds 1-3 whose inputs do not depend
-// on c1 are computed once (the result is identical to philox10 of each counter).
+// Philox4x32-10 for the counters (c0, c1_g, c2, c3) of one item, which differ
+// only in word 1: the products of rounds 1-3 whose inputs do not depend on c1
+// are computed once (the result is identical to philox10 of each counter).
 struct PhiloxShared {
     uint32_t u1;      // round 1: hi(M1 c2) ^ k0        (uniform)
     uint32_t l1;      // round 1: lo(M1 c2)              (uniform)
@@ -682,58 +691,6 @@ __device__ __forceinline__ PhiloxShared philox_shared(uint32_t c0, uint32_t c2, 
     p.s0 = hi ^ p.l1 ^ (k0 + 0x9E3779B9u);
     mul_wide(0xD2511F53u, p.s0, p.l3, p.h3);
     return p;
-}
-
-// Energy bookkeeping of the multi-spin-coded kernels. With |m| <= 31
-// (NPL <= 5) every item adds, per replica 4g + q, 32 + m for an accepted flip
-// and 32 for a rejected attempt into byte q of the lane's word ebias[g]; four
-// items stay below 256 in every byte. After at most four items per lane the
-// warp flushes: the 16-bit halves of the words are summed over the 32 lanes
-// (at most 32 * 252 < 2^16, so no half carries into the next), the bias of 32
-// per item is removed and lane r adds twice the result, the energy change of
-// replica r, to Eacc[r]. This replaces one divergent shared atomic per accepted
-// flip by branch-free byte arithmetic; the sums are exact integers, so the
-// energies are the same as with per-flip updates. Wider counters (|m| up to
-// 127) keep the per-flip atomics.
-template <int NPL>
-struct MscPackedE {
-    static constexpr bool value = NPL <= 5;
-};
-
-// Pair decision table of the packed-energy items: entry (m0 + H/2) + H (m1 + H/2)
-// holds E(m0) in its low and E(m1) in its high 16-bit lane, H = 2^(NPL+1)
-// (|m| < H/2). One load decides two replicas; the byte offset of the entry
-// is one dot product of the item's index bytes 4(m + H/2) with (1, H).
-template <int NPL>
-struct MscPairTab {
-    static constexpr int H = 2 << NPL;
-    static constexpr int words = MscPackedE<NPL>::value ? H * H : 0;
-};
-
-__host__ __device__ inline int msc_pair_words(int mmax) {
-    return mmax <= 7 ? 256 : mmax <= 15 ? 1024 : mmax <= 31 ? 4096 : 0;
-}
-
-template <int NPL>
-__device__ __forceinline__ void msc_fill_pair_table(uint32_t *PT, const uint32_t *T256, int tid, int NT) {
-    constexpr int H = MscPairTab<NPL>::H;
-    for (int i = tid; i < MscPairTab<NPL>::words; i += NT)
-        PT[i] = (T256[i % H - H / 2 + 32] & 0xFFFFu) | (T256[i / H - H / 2 + 32] & 0xFFFF0000u);
-}
-
-__device__ __forceinline__ void msc_flush_energy(uint32_t (&ebias)[8], int &cnt, int32_t *Eacc, int lane) {
-    const int nwarp = (int)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)cnt);
-    uint32_t mine = 0;
-#pragma unroll
-    for (int g = 0; g < 8; ++g) {
-        const uint32_t slo = __reduce_add_sync(0xFFFFFFFFu, ebias[g] & 0x00FF00FFu);          // bytes 0, 2
-        const uint32_t shi = __reduce_add_sync(0xFFFFFFFFu, (ebias[g] >> 8) & 0x00FF00FFu);   // bytes 1, 3
-        if ((lane >> 2) == g) mine = (lane & 1) ? shi : slo;
-        ebias[g] = 0u;
-    }
-    const int dm = (int)((lane & 2) ? (mine >> 16) : (mine & 0xFFFFu)) - 32 * nwarp;
-    if (dm) atomicAdd(&Eacc[lane], 2 * dm);
-    cnt = 0;
 }
 
 // Philox4x32-10 of two counters of one item (word 1 = c1a, c1b), finished
@@ -769,428 +726,445 @@ __device__ __forceinline__ void philox_from_shared2(const PhiloxShared &p, uint3
     rb = b;
 }
 
-// One (position, word) item of a multi-spin-coded sweep: counts the frustrated
-// bonds of the 32 replicas, decides the 32 attempts and records the energy
-// change of every accepted flip, either in the lane's packed counters ebias
-// (MscPackedE) or by a shared atomic on Eacc (local or a cluster peer's shared
-// memory). Returns the mask of accepted replicas.
-// Adds four bonds to the bit-sliced counters pl (one counter per replica):
-// bit r of d_j = x ^ w_j is 1 iff bond j contributes +1 to m_r. Carry-save
-// adders: d0 + d1 = s01 + 2 c01, d0 + .. + d3 = s + 2 (c01 + c23 + cs).
-template <int NPL>
-__device__ __forceinline__ void msc_csa4(uint32_t (&pl)[NPL], uint32_t x, uint32_t w0, uint32_t w1, uint32_t w2,
-                                         uint32_t w3) {
-    const uint32_t s01 = w0 ^ w1, c01 = (x ^ w0) & (x ^ w1);
-    const uint32_t s23 = w2 ^ w3, c23 = (x ^ w2) & (x ^ w3);
-    const uint32_t s = s01 ^ s23, cs = s01 & s23;
-    const uint32_t t = pl[0] & s;
-    pl[0] ^= s;
-    const uint32_t u1 = pl[1] ^ c01 ^ c23, k1 = (pl[1] & c01) | (c23 & (pl[1] | c01));
-    const uint32_t k2 = (u1 & cs) | (t & (u1 | cs));
-    pl[1] = u1 ^ cs ^ t;
-    uint32_t k = (pl[2] & k1) | (k2 & (pl[2] | k1));
-    pl[2] ^= k1 ^ k2;
-#pragma unroll
-    for (int b = 3; b < NPL; ++b) {
-        const uint32_t carry = pl[b] & k;
-        pl[b] ^= k;
-        k = carry;
-    }
+// One three-input logic instruction; LUT is the function of 0xF0, 0xCC, 0xAA.
+// Written out, because the compiler does not always find the single
+// instruction for a majority or a bit select.
+template <int LUT>
+__device__ __forceinline__ uint32_t lop3(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t d;
+    asm("lop3.b32 %0, %1, %2, %3, %4;" : "=r"(d) : "r"(a), "r"(b), "r"(c), "n"(LUT));
+    return d;
+}
+constexpr int L_MAJ = 0xE8, L_XOR = 0x96, L_SEL = 0xCA;   // a b + b c + c a; a ^ b ^ c; a ? b : c
+
+// Full adder of the planes a, b, c: returns the carry, a becomes the sum.
+__device__ __forceinline__ uint32_t msc_fa(uint32_t &a, uint32_t b, uint32_t c) {
+    const uint32_t k = lop3<L_MAJ>(a, b, c);
+    a = lop3<L_XOR>(a, b, c);
+    return k;
 }
 
-// Adds four bonds to counters kept in complemented form A_b = plane_b ^ x,
-// where the input words are the raw neighbour words w_j (= d_j ^ x). A full
+// Adds one carry plane into counters kept in complemented form (below), from
+// plane FROM upwards: full adders whose third input is a zero, that is x.
+template <int N, int FROM>
+__device__ __forceinline__ void msc_ripple(uint32_t (&A)[N], uint32_t x, uint32_t c) {
+#pragma unroll
+    for (int b = FROM; b < N; ++b) c = msc_fa(A[b], c, x);
+}
+
+// Adds four or eight bonds to counters kept in complemented form A_b =
+// plane_b ^ x, where the input words are the raw neighbour words w_j. A full
 // adder keeps the form: (a^x) ^ (p^x) ^ (q^x) = (a^p^q) ^ x and, majority
-// being self-dual, maj(a^x, p^x, q^x) = maj(a, p, q) ^ x. So two full adders
-// take w0..w3 into the ones plane, one more takes their carries into the twos
-// plane, and half adders (a^p^x, ((a^x) & (p^x)) ^ x) ripple the single carry
-// upwards: 7 + 2 (NPL - 3) three-input logic ops per four bonds.
-template <int NPL>
-__device__ __forceinline__ void msc_step4x(uint32_t (&A)[NPL], uint32_t x, uint32_t w0, uint32_t w1, uint32_t w2,
-                                           uint32_t w3) {
-    const uint32_t c1 = (A[0] & w0) | (w1 & (A[0] | w0));
-    A[0] ^= w0 ^ w1;
-    const uint32_t c2 = (A[0] & w2) | (w3 & (A[0] | w2));
-    A[0] ^= w2 ^ w3;
-    uint32_t c = (A[1] & c1) | (c2 & (A[1] | c1));
-    A[1] ^= c1 ^ c2;
+// being self-dual, maj(a^x, p^x, q^x) = maj(a, p, q) ^ x. Eight bonds: seven
+// full adders (four on the ones, two on the twos, one on the fours) and one
+// carry to ripple, 14 + 2 (N - 3) - 1 operations against 2 (6 + 2 (N - 2) - 1)
+// for two steps of four.
+template <int N>
+__device__ __forceinline__ void msc_step4x(uint32_t (&A)[N], uint32_t x, const uint32_t (&w)[4]) {
+    const uint32_t c1 = msc_fa(A[0], w[0], w[1]);
+    const uint32_t c2 = msc_fa(A[0], w[2], w[3]);
+    msc_ripple<N, 2>(A, x, msc_fa(A[1], c1, c2));
+}
+
+template <int N>
+__device__ __forceinline__ void msc_step8x(uint32_t (&A)[N], uint32_t x, const uint32_t (&w)[4],
+                                           const uint32_t (&v)[4]) {
+    const uint32_t c1 = msc_fa(A[0], w[0], w[1]);
+    const uint32_t c2 = msc_fa(A[0], w[2], w[3]);
+    const uint32_t c3 = msc_fa(A[0], v[0], v[1]);
+    const uint32_t c4 = msc_fa(A[0], v[2], v[3]);
+    const uint32_t d1 = msc_fa(A[1], c1, c2);
+    const uint32_t d2 = msc_fa(A[1], c3, c4);
+    msc_ripple<N, 3>(A, x, msc_fa(A[2], d1, d2));
+}
+
+// 8 x 8 bit transpose in every byte lane: bit i of byte q of r[j] goes to bit
+// j of byte q of r[i]. Words NZ..7 are zero on input (their swaps fold).
+template <int NZ>
+__device__ __forceinline__ void msc_transpose8(uint32_t (&r)[8]) {
+    auto swap = [](uint32_t &x, uint32_t &y, int s, uint32_t M, bool zx, bool zy) {
+        if (zx && zy) return;
+        const uint32_t lo = zy ? (x & M) : lop3<L_SEL>(M, x, y << s);
+        y = zy ? ((x >> s) & M) : lop3<L_SEL>(M, x >> s, y);
+        x = lo;
+    };
 #pragma unroll
-    for (int b = 2; b < NPL; ++b) {
-        const uint32_t nc = b + 1 < NPL ? (((A[b] ^ x) & (c ^ x)) ^ x) : 0u;
-        A[b] ^= c ^ x;
-        c = nc;
+    for (int b = 0; b < 4; ++b) swap(r[b], r[b + 4], 4, 0x0F0F0F0Fu, b >= NZ, b + 4 >= NZ);
+#pragma unroll
+    for (int b = 0; b < 8; b += (b & 1) ? 3 : 1)   // 0, 1, 4, 5
+        swap(r[b], r[b + 2], 2, 0x33333333u, (b & 3) >= NZ, ((b + 2) & 3) >= NZ);
+#pragma unroll
+    for (int b = 0; b < 8; b += 2)
+        swap(r[b], r[b + 1], 1, 0x55555555u, (b & 3) >= NZ && ((b ^ 2) & 3) >= NZ,
+             ((b + 1) & 3) >= NZ && (((b + 1) ^ 2) & 3) >= NZ);
+}
+
+// Shape of the multi-spin-coded tables for N counter planes (max degree below
+// 2^N). lvl: masks of the eight bits of T[m] >> 24 for every m = 2e + 1
+// (odd degree) and 2e + 2 (even degree) in that order, as words (N <= 5) or,
+// to keep the table small at wide degrees, as bytes. init: the
+// planes 0 .. N-2 of -(deg/2 + 1) as masks by degree (the top plane is always
+// set; wider counters derive them from the number).
+template <int N>
+struct MscShape {
+    static constexpr bool wide = N > 5;
+    static constexpr int nm = 1 << N;                        // values of m in the table
+    static constexpr int lvl_words = wide ? 2 * nm : 8 * nm;
+    static constexpr int init_words = wide ? 0 : 4 * nm;
+    static constexpr int acc_planes = N + 7;                 // energy accumulators
+    static constexpr int flush_items = 64;                   // 64 (2^N - 1) < 2^(N + 6)
+    static constexpr int entry = (N + 3) & ~1;               // words of a tie-queue entry: 3 and N - 1 planes, made even
+};
+
+// Words of shared memory a block may use beside the words of the positions
+// and the class bounds: fixed by the degree class, so that the largest graph
+// that fits does not move when the tables change. The tie queues take what the
+// tables leave, and more when the graph leaves room.
+__host__ __device__ inline int msc_reserved_words(int mmax) {
+    return 256 + (mmax <= 7 ? 256 : mmax <= 15 ? 1024 : mmax <= 31 ? 4096 : 0) + 72 + 512;
+}
+
+__host__ __device__ inline int msc_planes(int mmax) {
+    return mmax <= 7 ? 3 : mmax <= 15 ? 4 : mmax <= 31 ? 5 : mmax <= 63 ? 6 : 7;
+}
+
+__host__ __device__ inline int msc_entry_words(int mmax) { return (msc_planes(mmax) + 3) & ~1; }
+
+__host__ __device__ inline int msc_table_words(int mmax) {   // lvl, init, thresholds
+    const int nm = 1 << msc_planes(mmax);
+    return (nm > 32 ? 2 * nm : 12 * nm) + nm;
+}
+
+// Uniform parameters of a step's decisions, found once per block.
+struct MscLevels {
+    int top;    // values e >= top have thresholds with a zero top byte
+    int zero;   // values e >= zero have a zero threshold: their ties reject
+};
+
+// One unit (four bonds) of a lane's row: the neighbours' words, complemented
+// for weight -1. BIG: 32-bit entries (byte offset | sign); otherwise pairs of
+// 16-bit byte offsets with the pair's signs in the low bits of the first.
+template <bool BIG>
+using MscUnit = std::conditional_t<BIG, uint4, uint2>;
+
+template <bool WEIGHTED>
+__device__ __forceinline__ void msc_unit_words(const unsigned char *Wb, const uint2 &v, uint32_t (&w)[4]) {
+    const uint32_t vv[2] = {v.x, v.y};
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        w[2 * j] = *reinterpret_cast<const uint32_t *>(Wb + (vv[j] & 0xFFFCu));
+        w[2 * j + 1] = *reinterpret_cast<const uint32_t *>(Wb + (vv[j] >> 16));
+        if (WEIGHTED) {
+            w[2 * j] ^= (uint32_t)((int32_t)(vv[j] << 31) >> 31);
+            w[2 * j + 1] ^= (uint32_t)((int32_t)(vv[j] << 30) >> 31);
+        }
     }
 }
 
-// Delta swap of the bits selected by M between x >> s and y; zx, zy say that
-// x or y is known to be zero (then the swap is a mask and a shift).
-__device__ __forceinline__ void msc_swap(uint32_t &x, uint32_t &y, int s, uint32_t M, bool zx, bool zy) {
-    if (zx && zy) return;
-    if (zy) {
-        y = (x >> s) & M;
-        x &= ~(M << s);
-    } else if (zx) {
-        x = (y & M) << s;
-        y &= ~M;
-    } else {
-        const uint32_t t = ((x >> s) ^ y) & M;
-        x ^= t << s;
-        y ^= t;
+template <bool WEIGHTED>
+__device__ __forceinline__ void msc_unit_words(const unsigned char *Wb, const uint4 &v, uint32_t (&w)[4]) {
+    const uint32_t vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        w[j] = *reinterpret_cast<const uint32_t *>(Wb + (WEIGHTED ? vv[j] & ~3u : vv[j]));
+        if (WEIGHTED) w[j] ^= (uint32_t)((int32_t)(vv[j] << 31) >> 31);
     }
 }
 
-template <int NPL, bool WEIGHTED>
-__device__ __forceinline__ uint32_t msc_item(const SweepArgs &a, const uint32_t *Wsm, const uint32_t *T256, int p,
-                                             uint32_t x, uint32_t c3, int blk, int32_t *Eacc,
-                                             uint32_t (&ebias)[8], uint32_t &tent) {
-    const uint32_t vid = __ldg(&a.g.vid[p]);
-    uint32_t pl[NPL];
-#pragma unroll
-    for (int b = 0; b < NPL; ++b) pl[b] = 0u;
-    uint32_t deg;
-    if (a.g.mcol) {
-        // Rows padded to whole 4-bond steps, entries = byte offsets of the
-        // neighbours' words: one 8-byte load per step, no single-bond tail.
-        const uint32_t h0 = __ldg(&a.g.mrp[p]), h1 = __ldg(&a.g.mrp[p + 1]);
-        deg = h0 & 0xFFu;
-        const unsigned char *Wb = reinterpret_cast<const unsigned char *>(Wsm);
-        // The planes in complemented form (msc_step4x). With NPL = 3 (degree <= 7,
-        // at most two steps) the plain adders starting from zero fold further
-        // and stay cheaper.
-        uint32_t A[NPL];
-#pragma unroll
-        for (int b = 0; b < NPL; ++b) A[b] = NPL >= 4 ? x : 0u;
-        for (uint32_t q = h0 >> 8; q < (h1 >> 8); ++q) {
-            const uint2 v = __ldg(&a.g.mcol[q]);
-            const uint32_t o[4] = {v.x & 0xFFFFu, v.x >> 16, v.y & 0xFFFFu, v.y >> 16};
-            uint32_t w[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                w[j] = *reinterpret_cast<const uint32_t *>(Wb + (WEIGHTED ? (o[j] & ~3u) : o[j]));
-                if (WEIGHTED && (o[j] & 1u)) w[j] = ~w[j];
-            }
-            if (NPL >= 4) msc_step4x<NPL>(A, x, w[0], w[1], w[2], w[3]);
-            else msc_csa4<NPL>(A, x, w[0], w[1], w[2], w[3]);
-        }
-#pragma unroll
-        for (int b = 0; b < NPL; ++b) pl[b] = NPL >= 4 ? A[b] ^ x : A[b];
-    } else {
-        const uint32_t e0 = __ldg(&a.g.rp[p]), e1 = __ldg(&a.g.rp[p + 1]);
-        deg = e1 - e0;
-        uint32_t e = e0;
-        for (; e + 4 <= e1; e += 4) {   // four bonds per step through carry-save adders
-            uint32_t w0 = Wsm[__ldg(&a.g.col[e])], w1 = Wsm[__ldg(&a.g.col[e + 1])];
-            uint32_t w2 = Wsm[__ldg(&a.g.col[e + 2])], w3 = Wsm[__ldg(&a.g.col[e + 3])];
-            if (WEIGHTED) {
-                if (__ldg(&a.g.wt[e]) < 0) w0 = ~w0;
-                if (__ldg(&a.g.wt[e + 1]) < 0) w1 = ~w1;
-                if (__ldg(&a.g.wt[e + 2]) < 0) w2 = ~w2;
-                if (__ldg(&a.g.wt[e + 3]) < 0) w3 = ~w3;
-            }
-            msc_csa4<NPL>(pl, x, w0, w1, w2, w3);
-        }
-        for (; e < e1; ++e) {
-            uint32_t d = x ^ Wsm[__ldg(&a.g.col[e])];
-            if (WEIGHTED && __ldg(&a.g.wt[e]) < 0) d = ~d;
-#pragma unroll
-            for (int b = 0; b < NPL; ++b) {   // ripple-carry add of one bit per replica
-                const uint32_t carry = pl[b] & d;
-                pl[b] ^= d;
-                d = carry;
-            }
-        }
-    }
-    constexpr bool PK = MscPackedE<NPL>::value;
-    constexpr uint32_t H = (uint32_t)MscPairTab<NPL>::H;
-    const uint32_t base = PK ? 2u * H - 4u * deg : 128u - deg;   // mb byte = 4(m + H/2) (PK) or m + 128
+// One slice as a warp sees it.
+struct MscSlice {
+    uint32_t vd;            // vertex | degree << 16 | 1 << 31 on lanes past the class
+    uint32_t off, units;    // byte offset of the lane's first unit; units of the slice (uniform)
+};
+
+template <bool BIG>
+__device__ __forceinline__ MscUnit<BIG> msc_unit(const SweepArgs &a, uint32_t off, uint32_t u) {
+    constexpr uint32_t bytes = 32u * sizeof(MscUnit<BIG>);
+    return __ldg(reinterpret_cast<const MscUnit<BIG> *>(reinterpret_cast<const char *>(a.g.mcol) + (off + u * bytes)));
+}
+
+// One (position, word) item: 32 attempts. Returns the mask of accepted
+// replicas; `tie` are the undecided ones, E the counter planes of e. Lanes past
+// their class run along and accept nothing.
+// The first two units are read before the random numbers are drawn, which
+// covers their latency.
+template <int N, bool WEIGHTED, bool BIG>
+__device__ __forceinline__ uint32_t msc_item(const SweepArgs &a, const uint32_t *Wsm, const uint32_t *lvl,
+                                             const uint32_t *init, const MscLevels &L, const MscSlice &sl,
+                                             uint32_t x, uint32_t c3, int blk, uint32_t (&E)[N],
+                                             uint32_t (&S)[MscShape<N>::acc_planes], uint32_t &tie,
+                                             uint32_t &odd_out) {
+    const uint32_t vid = sl.vd & 0xFFFFu, deg = (sl.vd >> 16) & 0x7Fu;
+    const MscUnit<BIG> v0 = msc_unit<BIG>(a, sl.off, 0u), v1 = msc_unit<BIG>(a, sl.off, sl.units > 1u ? 1u : 0u);
     // Both Philox calls of the item (slots 32 blk .. +15 and +16 .. +31).
     uint4 u0, u1;
     philox_from_shared2(philox_shared(vid, (uint32_t)a.k, c3, a.key0, a.key1), 2u * blk, 2u * blk + 1u, a.rk0, a.rk1,
                         u0, u1);
-    // Byte q of r[g] = c of replica 4g + q: an 8 x 8 bit transpose in every byte lane.
-    // Planes NPL..7 are zero, so a swap with a known-zero partner is a mask and
-    // a shift (msc_swap); the zero set after each stage follows from NPL alone.
-    uint32_t r[8];
+    uint32_t U[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
+    msc_transpose8<8>(U);
+    // Counter planes of -(deg/2 + 1), complemented by x.
+    uint32_t A[N];
+    if (MscShape<N>::wide) {
+        const uint32_t k = ~(deg >> 1);   // -(deg/2 + 1)
 #pragma unroll
-    for (int b = 0; b < 8; ++b) r[b] = b < NPL ? pl[b] : 0u;
+        for (int b = 0; b < N - 1; ++b) A[b] = x ^ (uint32_t)((int32_t)(k << (31 - b)) >> 31);
+    } else {
+        const uint4 i4 = *reinterpret_cast<const uint4 *>(init + 4 * deg);
+        const uint32_t iv[4] = {i4.x, i4.y, i4.z, i4.w};
 #pragma unroll
-    for (int b = 0; b < 4; ++b) msc_swap(r[b], r[b + 4], 4, 0x0F0F0F0Fu, b >= NPL, b + 4 >= NPL);
-#pragma unroll
-    for (int b = 0; b < 8; b += (b & 1) ? 3 : 1)   // 0, 1, 4, 5
-        msc_swap(r[b], r[b + 2], 2, 0x33333333u, (b & 3) >= NPL, ((b + 2) & 3) >= NPL);
-#pragma unroll
-    for (int b = 0; b < 8; b += 2)
-        msc_swap(r[b], r[b + 1], 1, 0x55555555u, (b & 3) >= NPL && ((b ^ 2) & 3) >= NPL,
-                 ((b + 1) & 3) >= NPL && (((b + 1) ^ 2) & 3) >= NPL);
-    uint32_t acc32 = 0, acct32 = 0;   // accepted; accepted or tied
-    const uint32_t mq0 = (32u - deg) * 0x01010101u;   // 2c + 32 - deg = m + 32 per byte (PK)
-    const unsigned char *tb = reinterpret_cast<const unsigned char *>(T256);
-#pragma unroll
-    for (int g = 0; g < 8; ++g) {
-        const uint32_t mb = r[g] * (PK ? 8u : 2u) + base * 0x01010101u;
-        const uint4 &uq = g < 4 ? u0 : u1;
-        const uint32_t uw = (g & 3) == 0 ? uq.x : (g & 3) == 1 ? uq.y : (g & 3) == 2 ? uq.z : uq.w;
-        uint32_t e01, e23;
-        if (PK) {   // byte offsets of the pair entries: b0 + H b1 and b2 + H b3 of the bytes b = 4(m + H/2)
-            e01 = *reinterpret_cast<const uint32_t *>(tb + __dp4a(mb, 0x00000001u | (H << 8), 0u));
-            e23 = *reinterpret_cast<const uint32_t *>(tb + __dp4a(mb, 0x00010000u | (H << 24), 0u));
+        for (int b = 0; b < N - 1; ++b) A[b] = x ^ iv[b];
+    }
+    A[N - 1] = ~x;
+    {
+        const unsigned char *Wb = reinterpret_cast<const unsigned char *>(Wsm);
+        uint32_t w[4], v[4];
+        msc_unit_words<WEIGHTED>(Wb, v0, w);
+        if (sl.units > 1) {
+            msc_unit_words<WEIGHTED>(Wb, v1, v);
+            msc_step8x<N>(A, x, w, v);
+            uint32_t u = 2;
+            for (; u + 2 <= sl.units; u += 2) {
+                msc_unit_words<WEIGHTED>(Wb, msc_unit<BIG>(a, sl.off, u), w);
+                msc_unit_words<WEIGHTED>(Wb, msc_unit<BIG>(a, sl.off, u + 1u), v);
+                msc_step8x<N>(A, x, w, v);
+            }
+            if (u < sl.units) {
+                msc_unit_words<WEIGHTED>(Wb, msc_unit<BIG>(a, sl.off, u), w);
+                msc_step4x<N>(A, x, w);
+            }
         } else {
-            uint32_t e[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                e[q] = *reinterpret_cast<const uint32_t *>(tb + 4u * ((mb >> (8 * q)) & 0xFFu));
-            e01 = __byte_perm(e[0], e[1], 0x5410u);
-            e23 = __byte_perm(e[2], e[3], 0x5410u);
-        }
-        const uint32_t slo = __byte_perm(uw, 0u, 0x4140u) * 128u + e01;
-        const uint32_t shi = __byte_perm(uw, 0u, 0x4342u) * 128u + e23;
-        const uint32_t RT = prmt_sign(slo, shi, 0xFDB9u);                               // reject or tie
-        const uint32_t RS = prmt_sign(slo - 0x00010001u, shi - 0x00010001u, 0xFDB9u);   // reject
-        const uint32_t M = 0x01010101u << g;
-        acc32 |= ~RT & M;
-        acct32 |= ~RS & M;
-        if (PK) {
-            ebias[g] += ((r[g] * 2u + mq0) & ~RT) | (0x20202020u & RT);   // byte q: accepted ? 32 + m : 32
-        } else if (~RT & 0x80808080u) {   // energy change 2m = 2(mb byte - 128) of each accepted replica
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (!((RT >> (8 * q)) & 1u)) atomicAdd(&Eacc[4 * g + q], 2 * ((int)((mb >> (8 * q)) & 0xFFu) - 128));
+            msc_step4x<N>(A, x, w);
         }
     }
-    uint32_t tie = acct32 & ~acc32;
-    tent = 0u;
-    if (tie) {   // the low 24 bits of the uniform decide: the item's first tie is queued for
-                 // the warp (msc_queue_tie), further ties of the same item are settled here
-        const uint32_t *tab = a.tables + (size_t)a.tidx[a.k] * (a.g.mmax + 1);
-        bool first = true;
+#pragma unroll
+    for (int b = 0; b < N; ++b) E[b] = A[b] ^ x;
+    const uint32_t neg = E[N - 1];
+    uint32_t high = 0u;   // e >= 4 (or negative)
+#pragma unroll
+    for (int b = 2; b < N; ++b) high |= E[b];
+    uint32_t lt = 0u, eq;
+    if (L.top == 0) {   // every threshold has a zero top byte: only a zero byte can accept
+        eq = ~((U[0] | U[1] | U[2]) | (U[3] | U[4] | U[5]) | (U[6] | U[7]));
+    } else {
+        // Planes of the threshold's top byte: for every value of e below L.top,
+        // the replicas with that e take the bits of their own parity's m.
+        uint32_t TP[8];
+        const uint32_t *lv = lvl + ((deg & 1u) ? 0 : MscShape<N>::wide ? 2 : 8);
+        auto take = [&](int e, uint32_t who, bool first) {
+            uint32_t v[8];
+            if (MscShape<N>::wide) {
+                const uint2 q = *reinterpret_cast<const uint2 *>(lv + 4 * e);
+#pragma unroll
+                for (int b = 0; b < 8; ++b) v[b] = __byte_perm(b < 4 ? q.x : q.y, 0u, 0x1111u * (b & 3));
+            } else {
+                const uint4 q0 = *reinterpret_cast<const uint4 *>(lv + 16 * e);
+                const uint4 q1 = *reinterpret_cast<const uint4 *>(lv + 16 * e + 4);
+                v[0] = q0.x; v[1] = q0.y; v[2] = q0.z; v[3] = q0.w;
+                v[4] = q1.x; v[5] = q1.y; v[6] = q1.z; v[7] = q1.w;
+            }
+#pragma unroll
+            for (int b = 0; b < 8; ++b) TP[b] = first ? (who & v[b]) : lop3<0xF8>(TP[b], who, v[b]);   // | who & v
+        };
+        take(0, ~(high | E[0] | E[1]), true);
+        if (L.top > 1) {
+            take(1, lop3<0x10>(E[0], E[1], high) , false);   // E0 & ~E1 & ~high
+            if (L.top > 2) {
+                take(2, lop3<0x04>(E[0], E[1], high), false);   // ~E0 & E1 & ~high
+                if (L.top > 3) take(3, lop3<0x40>(E[0], E[1], high), false);   // E0 & E1 & ~high
+            }
+#pragma unroll 1
+            for (int j = 1; N > 3 && 4 * j < L.top; ++j) {
+                uint32_t no = neg;   // not in this group of four values
+#pragma unroll
+                for (int b = 2; b < N - 1; ++b) no |= ((j >> (b - 2)) & 1) ? ~E[b] : E[b];
+                take(4 * j, ~(no | E[0] | E[1]), false);
+                take(4 * j + 1, lop3<0x10>(E[0], E[1], no), false);
+                take(4 * j + 2, lop3<0x04>(E[0], E[1], no), false);
+                take(4 * j + 3, lop3<0x40>(E[0], E[1], no), false);
+            }
+        }
+        eq = ~0u;
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            lt = lop3<0xB2>(TP[b], U[b], lt);   // T & ~U | ~(T ^ U) & lt
+            eq = lop3<0x82>(TP[b], U[b], eq);   // ~(T ^ U) & eq
+        }
+    }
+    const uint32_t live = ~(uint32_t)((int32_t)sl.vd >> 31);
+    const uint32_t acc = (neg | lt) & live;
+    // Ties of a zero threshold reject: e >= 4 (e >= 2) where no such threshold is left.
+    tie = eq & ~neg & live;
+    if (L.zero <= 4) tie &= ~high;
+    if (L.zero <= 2) tie &= ~E[1];
+    // Energies: S += m = 2e + 1 + (even degree) of the accepted replicas, in
+    // two's complement (the carry-in is the 1).
+    const uint32_t odd = 0u - (deg & 1u);
+    odd_out = odd;
+    uint32_t c = lop3<0xD0>(acc, S[0], odd);   // acc & (S0 | ~odd)
+    S[0] = lop3<0x78>(S[0], acc, odd);         // S0 ^ (acc & odd)
+#pragma unroll
+    for (int b = 0; b < N; ++b) c = msc_fa(S[b + 1], E[b] & acc, c);
+    const uint32_t sign = neg & acc;
+#pragma unroll
+    for (int b = N + 1; b < MscShape<N>::acc_planes; ++b) c = msc_fa(S[b], sign, c);
+    return acc;
+}
+
+// Adds the accumulated m of the warp's lanes to the energies (dE = 2m) and
+// clears them: the planes become bytes by transposes (the low eight planes,
+// then the rest with the sign plane inverted, that is plus 2^(W-1)), which sum
+// over the lanes in 16-bit halves without carries. Runs after at most 64 items
+// per lane, so about once per sweep.
+template <int N>
+__device__ __forceinline__ void msc_flush_energy(uint32_t (&S)[MscShape<N>::acc_planes], int32_t *Eacc, int lane) {
+    constexpr int W = MscShape<N>::acc_planes, NH = W - 8;
+    uint32_t lo[8], hi[8];
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        lo[b] = S[b];
+        hi[b] = b < NH ? (b == NH - 1 ? ~S[b + 8] : S[b + 8]) : 0u;
+    }
+    msc_transpose8<8>(lo);
+    msc_transpose8<NH>(hi);
+    uint32_t mlo = 0u, mhi = 0u;
+#pragma unroll
+    for (int g = 0; g < 8; ++g) {
+        const uint32_t a0 = __reduce_add_sync(0xFFFFFFFFu, lo[g] & 0x00FF00FFu);          // bytes 0, 2
+        const uint32_t a1 = __reduce_add_sync(0xFFFFFFFFu, (lo[g] >> 8) & 0x00FF00FFu);   // bytes 1, 3
+        const uint32_t b0 = __reduce_add_sync(0xFFFFFFFFu, hi[g] & 0x00FF00FFu);
+        const uint32_t b1 = __reduce_add_sync(0xFFFFFFFFu, (hi[g] >> 8) & 0x00FF00FFu);
+        if ((lane >> 2) == g) {
+            mlo = (lane & 1) ? a1 : a0;
+            mhi = (lane & 1) ? b1 : b0;
+        }
+    }
+    const int sh = (lane & 2) ? 16 : 0;
+    const int m = (int)((mlo >> sh) & 0xFFFFu) + 256 * (int)((mhi >> sh) & 0xFFFFu) - (32 << (W - 1));
+    if (m) atomicAdd(&Eacc[lane], 2 * m);
+#pragma unroll
+    for (int b = 0; b < W; ++b) S[b] = 0u;
+}
+
+// Copies of the word array that a block writes besides its own: the other
+// CTAs of its cluster (none outside a cluster).
+template <bool CL>
+struct MscPeers {
+    uint32_t *Wsm;
+    int rank, size;
+    __device__ __forceinline__ void store(int p, uint32_t v) const {
+        Wsm[p] = v;
+        if (CL)
+            for (int d = 1; d < size; ++d) cooperative_groups::this_cluster().map_shared_rank(Wsm, rank ^ d)[p] = v;
+    }
+    __device__ __forceinline__ void flip(int p, uint32_t bits) const {
+        atomicXor(&Wsm[p], bits);
+        if (CL)
+            for (int d = 1; d < size; ++d)
+                atomicXor(&cooperative_groups::this_cluster().map_shared_rank(Wsm, rank ^ d)[p], bits);
+    }
+};
+
+// Ties queued by the items of a warp (entry: tie mask, position | vertex << 16,
+// odd-degree mask, planes of e) are settled together: each lane takes one entry, draws
+// the low 24 bits of its uniforms and applies an accepted flip to the word
+// (and its copies), the energy and the accept count. Items of one colour class
+// never read each other's words, so a flip applied after the other items of
+// the class is the same as one applied at once; every queue is emptied before
+// the class barrier.
+template <int N, bool CL>
+__device__ __forceinline__ void msc_drain_ties(const SweepArgs &a, const uint32_t *Tt, const uint32_t *TQ, int qc,
+                                               const MscPeers<CL> &W, int32_t *Eacc, int blk, uint32_t c3,
+                                               uint32_t vmask, uint32_t &nacc, int lane) {
+    __syncwarp();
+    for (int i = lane; i < qc; i += 32) {
+        const uint32_t *q = TQ + MscShape<N>::entry * i;
+        uint32_t tie = q[0];
+        const int p = (int)(q[1] & 0xFFFFu), odd = (int)(q[2] & 1u);
+        const uint32_t vid = q[1] >> 16;
         do {
             const int bit = __ffs(tie) - 1;
             tie &= tie - 1u;
-            const int g = bit & 7;
-            uint32_t rg = r[0];   // count byte of the replica at this bit: byte bit >> 3 of r[bit & 7]
+            uint32_t e = 0u;
 #pragma unroll
-            for (int j = 1; j < 8; ++j)
-                if (g == j) rg = r[j];
-            const int m = 2 * (int)((rg >> (bit & 24)) & 0xFFu) - (int)deg;
-            if (first) {   // the item's first tie goes to the warp's queue
-                tent = 0x80000000u | (uint32_t)p << 13 | (uint32_t)bit << 8 | (uint32_t)m;
-                first = false;
-                continue;
-            }
-            const uint32_t T = __ldg(&tab[m]);
+            for (int b = 0; b < N - 1; ++b) e |= ((q[3 + b] >> bit) & 1u) << b;
+            const int m = 2 * (int)e + 2 - odd;
             const int rep = 4 * (bit & 7) + (bit >> 3);
-            if (sweep_tail_bits(vid, 32u * blk + rep, (uint32_t)a.k, c3, a.key0, a.key1) < (T & 0xFFFFFFu)) {
-                acc32 |= 1u << bit;
+            if (sweep_tail_bits(vid, 32u * blk + rep, (uint32_t)a.k, c3, a.key0, a.key1) < (Tt[m] & 0xFFFFFFu)) {
+                W.flip(p, 1u << bit);
                 atomicAdd(&Eacc[rep], 2 * m);
+                nacc += (vmask >> bit) & 1u;
             }
         } while (tie);
     }
-    return acc32;
-}
-
-// Ties queued by the items of a warp (entry = flag | p << 13 | bit << 8 | m)
-// are settled together: each lane takes one entry, draws the low 24 bits of
-// its uniform and applies an accepted flip to the word (and its copy in the
-// peer CTA), the energy and the accept count. Items of one colour class never
-// read each other's words, so a flip applied after the other items of the
-// class is the same as one applied at once; every queue is emptied before the
-// class barrier.
-__device__ __forceinline__ void msc_drain_ties(const SweepArgs &a, const uint32_t *TQ, int qc, uint32_t *Wsm,
-                                               uint32_t *Wpeer, int32_t *Eacc, int blk, uint32_t c3, uint32_t vmask,
-                                               uint32_t &nacc, int lane) {
-    __syncwarp();
-    const uint32_t *tab = a.tables + (size_t)a.tidx[a.k] * (a.g.mmax + 1);
-    for (int i = lane; i < qc; i += 32) {
-        const uint32_t e = TQ[i];
-        const int p = (int)((e >> 13) & 0xFFFFu), bit = (int)((e >> 8) & 31u), m = (int)(e & 0xFFu);
-        const int rep = 4 * (bit & 7) + (bit >> 3);
-        const uint32_t T = __ldg(&tab[m]);
-        if (sweep_tail_bits(__ldg(&a.g.vid[p]), 32u * blk + rep, (uint32_t)a.k, c3, a.key0, a.key1) <
-            (T & 0xFFFFFFu)) {
-            atomicXor(&Wsm[p], 1u << bit);
-            if (Wpeer) atomicXor(&Wpeer[p], 1u << bit);
-            atomicAdd(&Eacc[rep], 2 * m);
-            nacc += (vmask >> bit) & 1u;
-        }
-    }
     __syncwarp();
 }
 
-// Appends the lanes' queue entries (tent != 0) to the warp's tie queue; drains
-// it once it holds more than 32 entries (capacity 64).
-__device__ __forceinline__ void msc_queue_tie(const SweepArgs &a, uint32_t *TQ, int &qc, uint32_t tent, uint32_t *Wsm,
-                                              uint32_t *Wpeer, int32_t *Eacc, int blk, uint32_t c3, uint32_t vmask,
-                                              uint32_t &nacc, int lane) {
-    const uint32_t bal = __ballot_sync(0xFFFFFFFFu, tent != 0u);
-    if (bal) {
-        if (tent) TQ[qc + __popc(bal & ((1u << lane) - 1u))] = tent;
-        qc += __popc(bal);
-        if (qc > 32) {
-            msc_drain_ties(a, TQ, qc, Wsm, Wpeer, Eacc, blk, c3, vmask, nacc, lane);
-            qc = 0;
-        }
-    }
-}
-
-template <int NPL, bool WEIGHTED, int NTB, int MINB>
-__global__ void __launch_bounds__(NTB, MINB) k_sweep_msc(const SweepArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const bool act = !a.active || a.active[a.k];
-    const int nsweeps = act ? a.S : 0;
-    const int np = a.g.np, n = a.g.n;
-    uint32_t *T256 = reinterpret_cast<uint32_t *>(smem);          // [256] decision table (see above)
-    uint32_t *PT = T256 + 256;                                      // [H * H] pair table (packed energies)
-    uint32_t *Wsm = PT + MscPairTab<NPL>::words;                    // [np]
-    int32_t *cls = reinterpret_cast<int32_t *>(Wsm + np);
-    const int csz = (a.g.ncol + 1 + 3) & ~3;
-    int32_t *Eacc = cls + csz;      // [32]
-    int32_t *PS = Eacc + 32;        // [32]
-    int32_t *misc = PS + 32;        // best E, step, sweep, slot, copy-from (r+1), changed
-    uint32_t *TQ = reinterpret_cast<uint32_t *>(misc + 8) + (threadIdx.x >> 5) * 64;   // [warps][64] tie queues
-
-    const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31;
-    const uint32_t *tab = a.tables + (size_t)a.tidx[a.k] * (a.g.mmax + 1);
-    for (int i = tid; i < 256; i += NT) T256[i] = msc_entry(i, MscPackedE<NPL>::value, tab, a.g.mmax);
-    if (MscPackedE<NPL>::value) {
-        __syncthreads();
-        msc_fill_pair_table<NPL>(PT, T256, tid, NT);
-    }
-    for (int i = tid; i <= a.g.ncol; i += NT) cls[i] = a.g.cls[i];
-
-    for (int lb = blockIdx.x; lb < a.nblk; lb += gridDim.x) {
-        const int blk = a.blk_base + lb;
-        const int slot0 = blk * 32;
-        if (tid < 32) PS[tid] = act ? a.parent[slot0 + tid] : slot0 + tid;
-        if (tid == 0) {
-            const int4 br = a.best_rec[blk];
-            misc[0] = br.x; misc[1] = br.y; misc[2] = br.z; misc[3] = br.w;
-            misc[4] = 0; misc[5] = 0;
-        }
-        __syncthreads();
-        if (tid < 32) Eacc[tid] = a.E_in[PS[tid]];
-        // Load: 32 int8 spin rows -> one bit word per position.
-        for (int c = tid; c < (np >> 2); c += NT) {
-            uint32_t w4[4];
-            msc_pack_rows(a.spins_in, PS, np, c, w4);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) Wsm[4 * c + j] = w4[j];
-        }
-        __syncthreads();
-        uint32_t vmask = 0u;   // bits of the live replicas
-        for (int r = 0; r < 32; ++r) vmask |= (slot0 + r < a.R ? 1u : 0u) << msc_bit(r);
-        uint32_t nacc = 0;
-        uint32_t ebias[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-        int cnt = 0;
-        for (int s = 0; s < nsweeps; ++s) {
-            const uint32_t c3 = TAG_SWEEP | (uint32_t)s;
-            for (int c = 0; c < a.g.ncol; ++c) {
-                const int p0 = cls[c], p1 = cls[c + 1];
-                const int nr = (p1 - p0 + NT - 1) / NT;   // rounds of the class, uniform over the CTA
-                int qc = 0;   // entries in this warp's tie queue
-                for (int rd = 0; rd < nr; ++rd) {
-                    const int p = p0 + tid + rd * NT;
-                    uint32_t tent = 0u;
-                    if (p < p1) {
-                        const uint32_t x = Wsm[p];
-                        const uint32_t acc32 =
-                            msc_item<NPL, WEIGHTED>(a, Wsm, MscPackedE<NPL>::value ? PT : T256, p, x, c3, blk, Eacc,
-                                                    ebias, tent);
-                        if (acc32) {
-                            Wsm[p] = x ^ acc32;
-                            nacc += __popc(acc32 & vmask);
-                        }
-                        ++cnt;
-                    }
-                    msc_queue_tie(a, TQ, qc, tent, Wsm, nullptr, Eacc, blk, c3, vmask, nacc, lane);
-                    if (MscPackedE<NPL>::value && ((rd & 3) == 3 || rd == nr - 1))
-                        msc_flush_energy(ebias, cnt, Eacc, lane);
-                }
-                if (qc) msc_drain_ties(a, TQ, qc, Wsm, nullptr, Eacc, blk, c3, vmask, nacc, lane);
-                __syncthreads();
-            }
-            if (tid == 0) {
-                int bq = -1, bE = 0x7FFFFFFF;
-                for (int q = 0; q < 32; ++q)
-                    if (slot0 + q < a.R && Eacc[q] < bE) { bE = Eacc[q]; bq = q; }
-                misc[4] = 0;
-                if (bq >= 0) {
-                    atomicMin(&a.sweep_emin[(size_t)a.k * a.S + s], bE);
-                    if (bE < misc[0]) {
-                        misc[0] = bE; misc[1] = a.k; misc[2] = s; misc[3] = slot0 + bq;
-                        misc[4] = bq + 1; misc[5] = 1;
-                    }
-                }
-            }
-            __syncthreads();
-            if (misc[4]) {
-                const int rq = misc[4] - 1;
-                uint32_t *dst = reinterpret_cast<uint32_t *>(a.best_cfg + (size_t)blk * np);
-                for (int c = tid; c < (np >> 2); c += NT) {
-                    uint32_t v = 0;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const bool real = 4 * c + j < n;
-                        v |= (real ? (((Wsm[4 * c + j] >> msc_bit(rq)) & 1u) ? 0x01u : 0xFFu) : 0u) << (8 * j);
-                    }
-                    dst[c] = v;
-                }
-                __syncthreads();
-            }
-        }
-        // Store: bit words -> int8 spin rows (fields are not kept by this layout).
-        for (int c = tid; c < (np >> 2); c += NT) {
-            uint32_t w4[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) w4[j] = Wsm[4 * c + j];
-            msc_unpack_rows(w4, a.spins_out, slot0, np, n, c);
-        }
-        if (tid < 32) a.E_out[slot0 + tid] = Eacc[tid];
-        if (tid == 0 && misc[5]) a.best_rec[blk] = make_int4(misc[0], misc[1], misc[2], misc[3]);
-        const uint32_t wsum = __reduce_add_sync(0xFFFFFFFFu, nacc);
-        if (act && lane == 0 && wsum) atomicAdd(&a.accepts[a.k], (unsigned long long)wsum);
-        __syncthreads();
-    }
-}
-
-// Multi-spin coding with a thread-block cluster of two CTAs per word. Both
-// CTAs keep a full copy of the word array; inside a colour class CTA r takes
-// the items at even (r = 0) or odd (r = 1) offsets, and every changed word is
-// stored into both copies (the peer's through distributed shared memory). A
-// cluster barrier closes each class. The 32 energies live in CTA 0, which
-// also does the best tracking; CTA 1 adds its energy changes there remotely.
-// Halving the work unit lets the SMs balance 2 x words CTAs dynamically.
-template <int NPL, bool WEIGHTED>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 4) k_sweep_msc_pair(const SweepArgs a) {
+// Sweeps of multi-spin-coded words. CL: a thread-block cluster of two CTAs
+// shares a word. Every CTA keeps a full copy of the word array; inside a
+// colour class the CTAs take the positions in turns of 32, every changed word
+// is stored into all copies (the others' through distributed shared memory),
+// and a cluster barrier closes each class. The 32 energies live in CTA 0,
+// which also does the best tracking; the others add their changes there
+// remotely. Halving the work unit lets the SMs balance the words that do not
+// divide over them.
+template <int N, bool WEIGHTED, bool BIG, bool CL>
+__global__ void __launch_bounds__(256, 4) k_sweep_msc(const SweepArgs a) {
     namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int rank = (int)cluster.block_rank();
+    using Sh = MscShape<N>;
     extern __shared__ __align__(16) unsigned char smem[];
     const bool act = !a.active || a.active[a.k];
     const int nsweeps = act ? a.S : 0;
     const int np = a.g.np, n = a.g.n;
-    uint32_t *T256 = reinterpret_cast<uint32_t *>(smem);          // [256] decision table (see above)
-    uint32_t *PT = T256 + 256;                                      // [H * H] pair table (packed energies)
-    uint32_t *Wsm = PT + MscPairTab<NPL>::words;                    // [np]
+    uint32_t *lvl = reinterpret_cast<uint32_t *>(smem);            // top-byte masks by m
+    uint32_t *init = lvl + Sh::lvl_words;                           // counter start by degree
+    uint32_t *Tt = init + Sh::init_words;                           // [2^N] thresholds by m
+    uint32_t *Wsm = Tt + Sh::nm;                                    // [np]
     int32_t *cls = reinterpret_cast<int32_t *>(Wsm + np);
     const int csz = (a.g.ncol + 1 + 3) & ~3;
-    int32_t *Eacc = cls + csz;      // [32] (used in CTA 0)
+    int32_t *Eacc = cls + csz;      // [32] (in a cluster: CTA 0's)
     int32_t *PS = Eacc + 32;        // [32]
-    int32_t *misc = PS + 32;        // best E, step, sweep, slot, copy-from (r+1), changed
-    uint32_t *Wpeer = cluster.map_shared_rank(Wsm, rank ^ 1);
-    int32_t *E0 = cluster.map_shared_rank(Eacc, 0);
-    uint32_t *TQ = reinterpret_cast<uint32_t *>(misc + 8) + (threadIdx.x >> 5) * 64;   // [warps][64] tie queues
-
-    const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31;
-    const uint32_t *tab = a.tables + (size_t)a.tidx[a.k] * (a.g.mmax + 1);
-    for (int i = tid; i < 256; i += NT) T256[i] = msc_entry(i, MscPackedE<NPL>::value, tab, a.g.mmax);
-    if (MscPackedE<NPL>::value) {
-        __syncthreads();
-        msc_fill_pair_table<NPL>(PT, T256, tid, NT);
+    int32_t *misc = PS + 32;        // best E, step, sweep, slot, copy-from (r+1), changed, level bounds
+    constexpr int NT = 256;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
+    uint32_t *TQ = reinterpret_cast<uint32_t *>(misc + 8) + (size_t)warp * a.qcap * Sh::entry;   // this warp's tie queue
+    int rank = 0, csize = 1;
+    if (CL) {
+        rank = (int)cg::this_cluster().block_rank();
+        csize = (int)cg::this_cluster().num_blocks();
     }
-    for (int i = tid; i <= a.g.ncol; i += NT) cls[i] = a.g.cls[i];
+    const MscPeers<CL> W{Wsm, rank, csize};
+    int32_t *E0 = CL ? cg::this_cluster().map_shared_rank(Eacc, 0) : Eacc;
+    auto barrier = [&]() {
+        if (CL) cg::this_cluster().sync();
+        else __syncthreads();
+    };
 
-    const int ncl = (int)(gridDim.x >> 1);
-    for (int lb = (int)(blockIdx.x >> 1); lb < a.nblk; lb += ncl) {   // uniform within the cluster
+    if (tid < 2) misc[6 + tid] = 0;
+    __syncthreads();
+    const uint32_t *tab = a.tables + (size_t)a.tidx[a.k] * (a.g.mmax + 1);
+    for (int m = tid; m < Sh::nm; m += NT) {
+        const uint32_t Tm = m > 0 && m <= a.g.mmax ? tab[m] : 0u;
+        Tt[m] = Tm;
+        if (Tm >> 24) atomicMax(&misc[6], (m + 1) >> 1);   // e + 1 of this m
+        if (Tm) atomicMax(&misc[7], (m + 1) >> 1);
+        const uint32_t T = m + 1 <= a.g.mmax ? tab[m + 1] : 0u;   // entry m: m + 1 = 2e + 1 or 2e + 2
+        if (Sh::wide) {
+            uint32_t lo = 0u, hi = 0u;
+            for (int b = 0; b < 4; ++b) {
+                lo |= ((T >> (24 + b)) & 1u) * (0xFFu << (8 * b));
+                hi |= ((T >> (28 + b)) & 1u) * (0xFFu << (8 * b));
+            }
+            lvl[2 * m] = lo;
+            lvl[2 * m + 1] = hi;
+        } else {
+            for (int b = 0; b < 8; ++b) lvl[8 * m + b] = 0u - ((T >> (24 + b)) & 1u);
+            for (int b = 0; b < 4; ++b) init[4 * m + b] = 0u - ((~((uint32_t)m >> 1) >> b) & 1u);   // m: a degree here
+        }
+    }
+    for (int i = tid; i <= a.g.ncol; i += NT) cls[i] = a.g.csl[i];   // slices of each class
+
+    const int nunits = (int)gridDim.x / csize;
+    for (int lb = (int)blockIdx.x / csize; lb < a.nblk; lb += nunits) {   // uniform within a cluster
         const int blk = a.blk_base + lb;
         const int slot0 = blk * 32;
         if (tid < 32) PS[tid] = act ? a.parent[slot0 + tid] : slot0 + tid;
@@ -1201,51 +1175,99 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 4) k_sweep_msc_
         }
         __syncthreads();
         if (tid < 32 && rank == 0) Eacc[tid] = a.E_in[PS[tid]];
+        // Load: 32 int8 spin rows -> one bit word per position.
         for (int c = tid; c < (np >> 2); c += NT) {
             uint32_t w4[4];
             msc_pack_rows(a.spins_in, PS, np, c, w4);
 #pragma unroll
             for (int j = 0; j < 4; ++j) Wsm[4 * c + j] = w4[j];
         }
-        cluster.sync();   // both copies loaded, energies in place
+        barrier();   // all copies loaded, energies in place
+        const MscLevels L{misc[6], misc[7]};
         uint32_t vmask = 0u;   // bits of the live replicas
         for (int r = 0; r < 32; ++r) vmask |= (slot0 + r < a.R ? 1u : 0u) << msc_bit(r);
         uint32_t nacc = 0;
-        uint32_t ebias[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-        int cnt = 0;
+        uint32_t S[Sh::acc_planes];
+#pragma unroll
+        for (int b = 0; b < Sh::acc_planes; ++b) S[b] = 0u;
+        int cnt = 0;   // items per lane in S
+        const int w0 = warp * csize + rank, nw = (NT / 32) * csize;
+        // Descriptor and vertices of the warp's next slice, read one slice ahead.
+        uint2 d = make_uint2(0u, 0u);
+        uint32_t vd = 0u;
+        auto ahead = [&](int k) {
+            d = __ldg(&a.g.msl[k]);
+            vd = __ldg(&a.g.mvd[32 * k + lane]);
+        };
+        if (w0 < cls[1]) ahead(w0);
         for (int s = 0; s < nsweeps; ++s) {
             const uint32_t c3 = TAG_SWEEP | (uint32_t)s;
             for (int c = 0; c < a.g.ncol; ++c) {
-                const int p0 = cls[c], p1 = cls[c + 1];
-                const int nr = (p1 - p0 + 2 * NT - 1) / (2 * NT);   // rounds, uniform over the cluster
+                const int k1 = cls[c + 1];
                 int qc = 0;   // entries in this warp's tie queue
-                for (int rd = 0; rd < nr; ++rd) {
-                    const int p = p0 + 2 * tid + rank + rd * 2 * NT;
-                    uint32_t tent = 0u;
-                    if (p < p1) {
-                        const uint32_t x = Wsm[p];
-                        const uint32_t acc32 = msc_item<NPL, WEIGHTED>(a, Wsm, MscPackedE<NPL>::value ? PT : T256, p, x, c3,
-                                                                       blk, E0, ebias, tent);
-                        if (acc32) {
-                            Wsm[p] = x ^ acc32;
-                            Wpeer[p] = x ^ acc32;
-                            nacc += __popc(acc32 & vmask);
-                        }
-                        ++cnt;
+                for (int k = cls[c] + w0; k < k1; k += nw) {
+                    constexpr uint32_t bytes = sizeof(MscUnit<BIG>);
+                    const MscSlice sl{vd, (d.x & 0xFFFFFFu) * (32u * bytes) + bytes * (uint32_t)lane,
+                                      __shfl_sync(0xFFFFFFFFu, d.x >> 24, 0)};
+                    const uint32_t p = d.y + (uint32_t)lane;   // past the class: still inside the block's memory
+                    const uint32_t x = Wsm[p];
+                    if (k + nw < k1) ahead(k + nw);
+                    uint32_t tie, odd, E[N];
+                    const uint32_t acc = msc_item<N, WEIGHTED, BIG>(a, Wsm, lvl, init, L, sl, x, c3, blk, E, S, tie, odd);
+                    if (acc) {
+                        W.store(p, x ^ acc);
+                        nacc += __popc(acc & vmask);
                     }
-                    msc_queue_tie(a, TQ, qc, tent, Wsm, Wpeer, E0, blk, c3, vmask, nacc, lane);
-                    if (MscPackedE<NPL>::value && ((rd & 3) == 3 || rd == nr - 1))
-                        msc_flush_energy(ebias, cnt, E0, lane);
+                    const uint32_t bal = __ballot_sync(0xFFFFFFFFu, tie != 0u);
+                    const int nt = __popc(bal);
+                    if (qc + nt > a.qcap) {
+                        msc_drain_ties<N, CL>(a, Tt, TQ, qc, W, E0, blk, c3, vmask, nacc, lane);
+                        qc = 0;
+                    }
+                    int rk = qc + __popc(bal & ((1u << lane) - 1u));
+                    qc += nt;
+                    for (;;) {   // once, unless the queue is shorter than the ties of one slice
+                        if (tie && (uint32_t)rk < (uint32_t)a.qcap) {
+                            uint32_t *q = TQ + Sh::entry * rk;
+                            uint32_t v[10] = {tie, p | sl.vd << 16, odd, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+#pragma unroll
+                            for (int b = 0; b < N - 1; ++b) v[3 + b] = E[b];
+                            if (Sh::entry == 8) {
+                                *reinterpret_cast<uint4 *>(q) = make_uint4(v[0], v[1], v[2], v[3]);
+                                *reinterpret_cast<uint4 *>(q + 4) = make_uint4(v[4], v[5], v[6], v[7]);
+                            } else {
+#pragma unroll
+                                for (int b = 0; b < Sh::entry; b += 2)
+                                    *reinterpret_cast<uint2 *>(q + b) = make_uint2(v[b], v[b + 1]);
+                            }
+                        }
+                        if (qc <= a.qcap) break;
+                        msc_drain_ties<N, CL>(a, Tt, TQ, a.qcap, W, E0, blk, c3, vmask, nacc, lane);
+                        rk -= a.qcap;
+                        qc -= a.qcap;
+                    }
+                    if (++cnt == Sh::flush_items) {
+                        msc_flush_energy<N>(S, E0, lane);
+                        cnt = 0;
+                    }
                 }
-                if (qc) msc_drain_ties(a, TQ, qc, Wsm, Wpeer, E0, blk, c3, vmask, nacc, lane);
-                cluster.sync();
+                {
+                    const int cn = c + 1 < a.g.ncol ? c + 1 : 0, kc = cls[cn] + w0;
+                    if (kc < cls[cn + 1]) ahead(kc);
+                }
+                if (qc) msc_drain_ties<N, CL>(a, Tt, TQ, qc, W, E0, blk, c3, vmask, nacc, lane);
+                if (c + 1 == a.g.ncol && cnt) {
+                    msc_flush_energy<N>(S, E0, lane);
+                    cnt = 0;
+                }
+                barrier();
             }
-            if (rank == 0 && tid == 0) {
-                int bq = -1, bE = 0x7FFFFFFF;
-                for (int q = 0; q < 32; ++q)
-                    if (slot0 + q < a.R && Eacc[q] < bE) { bE = Eacc[q]; bq = q; }
-                misc[4] = 0;
-                if (bq >= 0) {
+            if (rank == 0 && warp == 0) {   // lowest energy of the sweep, the lowest slot first
+                const int v = slot0 + lane < a.R ? Eacc[lane] : 0x7FFFFFFF;
+                const int bE = __reduce_min_sync(0xFFFFFFFFu, v);
+                const int bq = __ffs(__ballot_sync(0xFFFFFFFFu, v == bE)) - 1;
+                if (lane == 0) {
+                    misc[4] = 0;
                     atomicMin(&a.sweep_emin[(size_t)a.k * a.S + s], bE);
                     if (bE < misc[0]) {
                         misc[0] = bE; misc[1] = a.k; misc[2] = s; misc[3] = slot0 + bq;
@@ -1254,7 +1276,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 4) k_sweep_msc_
                 }
             }
             __syncthreads();
-            if (misc[4]) {   // CTA 0 only (CTA 1 never sets it)
+            if (misc[4]) {   // in a cluster: CTA 0 only (the others never set it)
                 const int rq = misc[4] - 1;
                 uint32_t *dst = reinterpret_cast<uint32_t *>(a.best_cfg + (size_t)blk * np);
                 for (int c = tid; c < (np >> 2); c += NT) {
@@ -1266,11 +1288,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 4) k_sweep_msc_
                     }
                     dst[c] = v;
                 }
+                if (!CL) __syncthreads();
             }
-            cluster.sync();   // the copy reads CTA 0's words before the next sweep changes them
+            if (CL) barrier();   // the copy reads CTA 0's words before the next sweep changes them
         }
-        // Store: each CTA writes half of the columns from its own (complete) copy.
-        for (int c = 2 * tid + rank; c < (np >> 2); c += 2 * NT) {
+        // Store: bit words -> int8 spin rows (fields are not kept by this
+        // layout); the CTAs of a cluster share the columns.
+        for (int c = csize * tid + rank; c < (np >> 2); c += csize * NT) {
             uint32_t w4[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) w4[j] = Wsm[4 * c + j];
@@ -1282,26 +1306,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 4) k_sweep_msc_
         }
         const uint32_t wsum = __reduce_add_sync(0xFFFFFFFFu, nacc);
         if (act && lane == 0 && wsum) atomicAdd(&a.accepts[a.k], (unsigned long long)wsum);
-        cluster.sync();   // neither copy is reused before both CTAs are done with this word
+        barrier();   // no copy is reused before all CTAs are done with this word
     }
 }
 
-template <bool W>
-void *msc_pair_kernel(int mmax) {
-    if (mmax <= 7) return reinterpret_cast<void *>(&k_sweep_msc_pair<3, W>);
-    if (mmax <= 15) return reinterpret_cast<void *>(&k_sweep_msc_pair<4, W>);
-    if (mmax <= 31) return reinterpret_cast<void *>(&k_sweep_msc_pair<5, W>);
-    if (mmax <= 63) return reinterpret_cast<void *>(&k_sweep_msc_pair<6, W>);
-    return reinterpret_cast<void *>(&k_sweep_msc_pair<7, W>);
+template <bool W, bool BIG, bool CL>
+void *msc_kernel(int mmax) {
+    switch (msc_planes(mmax)) {
+        case 3: return reinterpret_cast<void *>(&k_sweep_msc<3, W, BIG, CL>);
+        case 4: return reinterpret_cast<void *>(&k_sweep_msc<4, W, BIG, CL>);
+        case 5: return reinterpret_cast<void *>(&k_sweep_msc<5, W, BIG, CL>);
+        case 6: return reinterpret_cast<void *>(&k_sweep_msc<6, W, BIG, CL>);
+        default: return reinterpret_cast<void *>(&k_sweep_msc<7, W, BIG, CL>);
+    }
 }
 
-template <bool W>
-void *msc_kernel(int mmax) {
-    if (mmax <= 7) return reinterpret_cast<void *>(&k_sweep_msc<3, W, 256, 4>);
-    if (mmax <= 15) return reinterpret_cast<void *>(&k_sweep_msc<4, W, 256, 4>);
-    if (mmax <= 31) return reinterpret_cast<void *>(&k_sweep_msc<5, W, 256, 4>);
-    if (mmax <= 63) return reinterpret_cast<void *>(&k_sweep_msc<6, W, 256, 4>);
-    return reinterpret_cast<void *>(&k_sweep_msc<7, W, 256, 4>);   // c <= 127: mb = 2c + 128 - deg stays in a byte
+template <bool W, bool BIG>
+void *msc_kernel(int mmax, bool cluster) {
+    return cluster ? msc_kernel<W, BIG, true>(mmax) : msc_kernel<W, BIG, false>(mmax);
 }
 
 template <bool W>
@@ -1322,9 +1344,11 @@ void *kernel_ptr() {
     return reinterpret_cast<void *>(&k_sweep<G, FB, W>);
 }
 
-void *select_kernel(int G, int fb, bool weighted, int threads, int mmax) {
-    if (fb == 1) return weighted ? msc_kernel<true>(mmax) : msc_kernel<false>(mmax);
-    if (fb == 2) return weighted ? msc_pair_kernel<true>(mmax) : msc_pair_kernel<false>(mmax);
+void *select_kernel(int G, int fb, bool weighted, int threads, int mmax, bool big) {
+    if (fb == 1 || fb == 2) {
+        if (big) return weighted ? msc_kernel<true, true>(mmax, fb == 2) : msc_kernel<false, true>(mmax, fb == 2);
+        return weighted ? msc_kernel<true, false>(mmax, fb == 2) : msc_kernel<false, false>(mmax, fb == 2);
+    }
     if (fb == 7) return weighted ? packed_kernel<true>(threads) : packed_kernel<false>(threads);
     if (G == 1) {
         if (fb == 16) return weighted ? kernel_ptr<1, 16, true>() : kernel_ptr<1, 16, false>();
@@ -1338,9 +1362,7 @@ void *select_kernel(int G, int fb, bool weighted, int threads, int mmax) {
 
 size_t sweep_smem_bytes(const GraphDev &g, int G, int field_bits, int threads) {
     if (field_bits == 1 || field_bits == 2)   // multi-spin coded: 32 replicas per word (2: CTA pairs)
-        return (size_t)g.np * 4 + (256 + (size_t)msc_pair_words(g.mmax)) * 4 + (size_t)((g.ncol + 1 + 3) & ~3) * 4 +
-               (32 + 32 + 8) * 4 +
-               (size_t)(threads / 32) * 64 * 4;   // tie queues
+        return ((size_t)g.np + msc_reserved_words(g.mmax) + ((g.ncol + 1 + 3) & ~3)) * 4;
     if (field_bits == 7)
         return (size_t)(g.np + 32) * 4 + 256 * 4 + (size_t)((g.ncol + 1 + 3) & ~3) * 4 + 16 * 4 +
                (size_t)((((g.np + 31) / 32) + 1) & ~1) * 4 + (size_t)(threads / 32) * PK_QCAP * 8;
@@ -1357,8 +1379,24 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
     } else if (field_bits == 7) {
         G = 1;
     }
-    const size_t smem = sweep_smem_bytes(g, G, field_bits, threads);
-    void *fn = select_kernel(G, field_bits, weighted, threads, g.mmax);
+    size_t smem = sweep_smem_bytes(g, G, field_bits, threads);
+    if (field_bits == 1 || field_bits == 2) {
+        // Tie queues: 64 entries per warp, 40 where 64 would cost a resident
+        // block, and what the reserved words leave when the graph fills shared
+        // memory.
+        int dev = 0, limit = 0, per_sm = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+        const size_t fixed = ((size_t)g.np + msc_table_words(g.mmax) + 72 + ((g.ncol + 1 + 3) & ~3)) * 4;
+        const size_t per_entry = (size_t)(threads / 32) * msc_entry_words(g.mmax) * 4;
+        auto resident = [&](int cap) { return std::min<size_t>(4, (size_t)per_sm / (fixed + cap * per_entry + 1024)); };
+        cfg->qcap = resident(64) < resident(40) ? 40 : 64;
+        if (fixed + cfg->qcap * per_entry > (size_t)limit) cfg->qcap = (int)((smem - fixed) / per_entry);
+        if (cfg->qcap < 1) return cudaErrorInvalidConfiguration;
+        smem = fixed + cfg->qcap * per_entry;
+    }
+    void *fn = select_kernel(G, field_bits, weighted, threads, g.mmax, g.mbig != 0);
     // The attribute belongs to the kernel function, not to a context: only ever
     // raise it, so that contexts configured earlier keep launching.
     {
@@ -1382,6 +1420,12 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
         lc.gridDim = dim3(2 * nblk);
         lc.blockDim = dim3(threads);
         lc.dynamicSmemBytes = smem;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 2;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        lc.attrs = at;
+        lc.numAttrs = 1;
         int ncl = 0;
         cudaError_t e = cudaOccupancyMaxActiveClusters(&ncl, fn, &lc);
         if (e != cudaSuccess) return e;
@@ -1405,9 +1449,22 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
 }
 
 cudaError_t launch_sweep(const SweepConfig &cfg, const SweepArgs &a, cudaStream_t st) {
-    void *fn = select_kernel(cfg.G, cfg.field_bits, a.g.wt != nullptr, cfg.threads, a.g.mmax);
-    void *args[] = {const_cast<SweepArgs *>(&a)};
-    return cudaLaunchKernel(fn, dim3(cfg.grid), dim3(cfg.threads), args, cfg.smem, st);
+    void *fn = select_kernel(cfg.G, cfg.field_bits, a.g.wt != nullptr, cfg.threads, a.g.mmax, a.g.mbig != 0);
+    SweepArgs b = a;
+    b.qcap = cfg.qcap;
+    void *args[] = {&b};
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(cfg.grid);
+    lc.blockDim = dim3(cfg.threads);
+    lc.dynamicSmemBytes = cfg.smem;
+    lc.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    lc.attrs = at;
+    lc.numAttrs = cfg.field_bits == 2 ? 1 : 0;
+    return cudaLaunchKernelExC(&lc, fn, args);
 }
 
 }  // namespace pa

@@ -151,8 +151,8 @@ struct pa_ctx {
     std::vector<uint32_t> rp_p;         // position-order CSR
     std::vector<uint16_t> col_p;
     std::vector<int8_t> w_p;
-    DevBuf d_rp, d_col, d_w, d_vid, d_cls, d_pos, d_parity, d_prp, d_pcol, d_mrp, d_mcol;
-    bool packed_ok = false, msc_rows = false;
+    DevBuf d_rp, d_col, d_w, d_vid, d_cls, d_pos, d_parity, d_prp, d_pcol, d_msl, d_csl, d_mvd, d_mcol;
+    bool packed_ok = false, msc_rows = false, msc_big = false;
     RunState run;
     std::string err;
     int64_t h2d = 0, d2h = 0;
@@ -172,8 +172,11 @@ struct pa_ctx {
         g.prp = d_prp.as<uint32_t>();
         g.pcol = d_pcol.as<uint2>();
         g.packed_ok = packed_ok ? 1 : 0;
-        g.mrp = msc_rows ? d_mrp.as<uint32_t>() : nullptr;
-        g.mcol = msc_rows ? d_mcol.as<uint2>() : nullptr;
+        g.msl = msc_rows ? d_msl.as<uint2>() : nullptr;
+        g.csl = msc_rows ? d_csl.as<int32_t>() : nullptr;
+        g.mvd = msc_rows ? d_mvd.as<uint32_t>() : nullptr;
+        g.mcol = msc_rows ? d_mcol.p : nullptr;
+        g.mbig = msc_big ? 1 : 0;
         return g;
     }
 };
@@ -481,29 +484,59 @@ int pa_create(pa_ctx **out, int32_t n, const uint32_t *row_ptr, const uint16_t *
         e1 = copy(c, c->d_prp.p, prp.data(), 4 * (size_t)(n + 1), cudaMemcpyHostToDevice);
         if (e1 == cudaSuccess) e1 = copy(c, c->d_pcol.p, pcol.data(), 2 * pcol.size(), cudaMemcpyHostToDevice);
     }
-    c->msc_rows = c->np <= 16384 && c->maxdeg <= 127;
+    c->msc_rows = c->maxdeg <= 127;
+    c->msc_big = c->np > 16384;
     if (e1 == cudaSuccess && c->msc_rows) {
-        std::vector<uint32_t> mrp(n + 1, 0u);
+        std::vector<uint2> msl;
+        std::vector<int32_t> csl(ncol + 1, 0);
+        std::vector<uint32_t> mvd;
         uint32_t units = 0;
-        for (int32_t p = 0; p < n; ++p) {
-            const uint32_t d = c->rp_p[p + 1] - c->rp_p[p];
-            mrp[p] = units << 8 | d;
-            units += (d + 3) / 4;
+        for (int32_t k = 0; k < ncol; ++k) {
+            for (int32_t p0 = c->cls[k]; p0 < c->cls[k + 1]; p0 += 32) {
+                const int32_t p1 = std::min(p0 + 32, c->cls[k + 1]);
+                uint32_t most = 1;   // at least one unit: lanes without neighbours count their own word
+                for (int32_t p = p0; p < p1; ++p) most = std::max(most, (c->rp_p[p + 1] - c->rp_p[p] + 3) / 4);
+                msl.push_back(make_uint2(units | most << 24, (uint32_t)p0));
+                for (int32_t p = p0; p < p0 + 32; ++p)
+                    mvd.push_back(p < p1 ? c->vid[p] | (c->rp_p[p + 1] - c->rp_p[p]) << 16 : 0x80000000u);
+                units += most;
+            }
+            csl[k + 1] = (int32_t)msl.size();
         }
-        mrp[n] = units << 8;
-        std::vector<uint16_t> mcol((size_t)units * 4 + 4);
-        for (int32_t p = 0; p < n; ++p) {
-            size_t o = (size_t)(mrp[p] >> 8) * 4;
-            for (uint32_t e = c->rp_p[p]; e < c->rp_p[p + 1]; ++e, ++o)
-                mcol[o] = (uint16_t)(4u * c->col_p[e] | (c->w_p[e] < 0 ? 1u : 0u));
-            for (; o < (size_t)(mrp[p + 1] >> 8) * 4; ++o) mcol[o] = (uint16_t)(4u * (uint32_t)p);
+        const size_t esz = c->msc_big ? 4 : 2;
+        std::vector<unsigned char> mcol((size_t)units * 128 * esz);
+        for (const uint2 &d : msl) {
+            const size_t k = (size_t)(&d - msl.data());
+            for (uint32_t u = 0; u < d.x >> 24; ++u)
+                for (uint32_t lane = 0; lane < 32; ++lane) {
+                    const bool live = !(mvd[32 * k + lane] >> 31);
+                    const uint32_t p = d.y + (live ? lane : 0u);
+                    const uint32_t e0 = c->rp_p[p] + 4 * u, e1p = live ? c->rp_p[p + 1] : 0u;
+                    uint32_t off[4], neg[4];
+                    for (uint32_t j = 0; j < 4; ++j) {
+                        const bool real = e0 + j < e1p;
+                        off[j] = 4u * (real ? (uint32_t)c->col_p[e0 + j] : p);
+                        neg[j] = real && c->w_p[e0 + j] < 0 ? 1u : 0u;
+                    }
+                    const size_t at = ((size_t)((d.x & 0xFFFFFFu) + u) * 32 + lane) * 4;
+                    for (uint32_t j = 0; j < 4; ++j) {
+                        if (c->msc_big)
+                            reinterpret_cast<uint32_t *>(mcol.data())[at + j] = off[j] | neg[j];
+                        else
+                            reinterpret_cast<uint16_t *>(mcol.data())[at + j] =
+                                (uint16_t)(off[j] | ((j & 1u) ? 0u : neg[j] | neg[j + 1] << 1));
+                    }
+                }
         }
-        if (!c->d_mrp.alloc(4 * (size_t)(n + 1)) || !c->d_mcol.alloc(2 * mcol.size())) {
+        if (!c->d_msl.alloc(8 * msl.size()) || !c->d_csl.alloc(4 * csl.size()) || !c->d_mvd.alloc(4 * mvd.size()) ||
+            !c->d_mcol.alloc(mcol.size())) {
             delete c;
             return PA_ENOMEM;
         }
-        e1 = copy(c, c->d_mrp.p, mrp.data(), 4 * (size_t)(n + 1), cudaMemcpyHostToDevice);
-        if (e1 == cudaSuccess) e1 = copy(c, c->d_mcol.p, mcol.data(), 2 * mcol.size(), cudaMemcpyHostToDevice);
+        e1 = copy(c, c->d_msl.p, msl.data(), 8 * msl.size(), cudaMemcpyHostToDevice);
+        if (e1 == cudaSuccess) e1 = copy(c, c->d_csl.p, csl.data(), 4 * csl.size(), cudaMemcpyHostToDevice);
+        if (e1 == cudaSuccess) e1 = copy(c, c->d_mvd.p, mvd.data(), 4 * mvd.size(), cudaMemcpyHostToDevice);
+        if (e1 == cudaSuccess) e1 = copy(c, c->d_mcol.p, mcol.data(), mcol.size(), cudaMemcpyHostToDevice);
     }
     if (e1 == cudaSuccess) {
         std::vector<uint32_t> par((c->np + 31) / 32, 0u);

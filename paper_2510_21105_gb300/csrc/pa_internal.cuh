@@ -94,13 +94,22 @@ struct GraphDev {
     const uint32_t *prp;     // [n+1] row starts in units of 4 entries
     const uint2 *pcol;       // [prp[n]] four 16-bit entries each
     int32_t packed_ok;       // the padded encoding exists (np + 32 <= 32768)
-    // Rows for the multi-spin-coded kernels (np <= 16384, degree <= 127), padded
-    // to multiples of 4 entries: entry = 4 * neighbour position (the byte
-    // offset of its word) | 1 if the weight is -1; padding entries point at the
-    // row's own position (its word XOR itself counts nothing). mrp[p] = (row
-    // start in units of 4 entries) << 8 | degree. nullptr when absent.
-    const uint32_t *mrp;     // [n+1]
-    const uint2 *mcol;       // [mrp[n] >> 8]
+    // Rows for the multi-spin-coded kernels (degree <= 127), in slices of 32
+    // consecutive positions of one colour class, one lane each: msl[k] = (first
+    // unit | units << 24, first position), csl the class bounds in slices,
+    // mvd[32 k + lane] = vertex | degree << 16, bit 31 on lanes past the class.
+    // A unit holds four bonds of each lane, lane after lane, so a warp reads it
+    // in one contiguous piece and all lanes run the slice's largest unit count
+    // (positions are sorted by degree). Entries are byte offsets of the
+    // neighbours' words (4 * position): 16 bits up to np = 16384, with the signs
+    // of entries 2j and 2j + 1 (weight -1) in bits 0 and 1 of entry 2j, else
+    // (mbig) 32 bits with the sign in bit 0. Padding entries point at the lane's
+    // own position (its word XOR itself counts nothing).
+    const uint2 *msl;
+    const int32_t *csl;      // [ncol+1]
+    const uint32_t *mvd;
+    const void *mcol;        // nullptr when absent
+    int32_t mbig;
 };
 
 struct SweepArgs {
@@ -117,6 +126,7 @@ struct SweepArgs {
     const int32_t *active;       // [K] 0 = skip the step (adaptive end), may be null
     int32_t R, nblk, S, k;       // nblk: replica blocks of this launch
     int32_t blk_base;            // first replica block of this launch (multi-spin-coded kernels)
+    int32_t qcap;                // multi-spin coded: tie-queue entries per warp
     uint32_t key0, key1;
     uint32_t rk0[10], rk1[10];   // Philox round keys key + r * (0x9E3779B9, 0xBB67AE85)
     int4 *best_rec;              // [all blocks] (E, step, sweep, slot) per replica block
@@ -161,6 +171,7 @@ struct SweepConfig {
     int threads;
     int grid;
     size_t smem;
+    int qcap = 0;   // multi-spin coded: tie-queue entries per warp
 };
 // Dynamic shared memory of one sweep CTA (G: 4-replica groups of the int8/int16 layouts;
 // field_bits 1/2 multi-spin coded, 7 packed, 8/16 int8/int16 fields).
