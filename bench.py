@@ -231,7 +231,7 @@ def run_reference(args, rank, world):
 # tail launches of the multi-spin-coded sweep, or the one launch of another
 # layout), from one ncu capture, with the SHA-256 prefix of the sweep source it
 # was taken on: reported only while that source is the one that runs.
-SWEEP_TRAFFIC = {"k_sweep_msc+pair": ((102.875648 + 44.824064 + 12.869376) * 1e6, "6ca9288e529d8511")}
+SWEEP_TRAFFIC = {}   # none captured on the current source
 SWEEP_SRC = os.path.join(ROOT, "paper_2510_21105_gb300", "csrc", "k_sweep.cu")
 INT_LANES_PER_SM = 128   # ALU pipe 64 + FMA pipe 64 integer lanes per SM and clock (unit counts)
 SMEM_BYTES_PER_SM = 128  # shared-memory bytes per SM and clock (32 banks x 4 B)
@@ -251,7 +251,10 @@ def msc_planes(max_degree: int) -> int:
 
 def msc_ops_per_attempt(mean_degree: float, max_degree: int = 31) -> float:
     """Algorithmic integer instructions of one multi-spin-coded attempt: one
-    item (one position of a 32-replica word) divided by its 32 attempts.
+    item (one position of a 32-replica word) divided by its 32 attempts, in the
+    byte-per-replica formulation. The kernel now decides in bit planes; the
+    count stays that of the byte formulation, so that the reported fraction of
+    the integer peak compares across builds.
       bond counting   per 4 bonds, three-input logic ops of the carry-save
                       adders: 7 + 2 (NPL - 3) with the planes kept
                       complemented (NPL >= 4), 13 with plain adders from
