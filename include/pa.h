@@ -417,15 +417,15 @@ void pa_set_allocator(pa_alloc_fn alloc, pa_free_fn free_fn, void *user);
  *             stream; with NULL the call only enqueues work and returns
  *   stream    cudaStream_t, NULL = legacy default stream
  *
- * Scratch lives in a fixed file-scope device array of about 0.6 MB that every
- * GPU loading the library holds until the process exits; no cudaMalloc,
- * cudaFree or allocating library routine is called. The first call on a
- * device looks up that array's device address (cudaGetSymbolAddress) with
- * the device current, so make the first call on each device before any stream
- * capture. All calls share the array and it keeps the last call's contents;
- * every call writes each scratch word before reading it, so nothing needs
- * clearing between calls. Calls that overlap on the GPU (other streams, other
- * threads) race on it. Returns PA_OK, PA_EINVAL or PA_ECUDA.
+ * The four results live in a fixed file-scope device record (24 bytes) that
+ * every GPU loading the library holds until the process exits; everything else
+ * stays in registers and shared memory. No cudaMalloc, cudaFree or allocating
+ * library routine is called. The first call on a device looks up that record's
+ * device address (cudaGetSymbolAddress) with the device current, so make the
+ * first call on each device before any stream capture. All calls share the
+ * record and it keeps the last call's contents; every call writes all of it.
+ * Calls that overlap on the GPU (other streams, other threads) race on it.
+ * Returns PA_OK, PA_EINVAL or PA_ECUDA.
  */
 #define PA_NOALLOC_MAX_R 32768
 

@@ -140,29 +140,6 @@ __global__ void __launch_bounds__(RS_CHUNK) k_rs_weights(ResampleArgs a) {
     }
 }
 
-// floor((P R 2^32 + o T) / (T 2^32)) for R <= 65536, written as
-// floor(P R / T) + [ (P R mod T) 2^32 >= T (2^32 - o) ]. The division by T
-// goes through m = floor((2^64 - 1) / T), computed once per step: q =
-// mulhi(X, m) satisfies X/T - 2 < q <= X/T (m >= (2^64 - T)/T and X < 2^64),
-// so at most two corrections make it exact.
-__device__ __forceinline__ int32_t systematic_count_m(unsigned long long P, int32_t R, unsigned long long T,
-                                                      unsigned long long m, uint32_t o) {
-    if (P >= T) return R;
-    const unsigned long long X = P * (unsigned long long)R;
-    unsigned long long q = __umul64hi(X, m), r = X - q * T;
-    if (r >= T) {
-        ++q;
-        r -= T;
-    }
-    if (r >= T) {
-        ++q;
-        r -= T;
-    }
-    const unsigned __int128 lhs = (unsigned __int128)r << 32;
-    const unsigned __int128 rhs = (unsigned __int128)T * (0x100000000ull - (unsigned long long)o);
-    return (int32_t)(q + (lhs >= rhs ? 1ull : 0ull));
-}
-
 __global__ void __launch_bounds__(RS_CHUNK) k_rs_parents(ResampleArgs a) {
     if (a.active && !a.active[a.k]) return;
     __shared__ unsigned long long sh_T, sh_off, sh_m;

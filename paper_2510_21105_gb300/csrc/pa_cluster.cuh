@@ -1,0 +1,186 @@
+// pa_cluster.cuh -- the weight arithmetic of one resampling over a population
+// (or one rank's shard of it) in a single thread-block cluster: used by the
+// resampling entry points on caller buffers, where a launch has to do all of
+// it by itself.
+//
+// n slots, padded with zero weights to L = 1024 K C: CTA c of the C <= 8 CTAs
+// holds the aligned range of L / C slots, thread t of it K consecutive ones in
+// registers. So the pairwise tree (s_i <- s_2i + s_2i+1) runs inside the thread,
+// over the lanes, over the warps and over the CTAs, in the order of the
+// level-by-level tree, and the integer prefix likewise; two cluster barriers
+// replace the passes over global memory.
+#pragma once
+
+#include <cooperative_groups.h>
+
+#include "pa_internal.cuh"
+
+namespace pa {
+
+constexpr int CL_THREADS = 1024;
+constexpr int CL_CTAS = 8;        // portable cluster size
+constexpr int CL_LOW = 8;         // low bits of E - E_min whose products are tabled
+
+struct QPow {
+    double v[32];   // squarings of q = exp(-(beta_k - beta_prev))
+};
+
+// CTAs and slots per thread for n slots (n <= 65536).
+struct ClusterShape {
+    int ctas, k;
+};
+__host__ inline ClusterShape cluster_shape(int32_t n) {
+    int L = CL_THREADS;
+    while (L < n) L <<= 1;
+    ClusterShape s;
+    s.ctas = L / CL_THREADS < CL_CTAS ? L / CL_THREADS : CL_CTAS;
+    s.k = L / (CL_THREADS * s.ctas);
+    return s;
+}
+
+struct ClusterShared {
+    double tab[1 << CL_LOW];          // products of the squarings over the bits of the index
+    double wsum[32];
+    unsigned long long tsum[32];
+    int32_t mn[32];
+    double ctaA;
+    unsigned long long ctaT;
+    int32_t ctaMin;
+    double A;                          // totals over the cluster (every CTA has them)
+    unsigned long long T, before;      // before: total of the lower CTAs
+    int32_t emin;
+};
+
+// Products over the low bits, multiplied in ascending bit order from 1.0, so a
+// weight that starts from its entry is rounded as the plain product is.
+__device__ __forceinline__ void cluster_table(ClusterShared &sh, const QPow &qp) {
+    for (int i = threadIdx.x; i < (1 << CL_LOW); i += CL_THREADS) {
+        double w = 1.0;
+#pragma unroll
+        for (int b = 0; b < CL_LOW; ++b)
+            if ((i >> b) & 1) w = __dmul_rn(w, qp.v[b]);
+        sh.tab[i] = w;
+    }
+}
+
+__device__ __forceinline__ double cluster_weight(const ClusterShared &sh, const QPow &qp, uint32_t d) {
+    double w = sh.tab[d & ((1u << CL_LOW) - 1u)];
+    d >>= CL_LOW;
+    while (d) {
+        w = __dmul_rn(w, qp.v[CL_LOW + __ffs(d) - 1]);
+        d &= d - 1u;
+    }
+    return w;
+}
+
+// E_min over the cluster of each thread's minimum.
+__device__ __forceinline__ int32_t cluster_min(ClusterShared &sh, int32_t v) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    v = __reduce_min_sync(0xFFFFFFFFu, v);
+    if (lane == 0) sh.mn[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        v = __reduce_min_sync(0xFFFFFFFFu, sh.mn[lane]);
+        if (lane == 0) sh.ctaMin = v;
+    }
+    cl.sync();
+    if (warp == 0) {
+        const int C = (int)cl.num_blocks();
+        v = *cl.map_shared_rank(&sh.ctaMin, lane < C ? lane : 0);
+        v = __reduce_min_sync(0xFFFFFFFFu, v);
+        if (lane == 0) sh.emin = v;
+    }
+    __syncthreads();
+    return sh.emin;
+}
+
+// Tree sum A, integer total T and each thread's exclusive prefix of t (over the
+// cluster) from the K weights a thread holds. Ends with sh.A, sh.T set in every
+// CTA; the caller closes with a cluster barrier before any CTA leaves.
+template <int K>
+__device__ __forceinline__ unsigned long long cluster_sums(ClusterShared &sh, const double (&w)[K],
+                                                           const unsigned long long (&t)[K]) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double s[K];
+    unsigned long long loc = 0ull;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        s[i] = w[i];
+        loc += t[i];
+    }
+#pragma unroll
+    for (int h = 1; h < K; h <<= 1)
+#pragma unroll
+        for (int i = 0; i < K; i += 2 * h) s[i] = __dadd_rn(s[i], s[i + h]);
+    double a = s[0];
+    unsigned long long inc = loc;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        a = __dadd_rn(a, __shfl_xor_sync(0xFFFFFFFFu, a, off));
+        const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, inc, off);
+        if (lane >= off) inc += y;
+    }
+    if (lane == 31) {
+        sh.wsum[warp] = a;
+        sh.tsum[warp] = inc;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        double b = sh.wsum[lane];
+        unsigned long long u = sh.tsum[lane];
+        const unsigned long long mine = u;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            b = __dadd_rn(b, __shfl_xor_sync(0xFFFFFFFFu, b, off));
+            const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, u, off);
+            if (lane >= off) u += y;
+        }
+        sh.tsum[lane] = u - mine;   // exclusive over the warps
+        if (lane == 31) {
+            sh.ctaA = b;
+            sh.ctaT = u;
+        }
+    }
+    cl.sync();
+    if (warp == 0) {
+        const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+        double b = lane < C ? *cl.map_shared_rank(&sh.ctaA, lane < C ? lane : 0) : 0.0;
+        unsigned long long T = lane < C ? *cl.map_shared_rank(&sh.ctaT, lane < C ? lane : 0) : 0ull;
+        unsigned long long before = lane < rank ? T : 0ull;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            b = __dadd_rn(b, __shfl_xor_sync(0xFFFFFFFFu, b, off));
+            T += __shfl_xor_sync(0xFFFFFFFFu, T, off);
+            before += __shfl_xor_sync(0xFFFFFFFFu, before, off);
+        }
+        if (lane == 0) {
+            sh.A = b;
+            sh.T = T;
+            sh.before = before;
+        }
+    }
+    __syncthreads();
+    return sh.before + sh.tsum[warp] + (inc - loc);
+}
+
+// Launches a cluster kernel of `shape` on st.
+template <class... P, class... A>
+cudaError_t launch_cluster(void (*kernel)(P...), const ClusterShape &shape, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(shape.ctas);
+    lc.blockDim = dim3(CL_THREADS);
+    lc.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = shape.ctas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, kernel, args...);
+}
+
+}  // namespace pa

@@ -77,6 +77,30 @@ static __device__ __forceinline__ bool accept_by_top_byte(uint32_t top, uint32_t
     return sweep_tail_bits(vid, slot, k, c3 & 0x0FFFFFFFu, key0, key1) < (T & 0xFFFFFFu);
 }
 
+// Systematic resampling: new slots filled by the weights before P.
+// floor((P R 2^32 + o T) / (T 2^32)) for R <= 65536, written as
+// floor(P R / T) + [ (P R mod T) 2^32 >= T (2^32 - o) ]. The division by T
+// goes through m = floor((2^64 - 1) / T), computed once per step: q =
+// mulhi(X, m) satisfies X/T - 2 < q <= X/T (m >= (2^64 - T)/T and X < 2^64),
+// so at most two corrections make it exact.
+static __device__ __forceinline__ int32_t systematic_count_m(unsigned long long P, int32_t R, unsigned long long T,
+                                                      unsigned long long m, uint32_t o) {
+    if (P >= T) return R;
+    const unsigned long long X = P * (unsigned long long)R;
+    unsigned long long q = __umul64hi(X, m), r = X - q * T;
+    if (r >= T) {
+        ++q;
+        r -= T;
+    }
+    if (r >= T) {
+        ++q;
+        r -= T;
+    }
+    const unsigned __int128 lhs = (unsigned __int128)r << 32;
+    const unsigned __int128 rhs = (unsigned __int128)T * (0x100000000ull - (unsigned long long)o);
+    return (int32_t)(q + (lhs >= rhs ? 1ull : 0ull));
+}
+
 constexpr int32_t EMIN_SENTINEL = 0x7F7F7F7F;  // byte-fillable "+infinity"
 constexpr int RS_CHUNK = 256;                   // slots per resampling CTA (power of two)
 
