@@ -68,11 +68,60 @@ __device__ __forceinline__ uint32_t pk_entry(int m, const uint32_t *tab, int mma
     return e * 0x00010001u;
 }
 
-template <int G, int FB, bool WEIGHTED>
-__device__ __forceinline__ void sweep_item(uint32_t *__restrict__ Ssm, uint32_t *__restrict__ Hsm,
-                                           const uint32_t *__restrict__ Tt, const SweepArgs &a,
-                                           int p, int g, uint32_t c1, uint32_t c3, uint32_t vmask,
-                                           int dE[4], uint32_t &nacc) {
+// ---------------------------------------------------------------------------
+// Field updates of accepted items, shared by the layouts that keep fields: an
+// accepted item (a position of one group of four replicas) adds its change to
+// every neighbour's field. The items of a round go to a queue of the block, and
+// after a barrier all threads of the block walk their rows, 2^lt lanes per row
+// with 2^lt the largest power of two that gives every queued item its lanes (so
+// few items on long rows still use the whole block). Bound: latency. n = 500,
+// mean degree 250, R = 1024, us per step of 4 sweeps: 765 with one thread per
+// row, 375 with the queue (512 threads).
+// Counters of three rounds and entries of two, so that one barrier per round
+// is enough: the counter a round uses was cleared after the barrier two rounds
+// before, and its entries were read before the barrier one round before.
+struct SweepQueue {
+    uint4 *ent;        // [2][threads]
+    int32_t *count;    // [3], zero at the start
+    int round;
+
+    __device__ __forceinline__ void push(bool have, const uint4 &e, int lane) {
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, have);
+        if (!bal) return;
+        int base = 0;
+        if (lane == 0) base = atomicAdd(&count[round % 3], __popc(bal));
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        if (have) ent[(size_t)(round & 1) * blockDim.x + base + __popc(bal & ((1u << lane) - 1u))] = e;
+    }
+    // Closes the round for the whole block; walk(entry, lane of the row, lanes per row).
+    template <class F>
+    __device__ __forceinline__ void drain(F walk) {
+        __syncthreads();
+        const int total = count[round % 3];
+        if (threadIdx.x == 0) count[(round + 2) % 3] = 0;
+        if (total) {
+            const int lt = min(31 - __clz((int)blockDim.x / total), 7);
+            for (int t = threadIdx.x; t < (total << lt); t += blockDim.x)
+                walk(ent[(size_t)(round & 1) * blockDim.x + (t >> lt)], t & ((1 << lt) - 1), 1 << lt);
+        }
+        ++round;
+    }
+};
+__host__ __device__ inline size_t sweep_queue_bytes(int threads) { return (size_t)threads * 32 + 16; }
+
+// Top bytes of the four uniforms of group c1 at vertex vid: word c1 & 3 of the
+// call of slots 16 (c1 >> 2) ..
+__device__ __forceinline__ uint32_t group_uniforms(const SweepArgs &a, uint32_t vid, uint32_t c1, uint32_t c3) {
+    return word_of(philox10(make_uint4(vid, c1 >> 2, (uint32_t)a.k, c3), a.key0, a.key1), c1 & 3u);
+}
+
+// Decides the four replicas of an item and applies its own part; returns
+// whether any flipped, with the packed field changes D0, D1 of its neighbours.
+template <int G, int FB>
+__device__ __forceinline__ bool sweep_item(uint32_t *__restrict__ Ssm, const uint32_t *__restrict__ Hsm,
+                                           const uint32_t *__restrict__ Tt, const SweepArgs &a, int p, int g,
+                                           uint32_t vid, uint32_t uw, uint32_t c1, uint32_t c3, uint32_t vmask,
+                                           int dE[4], uint32_t &nacc, uint32_t &D0, uint32_t &D1) {
     const int widx = p * G + g;
     const uint32_t sw = Ssm[widx];
     uint32_t hw0, hw1 = 0;
@@ -94,9 +143,6 @@ __device__ __forceinline__ void sweep_item(uint32_t *__restrict__ Ssm, uint32_t 
             h = (int)((hw0 >> (8 * q)) & 0xFFu) - 128;
         m[q] = x[q] > 0 ? -h : h;   // dE = -2 x h = 2m
     }
-    // Top bytes of the four uniforms: word c1 & 3 of the call of slots 16 (c1 >> 2) ..
-    const uint32_t vid = __ldg(&a.g.vid[p]);
-    const uint32_t uw = word_of(philox10(make_uint4(vid, c1 >> 2, (uint32_t)a.k, c3), a.key0, a.key1), c1 & 3u);
     uint32_t acc = 0;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -104,43 +150,25 @@ __device__ __forceinline__ void sweep_item(uint32_t *__restrict__ Ssm, uint32_t 
                                                           4u * c1 + q, (uint32_t)a.k, c3, a.key0, a.key1);
         acc |= (uint32_t)ok << q;
     }
-    if (acc) {
-        uint32_t flip = 0;
-        int d[4];
+    if (!acc) return false;
+    uint32_t flip = 0;
+    int d[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const bool f = (acc >> q) & 1u;
-            flip |= f ? (0xFEu << (8 * q)) : 0u;
-            dE[q] += f ? 2 * m[q] : 0;
-            d[q] = f ? -2 * x[q] : 0;
-        }
-        Ssm[widx] = sw ^ flip;
-        nacc += __popc(acc & vmask);
-        uint32_t D0, D1 = 0;
-        if (FB == 16) {
-            D0 = (uint32_t)(d[0] + d[1] * 65536);
-            D1 = (uint32_t)(d[2] + d[3] * 65536);
-        } else {
-            D0 = (uint32_t)(d[0] + d[1] * 256 + d[2] * 65536 + d[3] * 16777216);
-        }
-        const uint32_t e0 = __ldg(&a.g.rp[p]), e1 = __ldg(&a.g.rp[p + 1]);
-        for (uint32_t e = e0; e < e1; ++e) {
-            const int j = __ldg(&a.g.col[e]);
-            uint32_t s0 = D0, s1 = D1;
-            if (WEIGHTED) {
-                if (__ldg(&a.g.wt[e]) < 0) {
-                    s0 = 0u - D0;
-                    s1 = 0u - D1;
-                }
-            }
-            if (FB == 16) {
-                atomicAdd(&Hsm[2 * (j * G + g)], s0);
-                atomicAdd(&Hsm[2 * (j * G + g) + 1], s1);
-            } else {
-                atomicAdd(&Hsm[j * G + g], s0);
-            }
-        }
+    for (int q = 0; q < 4; ++q) {
+        const bool f = (acc >> q) & 1u;
+        flip |= f ? (0xFEu << (8 * q)) : 0u;
+        dE[q] += f ? 2 * m[q] : 0;
+        d[q] = f ? -2 * x[q] : 0;
     }
+    Ssm[widx] = sw ^ flip;
+    nacc += __popc(acc & vmask);
+    if (FB == 16) {
+        D0 = (uint32_t)(d[0] + d[1] * 65536);
+        D1 = (uint32_t)(d[2] + d[3] * 65536);
+    } else {
+        D0 = (uint32_t)(d[0] + d[1] * 256 + d[2] * 65536 + d[3] * 16777216);
+    }
+    return true;
 }
 
 template <int G, int FB, bool WEIGHTED>
@@ -160,11 +188,15 @@ __global__ void __launch_bounds__(1024) k_sweep(const SweepArgs a) {
     int32_t *Eacc = cls + csz;          // [4G]
     int32_t *PS = Eacc + 4 * G;         // [4G] parent slot of each replica
     int32_t *misc = PS + 4 * G;         // best E, step, sweep, slot, copy-from (q+1), changed
+    SweepQueue Q{reinterpret_cast<uint4 *>(misc + 8), nullptr, 0};
+    Q.count = reinterpret_cast<int32_t *>(Q.ent + 2 * blockDim.x);
+    const bool queued = a.qcap != 0;   // room for the queue
 
     const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31;
     const uint32_t *tab = a.tables + (size_t)a.tidx[a.k] * (a.g.mmax + 1);
     for (int i = tid; i <= a.g.mmax; i += NT) Tt[i] = tab[i];
     for (int i = tid; i <= a.g.ncol; i += NT) cls[i] = a.g.cls[i];
+    if (queued && tid < 3) Q.count[tid] = 0;
     const int gthr = tid % G;   // NT is a multiple of 32, so each thread keeps one group
 
     for (int blk = blockIdx.x; blk < a.nblk; blk += gridDim.x) {
@@ -220,15 +252,56 @@ __global__ void __launch_bounds__(1024) k_sweep(const SweepArgs a) {
         for (int q = 0; q < 4; ++q) vmask |= (slot0 + 4 * gthr + q < a.R) ? (1u << q) : 0u;
         const uint32_t c1 = (uint32_t)(blk * G + gthr);
         uint32_t nacc = 0;
+        // The uniforms of a thread's first item of the next class are drawn while
+        // the present class is finished (they depend on no spin).
+        uint32_t vid = 0, uw = 0;
+        auto draw = [&](int p, uint32_t c3) {
+            vid = __ldg(&a.g.vid[p]);
+            uw = group_uniforms(a, vid, c1, c3);
+        };
+        if (nsweeps && tid < cls[1] * G) draw(tid / G, TAG_SWEEP);
         for (int s = 0; s < nsweeps; ++s) {
             const uint32_t c3 = TAG_SWEEP | (uint32_t)s;
             int dE[4] = {0, 0, 0, 0};
             for (int c = 0; c < a.g.ncol; ++c) {
-                const int p0 = cls[c];
-                const int cnt = (cls[c + 1] - p0) * G;
-                for (int idx = tid; idx < cnt; idx += NT)
-                    sweep_item<G, FB, WEIGHTED>(Ssm, Hsm, Tt, a, p0 + idx / G, gthr, c1, c3, vmask,
-                                                dE, nacc);
+                const int p0 = cls[c], cnt = (cls[c + 1] - p0) * G;
+                for (int base = 0; base < cnt; base += NT) {   // uniform over the block
+                    const int idx = base + tid;
+                    bool have = false;
+                    uint4 ent = make_uint4(0u, 0u, 0u, 0u);
+                    if (idx < cnt) {
+                        const int p = p0 + idx / G;
+                        if (base) draw(p, c3);
+                        have = sweep_item<G, FB>(Ssm, Hsm, Tt, a, p, gthr, vid, uw, c1, c3, vmask, dE, nacc, ent.y, ent.z);
+                        ent.x = (uint32_t)p | (uint32_t)gthr << 16;
+                    }
+                    auto walk = [&](const uint4 &e, int sub, int lanes) {
+                        const uint32_t pe = e.x & 0xFFFFu, ge = e.x >> 16;
+                        const uint32_t e1 = __ldg(&a.g.rp[pe + 1]);
+                        for (uint32_t i = __ldg(&a.g.rp[pe]) + sub; i < e1; i += lanes) {
+                            const int j = __ldg(&a.g.col[i]);
+                            uint32_t s0 = e.y, s1 = e.z;
+                            if (WEIGHTED && __ldg(&a.g.wt[i]) < 0) {
+                                s0 = 0u - s0;
+                                s1 = 0u - s1;
+                            }
+                            if (FB == 16) {
+                                atomicAdd(&Hsm[2 * (j * G + ge)], s0);
+                                atomicAdd(&Hsm[2 * (j * G + ge) + 1], s1);
+                            } else {
+                                atomicAdd(&Hsm[j * G + ge], s0);
+                            }
+                        }
+                    };
+                    if (queued) Q.push(have, ent, lane);
+                    else if (have) walk(ent, 0, 1);
+                    if (base + NT >= cnt) {
+                        const int cn = c + 1 < a.g.ncol ? c + 1 : 0;
+                        if (tid < (cls[cn + 1] - cls[cn]) * G)
+                            draw(cls[cn] + tid / G, TAG_SWEEP | (uint32_t)(cn ? s : s + 1));
+                    }
+                    if (queued) Q.drain(walk);
+                }
                 __syncthreads();
             }
             // Energies after sweep s: reduce the per-thread changes of each replica.
@@ -344,14 +417,12 @@ __device__ __forceinline__ uint32_t pk_settle_ties(const SweepArgs &a, uint32_t 
 
 __device__ __forceinline__ void pk_decide(const uint32_t *__restrict__ Bsm, const uint32_t *__restrict__ T256,
                                           const uint32_t *__restrict__ Psm, const SweepArgs &a, int p,
-                                          uint32_t c1, uint32_t c3, PkItem &it) {
-    const uint32_t vid = __ldg(&a.g.vid[p]);
+                                          uint32_t vid, uint32_t uw, uint32_t c1, uint32_t c3, PkItem &it) {
     const uint32_t b = Bsm[p];
     const uint32_t par = (Psm[p >> 5] >> (p & 31)) & 1u;
     const uint32_t smask = b & 0x01010101u;
     const uint32_t hb = (b & 0xFEFEFEFEu) | (par * 0x01010101u);
     const uint32_t mb = (hb ^ (smask * 0xFFu)) + smask;
-    const uint32_t uw = word_of(philox10(make_uint4(vid, c1 >> 2, (uint32_t)a.k, c3), a.key0, a.key1), c1 & 3u);
     // The four decisions in 16-bit lanes (pk_entry).
     const uint32_t e0 = T256[mb & 0xFFu], e1 = T256[(mb >> 8) & 0xFFu];
     const uint32_t e2 = T256[(mb >> 16) & 0xFFu], e3 = T256[mb >> 24];
@@ -398,6 +469,19 @@ __device__ __forceinline__ void pk_enqueue(uint2 *__restrict__ Q, uint32_t &qtai
     qtail += __popc(bal);
 }
 
+// Adds D to the fields of the four neighbours of one row unit.
+template <bool WEIGHTED>
+__device__ __forceinline__ void pk_add4(uint32_t *__restrict__ Bsm, const uint2 &v, uint32_t D) {
+    const uint32_t idx[4] = {v.x & 0xFFFFu, v.x >> 16, v.y & 0xFFFFu, v.y >> 16};
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        if (WEIGHTED)
+            atomicAdd(&Bsm[idx[t] & 0x7FFFu], (idx[t] & 0x8000u) ? 0u - D : D);
+        else
+            atomicAdd(&Bsm[idx[t]], D);
+    }
+}
+
 template <bool WEIGHTED>
 __device__ __forceinline__ void pk_round(uint32_t *__restrict__ Bsm, const uint2 *__restrict__ Q,
                                          uint32_t qhead, uint32_t count, const SweepArgs &a, int lane) {
@@ -406,17 +490,7 @@ __device__ __forceinline__ void pk_round(uint32_t *__restrict__ Bsm, const uint2
         const uint2 ent = Q[(qhead + lane) & (PK_QCAP - 1)];
         const uint32_t D = ent.y;
         const uint32_t e0 = __ldg(&a.g.prp[ent.x]), e1 = __ldg(&a.g.prp[ent.x + 1]);
-        for (uint32_t e = e0; e < e1; ++e) {
-            const uint2 v = __ldg(&a.g.pcol[e]);
-            const uint32_t idx[4] = {v.x & 0xFFFFu, v.x >> 16, v.y & 0xFFFFu, v.y >> 16};
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                if (WEIGHTED)
-                    atomicAdd(&Bsm[idx[t] & 0x7FFFu], (idx[t] & 0x8000u) ? 0u - D : D);
-                else
-                    atomicAdd(&Bsm[idx[t]], D);
-            }
-        }
+        for (uint32_t e = e0; e < e1; ++e) pk_add4<WEIGHTED>(Bsm, __ldg(&a.g.pcol[e]), D);
     }
     __syncwarp();
 }
@@ -436,7 +510,7 @@ __global__ void __launch_bounds__(NTB, MINB) k_sweep_packed(const SweepArgs a) {
     int32_t *misc = PS + 4;         // best E, step, sweep, slot, copy-from (q+1), changed
     uint32_t *Psm = reinterpret_cast<uint32_t *>(misc + 8);         // degree parity bits
     const int npw = (np + 31) >> 5;
-    uint2 *Qall = reinterpret_cast<uint2 *>(Psm + ((npw + 1) & ~1));  // [NT/32][PK_QCAP]
+    uint2 *Qall = reinterpret_cast<uint2 *>(Psm + ((npw + 3) & ~3));  // [NT/32][PK_QCAP]
 
     const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31;
     uint2 *Q = Qall + (size_t)(tid >> 5) * PK_QCAP;
@@ -498,8 +572,14 @@ __global__ void __launch_bounds__(NTB, MINB) k_sweep_packed(const SweepArgs a) {
                     PkItem A, Bi;
                     A.acc = 0;
                     Bi.acc = 0;
-                    if (pA < p1) pk_decide(Bsm, T256, Psm, a, pA, c1, c3, A);
-                    if (pB < p1) pk_decide(Bsm, T256, Psm, a, pB, c1, c3, Bi);
+                    if (pA < p1) {
+                        const uint32_t vA = __ldg(&a.g.vid[pA]);
+                        pk_decide(Bsm, T256, Psm, a, pA, vA, group_uniforms(a, vA, c1, c3), c1, c3, A);
+                    }
+                    if (pB < p1) {
+                        const uint32_t vB = __ldg(&a.g.vid[pB]);
+                        pk_decide(Bsm, T256, Psm, a, pB, vB, group_uniforms(a, vB, c1, c3), c1, c3, Bi);
+                    }
                     const uint32_t DA = pk_commit_self(Bsm, pA, A, vmask, dE, nacc);
                     const uint32_t DB = pk_commit_self(Bsm, pB, Bi, vmask, dE, nacc);
                     pk_enqueue(Q, qtail, pA, DA, lane);
@@ -570,6 +650,301 @@ __global__ void __launch_bounds__(NTB, MINB) k_sweep_packed(const SweepArgs a) {
                     sp[q] |= sv << (8 * j);
                     if (j < 2) fx[q] |= ((uint32_t)h & 0xFFFFu) << (16 * j);
                     else fy[q] |= ((uint32_t)h & 0xFFFFu) << (16 * (j - 2));
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const size_t row = (size_t)(slot0 + q) * np + 4 * c;
+                *reinterpret_cast<uint32_t *>(a.spins_out + row) = sp[q];
+                *reinterpret_cast<uint2 *>(a.fields_out + row) = make_uint2(fx[q], fy[q]);
+            }
+        }
+        if (tid < 4) a.E_out[slot0 + tid] = Eacc[tid];
+        if (tid == 0 && misc[5]) a.best_rec[blk] = make_int4(misc[0], misc[1], misc[2], misc[3]);
+        const uint32_t wsum = __reduce_add_sync(0xFFFFFFFFu, nacc);
+        if (act && lane == 0 && wsum) atomicAdd(&a.accepts[a.k], (unsigned long long)wsum);
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Small graphs in the layouts that keep fields (packed byte, FB = 7, or int8
+// spins with int16 fields, FB = 16): every colour class fits one round of the
+// block. With a few positions per class nothing is left but the latency of the
+// class's chain, and this kernel takes out of it what does not depend on spins:
+//   - all uniforms of a sweep are drawn before it (both Philox calls, so the
+//     full 32-bit uniform: no tie path), 16 bytes per position;
+//   - half of the warps decide (one lane per replica), the other half walk the
+//     rows (a power of two of lanes per position, fixed by the class size, no
+//     queue), and each half reads what it needs for its next turn while the
+//     other one works.
+// What stays per class: decide, barrier, field updates, barrier.
+// Bound: that latency, and shared-memory atomics with many neighbours. Measured
+// on GB300, us per step of 4 sweeps, general kernel / this one: n = 800, mean
+// degree 48 (packed): R = 256 100 / 50, R = 2048 98 / 80, R = 3000 106 / 90,
+// R = 4096 117 / 141; n = 96, degree 14, R = 24 35 / 24; n = 500, degree 250
+// (int16, the general kernel with its queue and 128 threads): R = 1024 388 / 149,
+// R = 4096 404 / 314, R = 8192 780 / 553. So it runs up to 5 (packed) or 16
+// (int16) blocks per SM, with half the threads from 3 on.
+// NH: deciding and walking threads, each.
+constexpr int SMALL_MAX_HALF = 256;
+constexpr int SMALL_UNITS = 3;   // row units a thread reads ahead
+
+template <int FB>
+__host__ __device__ inline size_t small_smem_words(int np, int ncol, int mmax, int half) {
+    // uniforms, words of the layout, field changes, row starts, thresholds, class bounds, records, parities
+    return 4 * (size_t)np + (FB == 7 ? (size_t)(np + 32) : 3 * (size_t)np + 64) + 2 * (size_t)half + (size_t)np + 4 +
+           (size_t)((mmax + 4) & ~3) + (size_t)((ncol + 4) & ~3) + 16 + (FB == 7 ? (size_t)((np + 127) >> 7) * 4 : 0);
+}
+
+template <int FB, bool WEIGHTED, int NH>
+__global__ void __launch_bounds__(2 * NH) k_sweep_small(const SweepArgs a) {
+    constexpr int NT = 2 * NH;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const bool act = !a.active || a.active[a.k];
+    const int nsweeps = act ? a.S : 0;
+    const int np = a.g.np, n = a.g.n, ncol = a.g.ncol;
+    uint32_t *U = reinterpret_cast<uint32_t *>(smem);              // [np][4] uniforms of the sweep
+    uint32_t *Bsm = U + 4 * np;                                    // FB 7: [np + 32] bytes; FB 16: [2 (np + 32)] fields
+    uint32_t *Ssm = Bsm + 2 * (np + 32);                           // FB 16: [np] spins
+    uint32_t *Dsm = FB == 7 ? Bsm + np + 32 : Ssm + np;            // [NH][2] field changes of the class
+    uint32_t *rows = Dsm + 2 * NH;                                 // [np + 4] row starts in units
+    uint32_t *T = rows + np + 4;                                   // thresholds by m
+    int32_t *cls = reinterpret_cast<int32_t *>(T + ((a.g.mmax + 4) & ~3));
+    int32_t *Eacc = cls + ((ncol + 4) & ~3);   // [4]
+    int32_t *PS = Eacc + 4;                    // [4]
+    int32_t *misc = PS + 4;                    // best E, step, sweep, slot, copy-from (q+1), changed
+    uint32_t *Psm = reinterpret_cast<uint32_t *>(misc + 8);        // FB 7: degree parity bits
+    const int tid = threadIdx.x, lane = tid & 31, ht = tid & (NH - 1);   // ht: thread of its half
+    const bool decides = tid < NH;
+    const uint32_t *tab = a.tables + (size_t)a.tidx[a.k] * (a.g.mmax + 1);
+    for (int i = tid; i <= a.g.mmax; i += NT) T[i] = tab[i];
+    for (int i = tid; i <= n; i += NT) rows[i] = a.g.prp[i];
+    if (FB == 7)
+        for (int i = tid; i < (np + 31) >> 5; i += NT) Psm[i] = a.g.parity[i];
+    for (int i = tid; i <= ncol; i += NT) cls[i] = a.g.cls[i];
+
+    for (int blk = blockIdx.x; blk < a.nblk; blk += gridDim.x) {
+        const int slot0 = blk * 4;
+        if (tid < 4) PS[tid] = act ? a.parent[slot0 + tid] : slot0 + tid;
+        if (tid == 0) {
+            const int4 br = a.best_rec[blk];
+            misc[0] = br.x; misc[1] = br.y; misc[2] = br.z; misc[3] = br.w;
+            misc[4] = 0; misc[5] = 0;
+        }
+        __syncthreads();
+        if (tid < 4) Eacc[tid] = a.E_in[PS[tid]];
+        for (int c = tid; c < (np >> 2); c += NT) {
+            uint32_t w[4];
+            uint2 f[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const size_t row = (size_t)PS[q] * np + 4 * c;
+                w[q] = __ldg(reinterpret_cast<const uint32_t *>(a.spins_in + row));
+                f[q] = __ldg(reinterpret_cast<const uint2 *>(a.fields_in + row));
+            }
+            uint32_t o[4];
+            transpose4x4_bytes(w[0], w[1], w[2], w[3], o);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                uint32_t h[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) h[q] = ((j < 2 ? f[q].x : f[q].y) >> (16 * (j & 1))) & 0xFFFFu;
+                if (FB == 7) {
+                    uint32_t word = 0;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        word |= (((h[q] + 128u) & 0xFEu) | (((o[j] >> (8 * q)) & 0xFFu) == 1u ? 1u : 0u)) << (8 * q);
+                    Bsm[4 * c + j] = word;
+                } else {
+                    Ssm[4 * c + j] = o[j];
+                    Bsm[2 * (4 * c + j)] = (h[0] | h[1] << 16) ^ 0x80008000u;
+                    Bsm[2 * (4 * c + j) + 1] = (h[2] | h[3] << 16) ^ 0x80008000u;
+                }
+            }
+        }
+        __syncthreads();
+        const int q = tid & 3;   // the thread's replica
+        const uint32_t live = slot0 + q < a.R ? 1u : 0u;
+        const uint32_t c1 = (uint32_t)blk;
+        uint32_t nacc = 0;
+        // A walking thread's share of the class's rows: item, its first units and
+        // where the rest would be.
+        int li = 0;
+        uint32_t nu = 0, enext = 0, lanes = 1;
+        uint2 un[SMALL_UNITS];
+        auto ahead = [&](int c) {
+            const int p0 = cls[c], P = cls[c + 1] - p0;
+            const int lt = P > 1 ? __clz(P - 1) - __clz(NH - 1) : 32 - __clz(NH - 1);   // log2(NH) less that of P rounded up
+            li = ht >> lt;
+            lanes = 1u << lt;
+            nu = 0;
+            if (li >= P) return;
+            const uint32_t e0 = rows[p0 + li] + (ht & (lanes - 1u)), e1 = rows[p0 + li + 1];
+            nu = e0 < e1 ? (e1 - e0 + lanes - 1u) >> lt : 0u;
+            enext = e0 + SMALL_UNITS * lanes;
+#pragma unroll
+            for (int i = 0; i < SMALL_UNITS; ++i)
+                if ((uint32_t)i < nu) un[i] = __ldg(&a.g.pcol[e0 + i * lanes]);
+        };
+        auto add4 = [&](const uint2 &v, const uint2 &D) {
+            const uint32_t idx[4] = {v.x & 0xFFFFu, v.x >> 16, v.y & 0xFFFFu, v.y >> 16};
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const bool neg = WEIGHTED && (idx[t] & 0x8000u);
+                const uint32_t j = idx[t] & 0x7FFFu;
+                if (FB == 7) {
+                    atomicAdd(&Bsm[j], neg ? 0u - D.x : D.x);
+                } else {
+                    atomicAdd(&Bsm[2 * j], neg ? 0u - D.x : D.x);
+                    atomicAdd(&Bsm[2 * j + 1], neg ? 0u - D.y : D.y);
+                }
+            }
+        };
+        auto draw = [&](int s) {   // top bytes and tail bits of the four uniforms of every position
+            const uint32_t c3 = TAG_SWEEP | (uint32_t)s;
+            for (int p = tid; p < n; p += NT) {
+                const uint32_t vid = __ldg(&a.g.vid[p]);
+                const uint4 top = philox10(make_uint4(vid, c1 >> 2, (uint32_t)a.k, c3), a.key0, a.key1);
+                const uint4 tl = philox10(make_uint4(vid, c1, (uint32_t)a.k, TAG_TAIL | (uint32_t)s), a.key0, a.key1);
+                const uint32_t uw = word_of(top, c1 & 3u);
+                *reinterpret_cast<uint4 *>(U + 4 * p) =
+                    make_uint4(uw << 24 | tl.x >> 8, (uw >> 8) << 24 | tl.y >> 8, (uw >> 16) << 24 | tl.z >> 8,
+                               (uw >> 24) << 24 | tl.w >> 8);
+            }
+        };
+        // A deciding thread's first attempt of the next class: all but the spin
+        // and the field.
+        int idx = 0, cnt = 0;   // 4 position + replica, attempts of the class
+        uint32_t u = 0, par = 0;
+        auto load = [&](int i) {
+            u = U[i];
+            if (FB == 7) par = (Psm[i >> 7] >> ((i >> 2) & 31)) & 1u;
+        };
+        auto first = [&](int c) {
+            idx = 4 * cls[c] + ht;
+            cnt = 4 * (cls[c + 1] - cls[c]);
+            if (ht < cnt) load(idx);
+        };
+        int dE = 0;
+        if (nsweeps) {
+            draw(0);
+            __syncthreads();
+            if (decides) first(0);
+        }
+        for (int s = 0; s < nsweeps; ++s) {
+            for (int c = 0; c < ncol; ++c) {
+                if (decides) {
+                    for (int base = 0; base < cnt; base += NH) {   // uniform over the deciding half
+                        const int i = idx + base, it = (base + ht) >> 2;
+                        int d = 0;   // change of the neighbours' fields: -2 x if the replica flips
+                        if (base + ht < cnt) {
+                            if (base) load(i);
+                            int h;
+                            unsigned char *byte;
+                            uint32_t up;   // x = +1
+                            if (FB == 7) {
+                                byte = reinterpret_cast<unsigned char *>(Bsm) + i;
+                                const uint32_t b = *byte;
+                                up = b & 1u;
+                                h = (int)((b & 0xFEu) | par) - 128;
+                            } else {
+                                byte = reinterpret_cast<unsigned char *>(Ssm) + i;
+                                h = (int)reinterpret_cast<const uint16_t *>(Bsm)[i] - 32768;
+                                up = *byte == 1u;
+                            }
+                            const int m = up ? -h : h;   // dE = -2 x h = 2m
+                            if (m <= 0 || u < T[min(m, a.g.mmax)]) {
+                                *byte ^= FB == 7 ? 1u : 0xFEu;
+                                d = up ? -2 : 2;
+                                dE += 2 * m;
+                                nacc += live;
+                            }
+                        }
+                        if (FB == 7) {
+                            int v = d * (1 << (8 * q));
+                            v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
+                            v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
+                            if (q == 0) Dsm[2 * it] = (uint32_t)v;
+                        } else {
+                            int v = d * (1 << (16 * (q & 1)));
+                            v += __shfl_xor_sync(0xFFFFFFFFu, v, 1);
+                            if ((q & 1) == 0) Dsm[2 * it + (q >> 1)] = (uint32_t)v;
+                        }
+                    }
+                } else {
+                    ahead(c);
+                }
+                __syncthreads();
+                if (decides) {
+                    if (c + 1 < ncol) {
+                        first(c + 1);
+                    } else {   // the energies after the sweep
+#pragma unroll
+                        for (int off = 4; off < 32; off <<= 1) dE += __shfl_xor_sync(0xFFFFFFFFu, dE, off);
+                        if (lane < 4 && dE != 0) atomicAdd(&Eacc[lane], dE);
+                        dE = 0;
+                    }
+                } else if (nu) {
+                    const uint2 D = make_uint2(Dsm[2 * li], FB == 7 ? 0u : Dsm[2 * li + 1]);
+                    if (D.x | D.y) {
+#pragma unroll
+                        for (int i = 0; i < SMALL_UNITS; ++i)
+                            if ((uint32_t)i < nu) add4(un[i], D);
+                        for (uint32_t i = SMALL_UNITS, e = enext; i < nu; ++i, e += lanes) add4(__ldg(&a.g.pcol[e]), D);
+                    }
+                }
+                __syncthreads();
+            }
+            if (tid < 32) {   // lowest energy of the sweep, the lowest slot first
+                const int v = lane < 4 && slot0 + lane < a.R ? Eacc[lane] : 0x7FFFFFFF;
+                const int bE = __reduce_min_sync(0xFFFFFFFFu, v);
+                const int bq = __ffs(__ballot_sync(0xFFFFFFFFu, v == bE)) - 1;
+                if (lane == 0) {
+                    misc[4] = 0;
+                    if (slot0 < a.R) atomicMin(&a.sweep_emin[(size_t)a.k * a.S + s], bE);
+                    if (slot0 < a.R && bE < misc[0]) {
+                        misc[0] = bE; misc[1] = a.k; misc[2] = s; misc[3] = slot0 + bq;
+                        misc[4] = bq + 1; misc[5] = 1;
+                    }
+                }
+            }
+            if (s + 1 < nsweeps) draw(s + 1);
+            __syncthreads();
+            if (misc[4]) {   // block-uniform: copy the new best configuration
+                const int sh = 8 * (misc[4] - 1);
+                for (int c = tid; c < np; c += NT) {
+                    const uint32_t w = FB == 7 ? Bsm[c] >> sh : Ssm[c] >> sh;
+                    a.best_cfg[(size_t)blk * np + c] =
+                        (int8_t)(FB == 16 ? (w & 0xFFu) : c < n ? ((w & 1u) ? 0x01u : 0xFFu) : 0u);
+                }
+                __syncthreads();   // before the next sweep changes the words
+            }
+            if (decides) first(0);
+        }
+        // Store to the next population buffers.
+        for (int c = tid; c < (np >> 2); c += NT) {
+            uint32_t sp[4] = {0u, 0u, 0u, 0u}, fx[4] = {0u, 0u, 0u, 0u}, fy[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int p = 4 * c + j;
+                const bool real = p < n;
+                const uint32_t word = FB == 7 ? Bsm[p] : Ssm[p];
+                const uint32_t pb = FB == 7 ? (Psm[p >> 5] >> (p & 31)) & 1u : 0u;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t byte = (word >> (8 * q)) & 0xFFu;
+                    uint32_t h, sv;
+                    if (FB == 7) {
+                        sv = real ? ((byte & 1u) ? 0x01u : 0xFFu) : 0u;
+                        h = real ? (uint32_t)((int)((byte & 0xFEu) | pb) - 128) & 0xFFFFu : 0u;
+                    } else {
+                        sv = byte;
+                        h = ((Bsm[2 * p + (q >> 1)] ^ 0x80008000u) >> (16 * (q & 1))) & 0xFFFFu;
+                    }
+                    sp[q] |= sv << (8 * j);
+                    if (j < 2) fx[q] |= h << (16 * j);
+                    else fy[q] |= h << (16 * (j - 2));
                 }
             }
 #pragma unroll
@@ -1326,6 +1701,12 @@ void *msc_kernel(int mmax, bool cluster) {
     return cluster ? msc_kernel<W, BIG, true>(mmax) : msc_kernel<W, BIG, false>(mmax);
 }
 
+template <int FB, bool W>
+void *small_kernel(int threads) {
+    return threads == 512 ? reinterpret_cast<void *>(&k_sweep_small<FB, W, 256>)
+                          : reinterpret_cast<void *>(&k_sweep_small<FB, W, 128>);
+}
+
 template <bool W>
 void *packed_kernel(int threads) {
     switch (threads) {
@@ -1344,10 +1725,14 @@ void *kernel_ptr() {
     return reinterpret_cast<void *>(&k_sweep<G, FB, W>);
 }
 
-void *select_kernel(int G, int fb, bool weighted, int threads, int mmax, bool big) {
+void *select_kernel(int G, int fb, bool weighted, int threads, int mmax, bool big, bool small) {
     if (fb == 1 || fb == 2) {
         if (big) return weighted ? msc_kernel<true, true>(mmax, fb == 2) : msc_kernel<false, true>(mmax, fb == 2);
         return weighted ? msc_kernel<true, false>(mmax, fb == 2) : msc_kernel<false, false>(mmax, fb == 2);
+    }
+    if (small) {
+        if (fb == 7) return weighted ? small_kernel<7, true>(threads) : small_kernel<7, false>(threads);
+        return weighted ? small_kernel<16, true>(threads) : small_kernel<16, false>(threads);
     }
     if (fb == 7) return weighted ? packed_kernel<true>(threads) : packed_kernel<false>(threads);
     if (G == 1) {
@@ -1365,7 +1750,7 @@ size_t sweep_smem_bytes(const GraphDev &g, int G, int field_bits, int threads) {
         return ((size_t)g.np + msc_reserved_words(g.mmax) + ((g.ncol + 1 + 3) & ~3)) * 4;
     if (field_bits == 7)
         return (size_t)(g.np + 32) * 4 + 256 * 4 + (size_t)((g.ncol + 1 + 3) & ~3) * 4 + 16 * 4 +
-               (size_t)((((g.np + 31) / 32) + 1) & ~1) * 4 + (size_t)(threads / 32) * PK_QCAP * 8;
+               (size_t)((((g.np + 31) / 32) + 3) & ~3) * 4 + (size_t)(threads / 32) * PK_QCAP * 8;
     const int HW = field_bits == 16 ? 2 : 1;
     return (size_t)g.np * G * 4 * (1 + HW) + (size_t)((g.mmax + 1 + 3) & ~3) * 4 +
            (size_t)((g.ncol + 1 + 3) & ~3) * 4 + (size_t)(8 * G + 8) * 4;
@@ -1373,21 +1758,37 @@ size_t sweep_smem_bytes(const GraphDev &g, int G, int field_bits, int threads) {
 
 cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int threads,
                             bool weighted, SweepConfig *cfg) {
-    if (field_bits == 1 || field_bits == 2) {
+    int dev = 0, sms = 0, occ = 0, limit = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    const bool msc = field_bits == 1 || field_bits == 2, automatic = threads == 0;
+    bool small = false;
+    if (msc) {
         G = 8;
         threads = 256;
     } else if (field_bits == 7) {
         G = 1;
+        // Few blocks: more threads each, so that an SM has about 1024 whatever the
+        // number of blocks (G63-shaped, us per step of 4 sweeps with 128 / 256 /
+        // 512 / 1024 threads: 128 blocks 214 / 137 / 107 / 98, 256 blocks 214 /
+        // 151 / 142 / 188, 475 blocks 269 / 230 / 274 / 363, 1024 blocks 376 / 448
+        // / 456 / 632), and no more than the largest class can use.
+        if (automatic) {
+            const int per = ((R + 3) / 4 + sms - 1) / sms;
+            threads = per <= 1 ? 1024 : per == 2 ? 512 : per <= 4 ? 256 : 128;
+            while (threads > 128 && threads / 2 >= g.maxcls) threads /= 2;
+        }
+    } else if (automatic) {   // as above; n = 500, degree 250, R = 4096: 404 us with 128 threads, 1375 with 512
+        const int per = ((R + 4 * G - 1) / (4 * G) + sms - 1) / sms;
+        threads = per <= 2 ? 512 : per <= 4 ? 256 : 128;
     }
     size_t smem = sweep_smem_bytes(g, G, field_bits, threads);
     if (field_bits == 1 || field_bits == 2) {
         // Tie queues: 64 entries per warp, 40 where 64 would cost a resident
         // block, and what the reserved words leave when the graph fills shared
         // memory.
-        int dev = 0, limit = 0, per_sm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
         const size_t fixed = ((size_t)g.np + msc_table_words(g.mmax) + 72 + ((g.ncol + 1 + 3) & ~3)) * 4;
         const size_t per_entry = (size_t)(threads / 32) * msc_entry_words(g.mmax) * 4;
         auto resident = [&](int cap) { return std::min<size_t>(4, (size_t)per_sm / (fixed + cap * per_entry + 1024)); };
@@ -1396,7 +1797,28 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
         if (cfg->qcap < 1) return cudaErrorInvalidConfiguration;
         smem = fixed + cfg->qcap * per_entry;
     }
-    void *fn = select_kernel(G, field_bits, weighted, threads, g.mmax, g.mbig != 0);
+    cfg->small = false;
+    if (!msc) {
+        cfg->qcap = 0;
+        // Every class within one round of the block, and blocks few enough: the
+        // small-graph kernel.
+        const int per = ((R + 3) / 4 + sms - 1) / sms, half = per <= 2 ? 256 : 128;
+        const size_t need = 4 * (field_bits == 7 ? small_smem_words<7>(g.np, g.ncol, g.mmax, half)
+                                                 : small_smem_words<16>(g.np, g.ncol, g.mmax, half));
+        small = automatic && G == 1 && field_bits != 8 && g.packed_ok && per <= (field_bits == 7 ? 5 : 16) && g.maxcls <= half &&
+                std::min(per, 2) * (need + 1024) <= (size_t)per_sm;
+        if (small) {
+            cfg->small = true;
+            threads = 2 * half;
+            smem = need;
+        } else if (field_bits != 7 && smem + sweep_queue_bytes(threads) <= (size_t)limit) {
+            // int8/int16: the block's queue of accepted items, where shared memory
+            // has room for it (without it each thread walks its own rows).
+            smem += sweep_queue_bytes(threads);
+            cfg->qcap = threads;
+        }
+    }
+    void *fn = select_kernel(G, field_bits, weighted, threads, g.mmax, g.mbig != 0, small);
     // The attribute belongs to the kernel function, not to a context: only ever
     // raise it, so that contexts configured earlier keep launching.
     {
@@ -1410,9 +1832,6 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
             cur = smem;
         }
     }
-    int dev = 0, sms = 0, occ = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int nblk = (R + 4 * G - 1) / (4 * G);
     if (field_bits == 2) {
         // One cluster of two CTAs per word; the hardware schedules them as slots free up.
@@ -1449,7 +1868,7 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
 }
 
 cudaError_t launch_sweep(const SweepConfig &cfg, const SweepArgs &a, cudaStream_t st) {
-    void *fn = select_kernel(cfg.G, cfg.field_bits, a.g.wt != nullptr, cfg.threads, a.g.mmax, a.g.mbig != 0);
+    void *fn = select_kernel(cfg.G, cfg.field_bits, a.g.wt != nullptr, cfg.threads, a.g.mmax, a.g.mbig != 0, cfg.small);
     SweepArgs b = a;
     b.qcap = cfg.qcap;
     void *args[] = {&b};

@@ -141,7 +141,7 @@ struct RunState {
 
 struct pa_ctx {
     int device = 0;
-    int32_t n = 0, np = 0, m2 = 0, maxdeg = 0, ncol = 0;
+    int32_t n = 0, np = 0, m2 = 0, maxdeg = 0, ncol = 0, maxcls = 0;
     int64_t W = 0;
     bool weighted = false;
     uint64_t graph_hash = 0;
@@ -163,6 +163,7 @@ struct pa_ctx {
         g.np = np;
         g.ncol = ncol;
         g.mmax = maxdeg;
+        g.maxcls = maxcls;
         g.rp = d_rp.as<uint32_t>();
         g.col = d_col.as<uint16_t>();
         g.wt = weighted ? d_w.as<int8_t>() : nullptr;
@@ -417,6 +418,7 @@ int pa_create(pa_ctx **out, int32_t n, const uint32_t *row_ptr, const uint16_t *
     // gives the 32 lanes of a warp neighbour loops of nearly equal length.
     c->cls.assign(ncol + 1, 0);
     for (int32_t i = 0; i < n; ++i) c->cls[c->colour[i] + 1]++;
+    for (int32_t k = 0; k < ncol; ++k) c->maxcls = std::max(c->maxcls, c->cls[k + 1]);
     for (int32_t k = 0; k < ncol; ++k) c->cls[k + 1] += c->cls[k];
     c->pos.assign(n, 0);
     c->vid.assign(n, 0);
@@ -653,7 +655,7 @@ int pa_anneal_begin(pa_ctx *c, const double *betas, int32_t K, int32_t R, int32_
     // Sweep kernel shape.
     const bool msc = o.variant == PA_VARIANT_MSC || o.variant == PA_VARIANT_MSC_PAIR;
     int G = o.replicas_per_cta == 8 ? 2 : 1;
-    int threads = o.threads_per_cta ? o.threads_per_cta : (msc ? 256 : (o.field_bits == 7 ? 128 : 512));
+    const int threads = o.threads_per_cta;   // 0: chosen by sweep_configure
     pa::GraphDev g = c->gdev();
     const int fcode = o.variant == PA_VARIANT_MSC_PAIR ? 2 : (msc ? 1 : o.field_bits);
     cudaError_t ce = pa::sweep_configure(g, R, G, fcode, threads, c->weighted, &r.sweep);

@@ -105,7 +105,7 @@ constexpr int32_t EMIN_SENTINEL = 0x7F7F7F7F;  // byte-fillable "+infinity"
 constexpr int RS_CHUNK = 256;                   // slots per resampling CTA (power of two)
 
 struct GraphDev {
-    int32_t n, np, ncol, mmax;
+    int32_t n, np, ncol, mmax, maxcls;   // maxcls: largest colour class
     const uint32_t *rp;   // [n+1] row pointers, position order
     const uint16_t *col;  // [2M] neighbour positions
     const int8_t *wt;     // [2M] weights or nullptr (all +1)
@@ -150,7 +150,7 @@ struct SweepArgs {
     const int32_t *active;       // [K] 0 = skip the step (adaptive end), may be null
     int32_t R, nblk, S, k;       // nblk: replica blocks of this launch
     int32_t blk_base;            // first replica block of this launch (multi-spin-coded kernels)
-    int32_t qcap;                // multi-spin coded: tie-queue entries per warp
+    int32_t qcap;                // multi-spin coded: tie-queue entries per warp; other layouts: entries of the block's queue
     uint32_t key0, key1;
     uint32_t rk0[10], rk1[10];   // Philox round keys key + r * (0x9E3779B9, 0xBB67AE85)
     int4 *best_rec;              // [all blocks] (E, step, sweep, slot) per replica block
@@ -195,11 +195,13 @@ struct SweepConfig {
     int threads;
     int grid;
     size_t smem;
-    int qcap = 0;   // multi-spin coded: tie-queue entries per warp
+    bool small = false;   // the small-graph kernel of the layout
+    int qcap = 0;   // multi-spin coded: tie-queue entries per warp; other layouts: entries of the block's queue (0: none)
 };
 // Dynamic shared memory of one sweep CTA (G: 4-replica groups of the int8/int16 layouts;
 // field_bits 1/2 multi-spin coded, 7 packed, 8/16 int8/int16 fields).
 size_t sweep_smem_bytes(const GraphDev &g, int G, int field_bits, int threads);
+// threads = 0: chosen here.
 cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int threads,
                             bool weighted, SweepConfig *cfg);
 cudaError_t launch_sweep(const SweepConfig &cfg, const SweepArgs &a, cudaStream_t st);
