@@ -247,11 +247,11 @@ int pa_set_state(pa_ctx *ctx, const int8_t *spins, int32_t steps_done);
 
 /* Energies E = sum over edges w_ij x_i x_j and cuts (W - E)/2 (Eq. 1 and
  * the sign convention of Sec. 2) of R host configurations int8[R][n] (+1/-1,
- * vertex order), evaluated on the device with the kernel that initialises a
- * population. Independent of any anneal: a verifier for configurations read
+ * vertex order), evaluated on the device. Independent of any anneal: a verifier for configurations read
  * back from files (e.g. the hexadecimal format of Sec. 3). energies int32[R]
  * and cuts int64[R] are caller buffers; either may be NULL. R = 0 is a no-op.
- * Allocates R*(3n + 4) bytes of device memory for the call. Errors: PA_EINVAL
+ * Allocates R*(n + 4) bytes of device memory for the call, R*(4n + 4) on graphs
+ * without multi-spin-coded layouts. Errors: PA_EINVAL
  * (spin not +1/-1, R < 0), PA_ENOMEM, PA_ECUDA. */
 int pa_energies(pa_ctx *ctx, const int8_t *spins, int32_t R, int32_t *energies, int64_t *cuts);
 

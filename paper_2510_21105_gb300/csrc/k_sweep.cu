@@ -30,6 +30,22 @@
 namespace pa {
 namespace {
 
+// Allows a kernel `smem` bytes of dynamic shared memory. The attribute belongs
+// to the kernel function, not to a context: only ever raise it, so that
+// contexts configured earlier keep launching.
+cudaError_t raise_smem(void *fn, size_t smem) {
+    static std::mutex mu;
+    static std::unordered_map<void *, size_t> raised;
+    std::lock_guard<std::mutex> lock(mu);
+    size_t &cur = raised[fn];
+    if (smem > cur) {
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        cur = smem;
+    }
+    return cudaSuccess;
+}
+
 __device__ __forceinline__ void transpose4x4_bytes(uint32_t w0, uint32_t w1, uint32_t w2,
                                                    uint32_t w3, uint32_t o[4]) {
     const uint32_t a_lo = __byte_perm(w0, w1, 0x5140);
@@ -1253,9 +1269,9 @@ struct MscSlice {
 };
 
 template <bool BIG>
-__device__ __forceinline__ MscUnit<BIG> msc_unit(const SweepArgs &a, uint32_t off, uint32_t u) {
+__device__ __forceinline__ MscUnit<BIG> msc_unit(const void *mcol, uint32_t off, uint32_t u) {
     constexpr uint32_t bytes = 32u * sizeof(MscUnit<BIG>);
-    return __ldg(reinterpret_cast<const MscUnit<BIG> *>(reinterpret_cast<const char *>(a.g.mcol) + (off + u * bytes)));
+    return __ldg(reinterpret_cast<const MscUnit<BIG> *>(reinterpret_cast<const char *>(mcol) + (off + u * bytes)));
 }
 
 // One (position, word) item: 32 attempts. Returns the mask of accepted
@@ -1270,7 +1286,7 @@ __device__ __forceinline__ uint32_t msc_item(const SweepArgs &a, const uint32_t 
                                              uint32_t (&S)[MscShape<N>::acc_planes], uint32_t &tie,
                                              uint32_t &odd_out) {
     const uint32_t vid = sl.vd & 0xFFFFu, deg = (sl.vd >> 16) & 0x7Fu;
-    const MscUnit<BIG> v0 = msc_unit<BIG>(a, sl.off, 0u), v1 = msc_unit<BIG>(a, sl.off, sl.units > 1u ? 1u : 0u);
+    const MscUnit<BIG> v0 = msc_unit<BIG>(a.g.mcol, sl.off, 0u), v1 = msc_unit<BIG>(a.g.mcol, sl.off, sl.units > 1u ? 1u : 0u);
     // Both Philox calls of the item (slots 32 blk .. +15 and +16 .. +31).
     uint4 u0, u1;
     philox_from_shared2(philox_shared(vid, (uint32_t)a.k, c3, a.key0, a.key1), 2u * blk, 2u * blk + 1u, a.rk0, a.rk1,
@@ -1299,12 +1315,12 @@ __device__ __forceinline__ uint32_t msc_item(const SweepArgs &a, const uint32_t 
             msc_step8x<N>(A, x, w, v);
             uint32_t u = 2;
             for (; u + 2 <= sl.units; u += 2) {
-                msc_unit_words<WEIGHTED>(Wb, msc_unit<BIG>(a, sl.off, u), w);
-                msc_unit_words<WEIGHTED>(Wb, msc_unit<BIG>(a, sl.off, u + 1u), v);
+                msc_unit_words<WEIGHTED>(Wb, msc_unit<BIG>(a.g.mcol, sl.off, u), w);
+                msc_unit_words<WEIGHTED>(Wb, msc_unit<BIG>(a.g.mcol, sl.off, u + 1u), v);
                 msc_step8x<N>(A, x, w, v);
             }
             if (u < sl.units) {
-                msc_unit_words<WEIGHTED>(Wb, msc_unit<BIG>(a, sl.off, u), w);
+                msc_unit_words<WEIGHTED>(Wb, msc_unit<BIG>(a.g.mcol, sl.off, u), w);
                 msc_step4x<N>(A, x, w);
             }
         } else {
@@ -1685,6 +1701,128 @@ __global__ void __launch_bounds__(256, 4) k_sweep_msc(const SweepArgs a) {
     }
 }
 
+// Energies of 32 configurations at a time, one CTA per word, for graphs with
+// slice rows: the configurations become words, the frustrated bonds of every
+// position are counted as in the sweep (7 planes for any degree) and summed in
+// bit-sliced accumulators; E = (stored entries / 2) - sum of the counts. SRC:
+//   WORDS_INIT  spins of the initial population: +1 iff bit 31 of its Philox
+//               word is set; written to the population rows
+//   WORDS_POP   rows of a population (position order, np bytes)
+//   WORDS_RAW   configurations in vertex order (n bytes each, any alignment);
+//               a byte other than +1 / -1 sets *bad
+// Against a byte per neighbour and replica from global memory the rows are read
+// once per 32 replicas. Torus, N = 10000, R = 32768: initial spins, fields and
+// energies took 1320 us, spins and energies alone (the multi-spin-coded layouts
+// read no fields) take 287 us; bound by the Philox calls.
+inline size_t word_energy_smem(const GraphDev &g) { return ((size_t)g.np + 32 + 64) * 4; }
+
+constexpr int WORDS_INIT = 0, WORDS_POP = 1, WORDS_RAW = 2;
+
+template <bool WEIGHTED, bool BIG, int SRC>
+__global__ void __launch_bounds__(256, 3) k_word_energy(GraphDev g, const int8_t *__restrict__ in,
+                                                        const int32_t *__restrict__ pos, int8_t *__restrict__ rows,
+                                                        int32_t *__restrict__ E, int32_t R, uint32_t key0,
+                                                        uint32_t key1, int32_t *__restrict__ bad) {
+    constexpr int N = 7, NT = 256;
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint32_t *Wsm = reinterpret_cast<uint32_t *>(smem);             // [np]
+    int32_t *Eacc = reinterpret_cast<int32_t *>(Wsm + g.np + 32);   // [32]; the 32 words before are read past a class
+    int32_t *PS = Eacc + 32;                                        // [32]
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
+    const int slot0 = (int)blockIdx.x * 32;
+    if (tid < 32) {
+        Eacc[tid] = 0;
+        PS[tid] = min(slot0 + tid, R - 1);
+    }
+    __syncthreads();
+    if (SRC == WORDS_RAW) {
+        bool wrong = false;
+        for (int i = tid; i < g.n; i += NT) {
+            uint32_t w = 0u;
+#pragma unroll 8
+            for (int r = 0; r < 32; ++r) {
+                const int v = __ldg(&in[(size_t)PS[r] * g.n + i]);
+                w |= (uint32_t)(v == 1) << msc_bit(r);
+                wrong |= v != 1 && v != -1;
+            }
+            Wsm[pos[i]] = w;
+        }
+        if (wrong) *bad = 1;
+    } else {
+        for (int c = tid; c < (g.np >> 2); c += NT) {
+            uint32_t w4[4];
+            if (SRC == WORDS_POP) {
+                msc_pack_rows(in, PS, g.np, c, w4);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    w4[j] = 0u;
+                    if (4 * c + j >= g.n) continue;
+                    const uint32_t vid = __ldg(&g.vid[4 * c + j]);
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const uint4 u = philox10(make_uint4(vid, (uint32_t)(slot0 >> 2) + q, 0u, TAG_INIT), key0, key1);
+                        w4[j] |= ((u.x >> 31) | (u.y >> 31) << 8 | (u.z >> 31) << 16 | (u.w >> 31) << 24) << q;
+                    }
+                }
+                msc_unpack_rows(w4, rows, slot0, g.np, g.n, c);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) Wsm[4 * c + j] = w4[j];
+        }
+    }
+    __syncthreads();
+    uint32_t S[MscShape<N>::acc_planes];
+#pragma unroll
+    for (int b = 0; b < MscShape<N>::acc_planes; ++b) S[b] = 0u;
+    int cnt = 0;
+    const unsigned char *Wb = reinterpret_cast<const unsigned char *>(Wsm);
+    const int nsl = g.csl[g.ncol];
+    for (int k = warp; k < nsl; k += NT / 32) {
+        const uint2 d = __ldg(&g.msl[k]);
+        const bool live = !(__ldg(&g.mvd[32 * k + lane]) >> 31);
+        const uint32_t x = Wsm[d.y + (uint32_t)lane], units = d.x >> 24;
+        const uint32_t off = ((d.x & 0xFFFFFFu) * 32u + (uint32_t)lane) * (uint32_t)sizeof(MscUnit<BIG>);
+        uint32_t A[N];
+#pragma unroll
+        for (int b = 0; b < N; ++b) A[b] = x;
+        for (uint32_t u = 0; u < units; ++u) {
+            uint32_t w[4];
+            msc_unit_words<WEIGHTED>(Wb, msc_unit<BIG>(g.mcol, off, u), w);
+            msc_step4x<N>(A, x, w);
+        }
+        uint32_t c = 0u;
+#pragma unroll
+        for (int b = 0; b < N; ++b) c = msc_fa(S[b], live ? A[b] ^ x : 0u, c);
+#pragma unroll
+        for (int b = N; b < MscShape<N>::acc_planes; ++b) c = msc_fa(S[b], c, 0u);
+        if (++cnt == MscShape<N>::flush_items) {
+            msc_flush_energy<N>(S, Eacc, lane);
+            cnt = 0;
+        }
+    }
+    if (cnt) msc_flush_energy<N>(S, Eacc, lane);   // adds twice the sums
+    __syncthreads();
+    if (tid < 32 && (SRC != WORDS_RAW || slot0 + tid < R)) E[slot0 + tid] = (int32_t)(((int64_t)g.m2 - Eacc[tid]) / 2);
+}
+
+template <bool W, bool BIG>
+const void *word_energy_kernel(int src) {
+    return src == WORDS_INIT  ? reinterpret_cast<const void *>(&k_word_energy<W, BIG, WORDS_INIT>)
+           : src == WORDS_POP ? reinterpret_cast<const void *>(&k_word_energy<W, BIG, WORDS_POP>)
+                              : reinterpret_cast<const void *>(&k_word_energy<W, BIG, WORDS_RAW>);
+}
+
+cudaError_t launch_word_energy(int src, GraphDev g, const int8_t *in, const int32_t *pos, int8_t *rows, int32_t *E,
+                               int32_t R, int32_t words, uint32_t key0, uint32_t key1, int32_t *bad, cudaStream_t st) {
+    const void *fn = g.wt ? (g.mbig ? word_energy_kernel<true, true>(src) : word_energy_kernel<true, false>(src))
+                          : (g.mbig ? word_energy_kernel<false, true>(src) : word_energy_kernel<false, false>(src));
+    const size_t smem = word_energy_smem(g);
+    if (cudaError_t e = raise_smem(const_cast<void *>(fn), smem)) return e;
+    void *args[] = {&g, &in, &pos, &rows, &E, &R, &key0, &key1, &bad};
+    return cudaLaunchKernel(fn, dim3(words), dim3(256), args, smem, st);
+}
+
 template <bool W, bool BIG, bool CL>
 void *msc_kernel(int mmax) {
     switch (msc_planes(mmax)) {
@@ -1819,19 +1957,7 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
         }
     }
     void *fn = select_kernel(G, field_bits, weighted, threads, g.mmax, g.mbig != 0, small);
-    // The attribute belongs to the kernel function, not to a context: only ever
-    // raise it, so that contexts configured earlier keep launching.
-    {
-        static std::mutex mu;
-        static std::unordered_map<void *, size_t> raised;
-        std::lock_guard<std::mutex> lock(mu);
-        size_t &cur = raised[fn];
-        if (smem > cur) {
-            cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            cur = smem;
-        }
-    }
+    if (cudaError_t e = raise_smem(fn, smem)) return e;
     const int nblk = (R + 4 * G - 1) / (4 * G);
     if (field_bits == 2) {
         // One cluster of two CTAs per word; the hardware schedules them as slots free up.
@@ -1884,6 +2010,27 @@ cudaError_t launch_sweep(const SweepConfig &cfg, const SweepArgs &a, cudaStream_
     lc.attrs = at;
     lc.numAttrs = cfg.field_bits == 2 ? 1 : 0;
     return cudaLaunchKernelExC(&lc, fn, args);
+}
+
+bool word_energy_fits(const GraphDev &g) {
+    int dev = 0, limit = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return g.mcol && word_energy_smem(g) <= (size_t)limit;
+}
+
+cudaError_t launch_init_words(const GraphDev &g, int8_t *spins, int32_t *E, int32_t Rpad, uint32_t key0, uint32_t key1,
+                              cudaStream_t st) {
+    return launch_word_energy(WORDS_INIT, g, nullptr, nullptr, spins, E, Rpad, Rpad / 32, key0, key1, nullptr, st);
+}
+
+cudaError_t launch_energy_words(const GraphDev &g, const int8_t *spins, int32_t *E, int32_t Rpad, cudaStream_t st) {
+    return launch_word_energy(WORDS_POP, g, spins, nullptr, nullptr, E, Rpad, Rpad / 32, 0u, 0u, nullptr, st);
+}
+
+cudaError_t launch_energy_raw(const GraphDev &g, const int8_t *raw, const int32_t *pos, int32_t *E, int32_t R,
+                              int32_t *bad, cudaStream_t st) {
+    return launch_word_energy(WORDS_RAW, g, raw, pos, nullptr, E, R, (R + 31) / 32, 0u, 0u, bad, st);
 }
 
 }  // namespace pa

@@ -163,6 +163,7 @@ struct pa_ctx {
         g.np = np;
         g.ncol = ncol;
         g.mmax = maxdeg;
+        g.m2 = m2;
         g.maxcls = maxcls;
         g.rp = d_rp.as<uint32_t>();
         g.col = d_col.as<uint16_t>();
@@ -734,8 +735,9 @@ int pa_anneal_begin(pa_ctx *c, const double *betas, int32_t K, int32_t R, int32_
     const int32_t Kc = std::max(K, 1);
     const int32_t Sc = std::max(sweeps, 1);
     const size_t nrs = (size_t)r.nch * pa::RS_CHUNK;
-    bool ok = r.spins[0].alloc(npR, ST) && r.spins[1].alloc(npR, ST) && r.fields[0].alloc(2 * npR, ST) &&
-              r.fields[1].alloc(2 * npR, ST) && r.E[0].alloc(4 * (size_t)r.Rpad, ST) &&
+    // The multi-spin-coded layouts keep no fields.
+    bool ok = r.spins[0].alloc(npR, ST) && r.spins[1].alloc(npR, ST) &&
+              (msc || (r.fields[0].alloc(2 * npR, ST) && r.fields[1].alloc(2 * npR, ST))) && r.E[0].alloc(4 * (size_t)r.Rpad, ST) &&
               r.E[1].alloc(4 * (size_t)r.Rpad, ST) && r.parent.alloc(4 * (size_t)r.Rpad, ST) &&
               r.partA.alloc(8 * (size_t)r.nch, ST) && r.partT.alloc(8 * (size_t)r.nch, ST) &&
               r.tval.alloc(8 * nrs, ST) && r.ploc.alloc(8 * nrs, ST) &&
@@ -798,14 +800,18 @@ int pa_anneal_begin(pa_ctx *c, const double *betas, int32_t K, int32_t R, int32_
         PA_CUDA(c, cudaMemsetAsync(r.ad_qsel.p, 0, 4 * (size_t)Kc, st));
         PA_CUDA(c, cudaMemsetAsync(r.ad_beta.p, 0, 8 * (size_t)Kc, st));
     }
-    // Initial population at beta = 0, fields and energies.
+    // Initial population at beta = 0 with its energies (and fields).
     r.cur = 0;
     const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-    PA_CUDA(c, cudaMemsetAsync(r.spins[0].p, 0, npR, st));
-    PA_CUDA(c, pa::launch_init(g, r.spins[0].as<int8_t>(), r.Rpad, k0, k1, st));
-    PA_CUDA(c, pa::launch_fields(g, r.spins[0].as<int8_t>(), r.fields[0].as<int16_t>(), r.E[0].as<int32_t>(),
-                                 r.Rpad, st));
-    r.launches += 2;
+    if (msc) {
+        PA_CUDA(c, pa::launch_init_words(g, r.spins[0].as<int8_t>(), r.E[0].as<int32_t>(), r.Rpad, k0, k1, st));
+        r.launches += 1;
+    } else {
+        PA_CUDA(c, pa::launch_init(g, r.spins[0].as<int8_t>(), r.Rpad, k0, k1, st));
+        PA_CUDA(c, pa::launch_fields(g, r.spins[0].as<int8_t>(), r.fields[0].as<int16_t>(), r.E[0].as<int32_t>(),
+                                     r.Rpad, st));
+        r.launches += 2;
+    }
     r.begun = true;
     return PA_OK;
 }
@@ -1213,11 +1219,12 @@ int pa_get_state(pa_ctx *c, int8_t *spins, int32_t *energies) {
     RunState &r = c->run;
     if (!r.begun) return fail(c, PA_ESTATE, "no anneal");
     if (int rc = pa_sync(c)) return rc;
-    if (spins) {
-        std::vector<int8_t> buf((size_t)r.R * c->np);
-        PA_CUDA(c, copy(c, buf.data(), r.spins[r.cur].p, buf.size(), cudaMemcpyDeviceToHost));
-        for (int32_t s = 0; s < r.R; ++s)
-            for (int32_t i = 0; i < c->n; ++i) spins[(size_t)s * c->n + i] = buf[(size_t)s * c->np + c->pos[i]];
+    if (spins) {   // vertex order, through the buffer the next step will write
+        int8_t *raw = r.spins[1 - r.cur].as<int8_t>();
+        PA_CUDA(c, pa::launch_rows_out(c->gdev(), c->d_pos.as<int32_t>(), r.spins[r.cur].as<int8_t>(), raw, r.R,
+                                       c->stream()));
+        PA_CUDA(c, copy(c, spins, raw, (size_t)r.R * c->n, cudaMemcpyDeviceToHost, c->stream(), true));
+        PA_CUDA(c, cudaStreamSynchronize(c->stream()));
     }
     if (energies)
         PA_CUDA(c, copy(c, energies, r.E[r.cur].p, 4 * (size_t)r.R, cudaMemcpyDeviceToHost));
@@ -1229,17 +1236,26 @@ int pa_set_state(pa_ctx *c, const int8_t *spins, int32_t steps_done) {
     RunState &r = c->run;
     if (!r.begun) return fail(c, PA_ESTATE, "pa_anneal_begin has not run");
     if (steps_done < 0 || steps_done > r.K) return fail(c, PA_EINVAL, "steps_done out of range");
-    for (size_t t = 0; t < (size_t)r.R * c->n; ++t)
-        if (spins[t] != 1 && spins[t] != -1) return fail(c, PA_EINVAL, "spins must be +1/-1");
     if (int rc = pa_sync(c)) return rc;
-    std::vector<int8_t> buf((size_t)r.Rpad * c->np, 0);
-    for (int32_t s = 0; s < r.Rpad; ++s) {
-        const int32_t src = s < r.R ? s : r.R - 1;   // padding slots mirror the last replica
-        for (int32_t i = 0; i < c->n; ++i) buf[(size_t)s * c->np + c->pos[i]] = spins[(size_t)src * c->n + i];
-    }
-    PA_CUDA(c, copy(c, r.spins[r.cur].p, buf.data(), buf.size(), cudaMemcpyHostToDevice));
-    PA_CUDA(c, pa::launch_fields(c->gdev(), r.spins[r.cur].as<int8_t>(), r.fields[r.cur].as<int16_t>(),
-                                 r.E[r.cur].as<int32_t>(), r.Rpad, c->stream()));
+    // The configurations go to the buffer the next step will write, are checked
+    // there, and only then replace the population.
+    cudaStream_t st = c->stream();
+    const pa::GraphDev g = c->gdev();
+    int8_t *raw = r.spins[1 - r.cur].as<int8_t>();
+    int32_t *bad = r.parent.as<int32_t>();   // written by the next step before it is read
+    int32_t wrong = 0;
+    PA_CUDA(c, copy(c, raw, spins, (size_t)r.R * c->n, cudaMemcpyHostToDevice, st, true));
+    PA_CUDA(c, cudaMemsetAsync(bad, 0, 4, st));
+    PA_CUDA(c, pa::launch_check(raw, (size_t)r.R * c->n, bad, st));
+    PA_CUDA(c, cudaMemcpyAsync(&wrong, bad, 4, cudaMemcpyDeviceToHost, st));
+    PA_CUDA(c, cudaStreamSynchronize(st));
+    if (wrong) return fail(c, PA_EINVAL, "spins must be +1/-1");
+    PA_CUDA(c, pa::launch_rows_in(g, raw, r.spins[r.cur].as<int8_t>(), r.R, r.Rpad, st));
+    if (r.variant == PA_VARIANT_MSC || r.variant == PA_VARIANT_MSC_PAIR)
+        PA_CUDA(c, pa::launch_energy_words(g, r.spins[r.cur].as<int8_t>(), r.E[r.cur].as<int32_t>(), r.Rpad, st));
+    else
+        PA_CUDA(c, pa::launch_fields(g, r.spins[r.cur].as<int8_t>(), r.fields[r.cur].as<int16_t>(),
+                                     r.E[r.cur].as<int32_t>(), r.Rpad, st));
     r.launches += 1;
     r.k_done = steps_done;
     return pa_sync(c);
@@ -1249,27 +1265,32 @@ int pa_energies(pa_ctx *c, const int8_t *spins, int32_t R, int32_t *energies, in
     if (!c || R < 0) return PA_EINVAL;
     if (R == 0 || (!energies && !cuts)) return PA_OK;
     if (!spins) return PA_EINVAL;
-    const size_t total = (size_t)R * c->n;
-    for (size_t t = 0; t < total; ++t)
-        if (spins[t] != 1 && spins[t] != -1) return fail(c, PA_EINVAL, "spins must be +1/-1");
-    // Same kernel that builds the fields and energies of a population at the
-    // start of an anneal; padding positions past n hold +1 and have no edges.
-    std::vector<int8_t> buf((size_t)R * c->np, 1);
-    for (int32_t s = 0; s < R; ++s)
-        for (int32_t i = 0; i < c->n; ++i) buf[(size_t)s * c->np + c->pos[i]] = spins[(size_t)s * c->n + i];
     cudaStream_t st = c->stream();
-    DevBuf dx, dh, dE;
+    const pa::GraphDev g = c->gdev();
+    const size_t raw = (size_t)R * c->n;
+    const bool words = pa::word_energy_fits(g);   // else rows and fields, as at the start of an anneal
+    DevBuf dx, dr, dh, dE;
     struct Drain {   // runs before the buffers are freed, on every return path
         cudaStream_t s;
         ~Drain() { cudaStreamSynchronize(s); }
     } drain{st};
-    if (!dx.alloc(buf.size(), st) || !dh.alloc(2 * buf.size(), st) || !dE.alloc(4 * (size_t)R, st))
+    if (!dx.alloc(raw, st) || !dE.alloc(4 * ((size_t)R + 1), st) ||
+        (!words && (!dr.alloc((size_t)R * c->np, st) || !dh.alloc(2 * (size_t)R * c->np, st))))
         return fail(c, PA_ENOMEM, "device allocation failed");
-    std::vector<int32_t> E(R);
-    PA_CUDA(c, copy(c, dx.p, buf.data(), buf.size(), cudaMemcpyHostToDevice, st, true));
-    PA_CUDA(c, pa::launch_fields(c->gdev(), dx.as<int8_t>(), dh.as<int16_t>(), dE.as<int32_t>(), R, st));
-    PA_CUDA(c, copy(c, E.data(), dE.p, 4 * (size_t)R, cudaMemcpyDeviceToHost, st, true));
+    std::vector<int32_t> E((size_t)R + 1);   // the last entry: a byte other than +1 / -1 was found
+    int32_t *bad = dE.as<int32_t>() + R;
+    PA_CUDA(c, copy(c, dx.p, spins, raw, cudaMemcpyHostToDevice, st, true));
+    PA_CUDA(c, cudaMemsetAsync(bad, 0, 4, st));
+    if (words) {
+        PA_CUDA(c, pa::launch_energy_raw(g, dx.as<int8_t>(), c->d_pos.as<int32_t>(), dE.as<int32_t>(), R, bad, st));
+    } else {
+        PA_CUDA(c, pa::launch_check(dx.as<int8_t>(), raw, bad, st));
+        PA_CUDA(c, pa::launch_rows_in(g, dx.as<int8_t>(), dr.as<int8_t>(), R, R, st));
+        PA_CUDA(c, pa::launch_fields(g, dr.as<int8_t>(), dh.as<int16_t>(), dE.as<int32_t>(), R, st));
+    }
+    PA_CUDA(c, copy(c, E.data(), dE.p, 4 * ((size_t)R + 1), cudaMemcpyDeviceToHost, st, true));
     PA_CUDA(c, cudaStreamSynchronize(st));
+    if (E[R]) return fail(c, PA_EINVAL, "spins must be +1/-1");
     for (int32_t s = 0; s < R; ++s) {
         if (energies) energies[s] = E[s];
         if (cuts) cuts[s] = (c->W - (int64_t)E[s]) / 2;

@@ -106,6 +106,7 @@ constexpr int RS_CHUNK = 256;                   // slots per resampling CTA (pow
 
 struct GraphDev {
     int32_t n, np, ncol, mmax, maxcls;   // maxcls: largest colour class
+    int32_t m2;           // stored entries (twice the edges)
     const uint32_t *rp;   // [n+1] row pointers, position order
     const uint16_t *col;  // [2M] neighbour positions
     const int8_t *wt;     // [2M] weights or nullptr (all +1)
@@ -184,6 +185,24 @@ cudaError_t launch_init(const GraphDev &g, int8_t *spins, int32_t Rpad, uint32_t
                         uint32_t key1, cudaStream_t st);
 cudaError_t launch_fields(const GraphDev &g, const int8_t *spins, int16_t *fields, int32_t *E,
                           int32_t Rpad, cudaStream_t st);
+// Word kernels (k_sweep.cu), for layouts that keep no fields: the initial
+// population with its energies, the energies of a population (both Rpad
+// replicas, a multiple of 32), and of R configurations in vertex order (*bad set
+// if a byte is not +1 / -1). They need slice rows and the words in shared memory.
+bool word_energy_fits(const GraphDev &g);
+cudaError_t launch_init_words(const GraphDev &g, int8_t *spins, int32_t *E, int32_t Rpad, uint32_t key0, uint32_t key1,
+                              cudaStream_t st);
+cudaError_t launch_energy_words(const GraphDev &g, const int8_t *spins, int32_t *E, int32_t Rpad, cudaStream_t st);
+cudaError_t launch_energy_raw(const GraphDev &g, const int8_t *raw, const int32_t *pos, int32_t *E, int32_t R,
+                              int32_t *bad, cudaStream_t st);
+// Population rows (position order, np bytes) <-> configurations in vertex order
+// (n bytes each): out writes R of them; in reads R of them into Rpad rows, the
+// padding rows repeating the last one; check sets *bad if a byte is not +1 / -1.
+cudaError_t launch_rows_out(const GraphDev &g, const int32_t *pos, const int8_t *rows, int8_t *raw, int32_t R,
+                            cudaStream_t st);
+cudaError_t launch_rows_in(const GraphDev &g, const int8_t *raw, int8_t *rows, int32_t R, int32_t Rpad,
+                           cudaStream_t st);
+cudaError_t launch_check(const int8_t *raw, size_t bytes, int32_t *bad, cudaStream_t st);
 // Minimum of the energies (and the step's start stamp), then weights + parents.
 cudaError_t launch_rs_min(const ResampleArgs &a, cudaStream_t st);
 cudaError_t launch_rs_rest(const ResampleArgs &a, cudaStream_t st);
