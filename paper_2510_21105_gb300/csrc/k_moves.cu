@@ -467,13 +467,59 @@ __global__ void __launch_bounds__(256) k_nlm_block(NlmArgs a) {
 }
 
 // -------------------------------------------------------------- adaptive ---
+// Pairwise tree sum of v[0..n) padded with zeros to a power of two, computed
+// left to right with a stack of completed subtrees (same additions as the
+// level-by-level tree).
+__device__ __forceinline__ double tree_sum_seq(const double *v, int n) {
+    double st[20];
+    int lv[20];
+    int top = 0;
+    int L = 1;
+    while (L < n) L <<= 1;
+    for (int i = 0; i < L; ++i) {
+        double x = i < n ? __ldcg(&v[i]) : 0.0;   // other CTAs of the launch wrote them
+        int l = 0;
+        while (top > 0 && lv[top - 1] == l) {
+            x = __dadd_rn(st[top - 1], x);
+            --top;
+            ++l;
+        }
+        st[top] = x;
+        lv[top] = l;
+        ++top;
+    }
+    return st[0];
+}
+
+// Level j of step k: the controller's outputs.
+__device__ __forceinline__ void ad_take(const AdaptArgs &a, int n_prev, int j) {
+    int dn = 1 << (a.J - j);
+    if (dn > a.nmax - n_prev) dn = a.nmax - n_prev;
+    const int nk = n_prev + dn;
+    a.state[0] = nk;
+    a.qsel[a.k] = dn - 1;
+    a.tidx[a.k] = nk;
+    a.jsel[a.k] = j;
+    a.beta[a.k] = __dmul_rn((double)nk, a.delta);
+    a.active[a.k] = 1;
+}
+
 // ESS partials, one CTA per (256-slot chunk, level j): w = q_j^(E - E_min) by
 // squarings and w*w for one slot per thread, then the chunk's pairwise tree
 // sums (lanes by butterflies, then the eight warp sums in pairs), the same
 // additions as the tree over the whole padded population.
+// The CTA that finishes last (a counter that wraps to zero, state[3]) chooses
+// the level: one warp per level sums the chunk partials of w and w*w in the
+// tree's order (each lane a contiguous power-of-two block of chunks, then
+// butterflies; zero padding adds exact zeros), ESS_j = A^2 / B, and the smallest
+// j with ESS_j >= rho R is taken (else J).
 __global__ void __launch_bounds__(RS_CHUNK) k_ad_partials(AdaptArgs a) {
     const int n_prev = a.state[0];
-    if (n_prev >= a.nmax) return;
+    if (n_prev >= a.nmax) {
+        if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) a.active[a.k] = 0;
+        return;
+    }
+    __shared__ int last, ok_lvl[32];
     __shared__ double sw[2][RS_CHUNK / 32];
     const int j = blockIdx.y;
     const int slot = blockIdx.x * RS_CHUNK + threadIdx.x;
@@ -506,71 +552,21 @@ __global__ void __launch_bounds__(RS_CHUNK) k_ad_partials(AdaptArgs a) {
         for (int h = 1; h < RS_CHUNK / 32; h <<= 1)
             for (int i = 0; i < RS_CHUNK / 32; i += 2 * h) v[i] = __dadd_rn(v[i], v[i + h]);
         a.part[((size_t)j * 2 + threadIdx.x) * a.nch + blockIdx.x] = v[0];
+        __threadfence();
     }
-}
-
-// Pairwise tree sum of v[0..n) padded with zeros to a power of two, computed
-// left to right with a stack of completed subtrees (same additions as the
-// level-by-level tree).
-__device__ double tree_sum_seq(const double *v, int n) {
-    double st[20];
-    int lv[20];
-    int top = 0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const unsigned total = gridDim.x * gridDim.y;
+        last = atomicInc(reinterpret_cast<unsigned *>(&a.state[3]), total - 1u) == total - 1u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
     int L = 1;
-    while (L < n) L <<= 1;
-    for (int i = 0; i < L; ++i) {
-        double x = i < n ? v[i] : 0.0;
-        int l = 0;
-        while (top > 0 && lv[top - 1] == l) {
-            x = __dadd_rn(st[top - 1], x);
-            --top;
-            ++l;
-        }
-        st[top] = x;
-        lv[top] = l;
-        ++top;
-    }
-    return st[0];
-}
-
-// Level choice. Mode 1: one warp per level j sums the chunk partials of w and
-// w*w in the tree's order (each lane a contiguous power-of-two block of
-// chunks, then butterflies; zero padding adds exact zeros), ESS_j = A^2 / B,
-// and the smallest j with ESS_j >= rho R is taken (else J).
-__global__ void k_ad_choose(AdaptArgs a) {
-    const int n_prev = a.state[0];
-    const int lane = threadIdx.x & 31, lvl = threadIdx.x >> 5;
-    __shared__ int ok_lvl[32];
-    if (n_prev >= a.nmax) {
-        if (threadIdx.x == 0) a.active[a.k] = 0;
-        return;
-    }
-    if (a.mode == 2) {
-        if (threadIdx.x == 0) {
-            int j = a.state[1];
-            if (a.k > 0) {
-                const double acc = (double)a.accepts[a.k - 1];
-                if (acc < a.acc_lo_n) j = min(j + 1, a.J);
-                else if (acc > a.acc_hi_n) j = max(j - 1, 0);
-            }
-            int dn = 1 << (a.J - j);
-            if (dn > a.nmax - n_prev) dn = a.nmax - n_prev;
-            const int nk = n_prev + dn;
-            a.state[0] = nk;
-            a.state[1] = j;
-            a.qsel[a.k] = dn - 1;
-            a.tidx[a.k] = nk;
-            a.jsel[a.k] = j;
-            a.beta[a.k] = __dmul_rn((double)nk, a.delta);
-            a.active[a.k] = 1;
-        }
-        return;
-    }
-    if (lvl <= a.J) {
-        int L = 1;
-        while (L < a.nch) L <<= 1;
-        const int blk = L > 32 ? L / 32 : 1;
-        const int lo = lane * blk, cnt = max(0, min(blk, a.nch - lo));
+    while (L < a.nch) L <<= 1;
+    const int blk = L > 32 ? L / 32 : 1;
+    const int lo = lane * blk, cnt = max(0, min(blk, a.nch - lo));
+    for (int lvl = warp; lvl <= a.J; lvl += RS_CHUNK / 32) {
         double A = tree_sum_seq(a.part + ((size_t)lvl * 2 + 0) * a.nch + min(lo, a.nch), cnt);
         double B = tree_sum_seq(a.part + ((size_t)lvl * 2 + 1) * a.nch + min(lo, a.nch), cnt);
 #pragma unroll
@@ -588,16 +584,25 @@ __global__ void k_ad_choose(AdaptArgs a) {
                 j = l;
                 break;
             }
-        int dn = 1 << (a.J - j);
-        if (dn > a.nmax - n_prev) dn = a.nmax - n_prev;
-        const int nk = n_prev + dn;
-        a.state[0] = nk;
-        a.qsel[a.k] = dn - 1;
-        a.tidx[a.k] = nk;
-        a.jsel[a.k] = j;
-        a.beta[a.k] = __dmul_rn((double)nk, a.delta);
-        a.active[a.k] = 1;
+        ad_take(a, n_prev, j);
     }
+}
+
+// Acceptance-rate rule, one thread.
+__global__ void k_ad_accept(AdaptArgs a) {
+    const int n_prev = a.state[0];
+    if (n_prev >= a.nmax) {
+        a.active[a.k] = 0;
+        return;
+    }
+    int j = a.state[1];
+    if (a.k > 0) {
+        const double acc = (double)a.accepts[a.k - 1];
+        if (acc < a.acc_lo_n) j = min(j + 1, a.J);
+        else if (acc > a.acc_hi_n) j = max(j - 1, 0);
+    }
+    a.state[1] = j;
+    ad_take(a, n_prev, j);
 }
 
 // ------------------------------------------------------------- reheating ---
@@ -712,8 +717,8 @@ cudaError_t launch_nonlocal(const NlmArgs &a, void *scratch, cudaStream_t st, in
 }
 
 cudaError_t launch_adapt(const AdaptArgs &a, cudaStream_t st) {
-    if (a.mode != 2) k_ad_partials<<<dim3(a.nch, a.J + 1), RS_CHUNK, 0, st>>>(a);
-    k_ad_choose<<<1, a.mode == 2 ? 32 : 32 * (a.J + 1), 0, st>>>(a);
+    if (a.mode == 2) k_ad_accept<<<1, 1, 0, st>>>(a);
+    else k_ad_partials<<<dim3(a.nch, a.J + 1), RS_CHUNK, 0, st>>>(a);
     return cudaGetLastError();
 }
 

@@ -13,9 +13,9 @@
 //   new slots [F(P_r), F(P_r + t_r)) copy replica r, with the systematic
 //   count F(P) = floor((P R 2^32 + o T) / (T 2^32)) and o the Philox word of
 //   (0, 0, k, tag 1). Sum of copies is exactly R.
-// Three kernels per step over chunks of RS_CHUNK slots: minimum, weights
-// (chunk tree sums of w, chunk totals and local prefixes of t), parents.
-#include "pa_internal.cuh"
+// The sweep kernels leave E_min of the next step; k_rs_min finds it where the
+// energies came another way. k_rs_step does the rest.
+#include "pa_cluster.cuh"
 
 namespace pa {
 namespace {
@@ -83,137 +83,67 @@ __global__ void k_fields_energy(GraphDev g, const int8_t *spins, int16_t *fields
     }
 }
 
-// The resampling kernels run one CTA of RS_CHUNK threads per chunk of
-// RS_CHUNK slots, one slot per thread.
 __global__ void __launch_bounds__(RS_CHUNK) k_rs_min(ResampleArgs a) {
-    if (a.active && !a.active[a.k]) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.stamp[a.k] = gtimer();
     const int r = blockIdx.x * RS_CHUNK + threadIdx.x;
     int v = r < a.R ? a.E[r] : 0x7FFFFFFF;
     v = __reduce_min_sync(0xFFFFFFFFu, v);
     if ((threadIdx.x & 31) == 0) atomicMin(&a.emin[a.k], v);
 }
 
-__global__ void __launch_bounds__(RS_CHUNK) k_rs_weights(ResampleArgs a) {
-    if (a.active && !a.active[a.k]) return;
+// Weights, sums and parents in one cluster (pa_cluster.cuh) of CTAs small enough
+// to find room beside other work. Bound by latency and the FP64 rate (about two
+// results per SM and cycle). With the minimum left by the sweep a step needs one
+// launch instead of three (minimum, weights, parents); us per step: R = 2048
+// 3.9 against 6.9 and two launch gaps, R = 32768 with long runs of one parent
+// 20.2 against 21.0. Whole anneals: n = 800, R = 256 6.40 -> 5.72 ms (100 steps),
+// ESS-adaptive R = 2048 56.7 -> 53.4 ms (384 steps).
+constexpr int RS_THREADS = 256;
+
+template <int K>
+__global__ void __launch_bounds__(RS_THREADS) k_rs_step(ResampleArgs a) {
+    namespace cg = cooperative_groups;
+    __shared__ ClusterShared sh;
     __shared__ double qs[32];
-    __shared__ double wsum[RS_CHUNK / 32];
-    __shared__ unsigned long long tsum[RS_CHUNK / 32];
+    const int rank = (int)cg::this_cluster().block_rank();
+    if (rank == 0 && threadIdx.x == 0) a.stamp[a.k] = gtimer();
+    if (a.active && !a.active[a.k]) return;   // the whole cluster
     const int row = a.qsel ? a.qsel[a.k] : a.k;
     if (threadIdx.x < 32) qs[threadIdx.x] = a.qpow[(size_t)row * 32 + threadIdx.x];
+    const int r0 = (rank * RS_THREADS + (int)threadIdx.x) * K;
+    const int32_t emin = a.emin[a.k];
+    int32_t e[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) e[i] = r0 + i < a.R ? a.E[r0 + i] : emin;
     __syncthreads();
-    const int r = blockIdx.x * RS_CHUNK + threadIdx.x;
-    double w = 0.0;
-    unsigned long long t = 0ull;
-    if (r < a.R) {
-        uint32_t d = (uint32_t)(a.E[r] - a.emin[a.k]);
-        w = 1.0;
-        while (d) {
-            w = __dmul_rn(w, qs[__ffs(d) - 1]);
-            d &= d - 1u;
-        }
-        t = (unsigned long long)__dmul_rn(w, 4294967296.0);
-    }
-    // Pairwise tree: lane butterflies (32 slots), then the eight warp sums in pairs.
-    double s = w;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) s = __dadd_rn(s, __shfl_xor_sync(0xFFFFFFFFu, s, off));
-    // Exclusive prefix of t over the chunk.
-    unsigned long long inc = t;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, inc, off);
-        if (lane >= off) inc += y;
-    }
-    if (lane == 31) {
-        wsum[warp] = s;
-        tsum[warp] = inc;
-    }
+    cluster_table(sh, qs);
     __syncthreads();
-    unsigned long long pre = inc - t;
-    for (int w2 = 0; w2 < warp; ++w2) pre += tsum[w2];
-    a.ploc[r] = pre;   // sized nch * RS_CHUNK; slots past R hold t = 0
-    a.tval[r] = t;
-    if (threadIdx.x == 0) {
-        for (int h = 1; h < RS_CHUNK / 32; h <<= 1)
-            for (int i = 0; i < RS_CHUNK / 32; i += 2 * h) wsum[i] = __dadd_rn(wsum[i], wsum[i + h]);
-        unsigned long long ct = 0;
-        for (int w2 = 0; w2 < RS_CHUNK / 32; ++w2) ct += tsum[w2];
-        a.partA[blockIdx.x] = wsum[0];
-        a.partT[blockIdx.x] = ct;
+    double w[K];
+    unsigned long long t[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        w[i] = r0 + i < a.R ? cluster_weight(sh, qs, (uint32_t)(e[i] - emin)) : 0.0;
+        t[i] = (unsigned long long)__dmul_rn(w[i], 4294967296.0);
     }
-}
-
-__global__ void __launch_bounds__(RS_CHUNK) k_rs_parents(ResampleArgs a) {
-    if (a.active && !a.active[a.k]) return;
-    __shared__ unsigned long long sh_T, sh_off, sh_m;
-    __shared__ uint32_t sh_o;
-    if (threadIdx.x < 32) {   // warp 0: totals over the chunks
-        const int lane = threadIdx.x;
-        // T and this chunk's offset: integer sums, in any order.
-        unsigned long long T = 0, off = 0;
-        for (int c = lane; c < a.nch; c += 32) {
-            const unsigned long long t = a.partT[c];
-            T += t;
-            off += c < (int)blockIdx.x ? t : 0ull;
-        }
+    unsigned long long P = cluster_sums<RS_THREADS, K>(sh, w, t);
+    const unsigned long long T = sh.T, m = ~0ull / T;
+    const uint32_t o = philox10(make_uint4(0u, 0u, (uint32_t)a.k, TAG_RESAMPLE), a.key0, a.key1).x;
+    // Slot r fills new slots [F(P_r), F(P_r + t_r)).
+    int32_t lo = systematic_count_m(P, a.R, T, m, o);
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            T += __shfl_xor_sync(0xFFFFFFFFu, T, d);
-            off += __shfl_xor_sync(0xFFFFFFFFu, off, d);
-        }
-        // A: the pairwise tree over the chunk sums padded with zeros to a power
-        // of two L <= 256. Lane l holds the aligned block of B = max(L/32, 1)
-        // chunks starting at l B: the tree levels inside the block run in the
-        // lane, the remaining levels pair lanes l and l ^ d, so every level adds
-        // elements 2i and 2i + 1 of the level below, as the sequential tree does.
-        double A = 0.0;
-        if (blockIdx.x == 0) {
-            int L = 1;
-            while (L < a.nch) L <<= 1;
-            const int B = L > 32 ? L / 32 : 1;
-            double v[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int c = lane * B + j;
-                v[j] = (j < B && c < a.nch) ? a.partA[c] : 0.0;
-            }
-#pragma unroll
-            for (int w = 1; w < 8; w <<= 1)
-#pragma unroll
-                for (int j = 0; j < 8; j += 2 * w)
-                    if (w < B) v[j] = __dadd_rn(v[j], v[j + w]);
-            A = v[0];
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) A = __dadd_rn(A, __shfl_xor_sync(0xFFFFFFFFu, A, d));
-        }
-        if (lane == 0) {
-            sh_T = T;
-            sh_m = T ? ~0ull / T : 0ull;
-            sh_off = off;
-            sh_o = philox10(make_uint4(0u, 0u, (uint32_t)a.k, TAG_RESAMPLE), a.key0, a.key1).x;
-            if (blockIdx.x == 0) {
-                a.recA[a.k] = A;
-                a.recT[a.k] = T;
-                a.reco[a.k] = sh_o;
-            }
-        }
+    for (int i = 0; i < K; ++i) {
+        P += t[i];
+        const int32_t hi = systematic_count_m(P, a.R, T, m, o);
+        const bool real = r0 + i < a.R;
+        if (real && a.counts) a.counts[(size_t)a.k * a.R + r0 + i] = hi - lo;
+        fill_parents(a.parent, lo, real ? hi : lo, r0 + i);
+        lo = hi;
     }
-    __syncthreads();
-    const unsigned long long T = sh_T, off = sh_off, m = sh_m;
-    const uint32_t o = sh_o;
-    const int r = blockIdx.x * RS_CHUNK + threadIdx.x;
-    // Slot r fills new slots [F(P_r), F(P_r + t_r)); P_r + t_r = P_{r+1} inside
-    // the chunk, so the upper end is the next lane's lower end.
-    const unsigned long long P = off + a.ploc[r];
-    const int32_t lo = systematic_count_m(P, a.R, T, m, o);
-    int32_t hi = __shfl_down_sync(0xFFFFFFFFu, lo, 1);
-    if ((threadIdx.x & 31) == 31) hi = systematic_count_m(P + a.tval[r], a.R, T, m, o);
-    if (r < a.R) {
-        for (int s = lo; s < hi; ++s) a.parent[s] = r;
-        if (a.counts) a.counts[(size_t)a.k * a.R + r] = hi - lo;
+    if (r0 == 0) {
+        a.recA[a.k] = sh.A;
+        a.recT[a.k] = T;
+        a.reco[a.k] = o;
     }
+    cg::this_cluster().sync();   // no CTA leaves while another may read its totals
 }
 
 // Rows <-> configurations in vertex order: one CTA per row, the row in shared
@@ -331,10 +261,15 @@ cudaError_t launch_rs_min(const ResampleArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_rs_rest(const ResampleArgs &a, cudaStream_t st) {
-    k_rs_weights<<<a.nch, RS_CHUNK, 0, st>>>(a);
-    k_rs_parents<<<a.nch, RS_CHUNK, 0, st>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_rs_step(const ResampleArgs &a, cudaStream_t st) {
+    const ClusterShape shape = cluster_shape(a.R, RS_THREADS);
+    auto *kernel = shape.k == 1   ? &k_rs_step<1>
+                   : shape.k == 2 ? &k_rs_step<2>
+                   : shape.k == 4 ? &k_rs_step<4>
+                   : shape.k == 8 ? &k_rs_step<8>
+                   : shape.k == 16 ? &k_rs_step<16>
+                                   : &k_rs_step<32>;
+    return launch_cluster(kernel, shape, RS_THREADS, st, a);
 }
 
 cudaError_t launch_stamp(unsigned long long *stamp, cudaStream_t st) {

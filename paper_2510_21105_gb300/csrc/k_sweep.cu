@@ -394,7 +394,10 @@ __global__ void __launch_bounds__(1024) k_sweep(const SweepArgs a) {
                 *reinterpret_cast<uint2 *>(a.fields_out + row) = f[q];
             }
         }
-        if (tid < 4 * G) a.E_out[slot0 + tid] = Eacc[tid];
+        if (tid < 4 * G) {
+            a.E_out[slot0 + tid] = Eacc[tid];
+            if (a.emin_next && slot0 + tid < a.R) atomicMin(a.emin_next, Eacc[tid]);
+        }
         if (tid == 0 && misc[5]) a.best_rec[blk] = make_int4(misc[0], misc[1], misc[2], misc[3]);
         const uint32_t wsum = __reduce_add_sync(0xFFFFFFFFu, nacc);
         if (act && lane == 0 && wsum) atomicAdd(&a.accepts[a.k], (unsigned long long)wsum);
@@ -675,7 +678,10 @@ __global__ void __launch_bounds__(NTB, MINB) k_sweep_packed(const SweepArgs a) {
                 *reinterpret_cast<uint2 *>(a.fields_out + row) = make_uint2(fx[q], fy[q]);
             }
         }
-        if (tid < 4) a.E_out[slot0 + tid] = Eacc[tid];
+        if (tid < 4) {
+            a.E_out[slot0 + tid] = Eacc[tid];
+            if (a.emin_next && slot0 + tid < a.R) atomicMin(a.emin_next, Eacc[tid]);
+        }
         if (tid == 0 && misc[5]) a.best_rec[blk] = make_int4(misc[0], misc[1], misc[2], misc[3]);
         const uint32_t wsum = __reduce_add_sync(0xFFFFFFFFu, nacc);
         if (act && lane == 0 && wsum) atomicAdd(&a.accepts[a.k], (unsigned long long)wsum);
@@ -970,7 +976,10 @@ __global__ void __launch_bounds__(2 * NH) k_sweep_small(const SweepArgs a) {
                 *reinterpret_cast<uint2 *>(a.fields_out + row) = make_uint2(fx[q], fy[q]);
             }
         }
-        if (tid < 4) a.E_out[slot0 + tid] = Eacc[tid];
+        if (tid < 4) {
+            a.E_out[slot0 + tid] = Eacc[tid];
+            if (a.emin_next && slot0 + tid < a.R) atomicMin(a.emin_next, Eacc[tid]);
+        }
         if (tid == 0 && misc[5]) a.best_rec[blk] = make_int4(misc[0], misc[1], misc[2], misc[3]);
         const uint32_t wsum = __reduce_add_sync(0xFFFFFFFFu, nacc);
         if (act && lane == 0 && wsum) atomicAdd(&a.accepts[a.k], (unsigned long long)wsum);
@@ -1692,7 +1701,11 @@ __global__ void __launch_bounds__(256, 4) k_sweep_msc(const SweepArgs a) {
             msc_unpack_rows(w4, a.spins_out, slot0, np, n, c);
         }
         if (rank == 0) {
-            if (tid < 32) a.E_out[slot0 + tid] = Eacc[tid];
+            if (warp == 0) {
+                a.E_out[slot0 + lane] = Eacc[lane];
+                const int v = __reduce_min_sync(0xFFFFFFFFu, slot0 + lane < a.R ? Eacc[lane] : 0x7FFFFFFF);
+                if (lane == 0 && a.emin_next) atomicMin(a.emin_next, v);
+            }
             if (tid == 0 && misc[5]) a.best_rec[blk] = make_int4(misc[0], misc[1], misc[2], misc[3]);
         }
         const uint32_t wsum = __reduce_add_sync(0xFFFFFFFFu, nacc);

@@ -118,7 +118,6 @@ struct RunState {
     int32_t ntables = 0, nq = 0;
     // device
     DevBuf spins[2], fields[2], E[2], parent;
-    DevBuf partA, partT, tval, ploc;
     DevBuf d_tables, d_tidx, d_qpow, d_qblk;
     DevBuf rec_emin, rec_A, rec_T, rec_o, rec_acc, rec_sweep, rec_stamp, rec_counts;
     DevBuf rec_nlm_pairs, rec_nlm_flips, rec_jsel;
@@ -130,6 +129,7 @@ struct RunState {
     double ad_delta = 0.0;
     int32_t ad_nmax = 0;
     int cur = 0;
+    bool have_emin = false;              // rec_emin[k_done] holds the minimum of the population's energies
     pa::SweepConfig sweep{};
     int variant = PA_VARIANT_I8;
     // accounting
@@ -734,13 +734,10 @@ int pa_anneal_begin(pa_ctx *c, const double *betas, int32_t K, int32_t R, int32_
     const size_t npR = (size_t)c->np * r.Rpad;
     const int32_t Kc = std::max(K, 1);
     const int32_t Sc = std::max(sweeps, 1);
-    const size_t nrs = (size_t)r.nch * pa::RS_CHUNK;
     // The multi-spin-coded layouts keep no fields.
     bool ok = r.spins[0].alloc(npR, ST) && r.spins[1].alloc(npR, ST) &&
               (msc || (r.fields[0].alloc(2 * npR, ST) && r.fields[1].alloc(2 * npR, ST))) && r.E[0].alloc(4 * (size_t)r.Rpad, ST) &&
               r.E[1].alloc(4 * (size_t)r.Rpad, ST) && r.parent.alloc(4 * (size_t)r.Rpad, ST) &&
-              r.partA.alloc(8 * (size_t)r.nch, ST) && r.partT.alloc(8 * (size_t)r.nch, ST) &&
-              r.tval.alloc(8 * nrs, ST) && r.ploc.alloc(8 * nrs, ST) &&
               r.d_tables.alloc(4 * r.tables.size(), ST) && r.d_tidx.alloc(4 * (size_t)Kc, ST) &&
               r.d_qpow.alloc(8 * r.qpow.size(), ST) && r.rec_emin.alloc(4 * (size_t)Kc, ST) &&
               r.rec_A.alloc(8 * (size_t)Kc, ST) && r.rec_T.alloc(8 * (size_t)Kc, ST) &&
@@ -802,6 +799,7 @@ int pa_anneal_begin(pa_ctx *c, const double *betas, int32_t K, int32_t R, int32_
     }
     // Initial population at beta = 0 with its energies (and fields).
     r.cur = 0;
+    r.have_emin = false;
     const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
     if (msc) {
         PA_CUDA(c, pa::launch_init_words(g, r.spins[0].as<int8_t>(), r.E[0].as<int32_t>(), r.Rpad, k0, k1, st));
@@ -854,18 +852,16 @@ int enqueue_step(pa_ctx *c, int32_t k, cudaStream_t st, bool time_sweep) {
     }
     ra.active = nullptr;   // the minimum runs before the adaptive decision
     ra.emin = r.rec_emin.as<int32_t>();
-    ra.partA = r.partA.as<double>();
-    ra.partT = r.partT.as<unsigned long long>();
-    ra.tval = r.tval.as<unsigned long long>();
-    ra.ploc = r.ploc.as<unsigned long long>();
     ra.parent = r.parent.as<int32_t>();
     ra.recA = r.rec_A.as<double>();
     ra.recT = r.rec_T.as<unsigned long long>();
     ra.reco = r.rec_o.as<uint32_t>();
     ra.counts = o.record_counts ? r.rec_counts.as<int32_t>() : nullptr;
     ra.stamp = r.rec_stamp.as<unsigned long long>();
-    PA_CUDA(c, pa::launch_rs_min(ra, st));
-    r.launches += 1;
+    if (!r.have_emin) {
+        PA_CUDA(c, pa::launch_rs_min(ra, st));
+        r.launches += 1;
+    }
     if (o.adaptive) {
         pa::AdaptArgs aa{};
         aa.E = r.E[cur].as<int32_t>();
@@ -891,11 +887,11 @@ int enqueue_step(pa_ctx *c, int32_t k, cudaStream_t st, bool time_sweep) {
         aa.acc_lo_n = o.acc_lo * attempts;
         aa.acc_hi_n = o.acc_hi * attempts;
         PA_CUDA(c, pa::launch_adapt(aa, st));
-        r.launches += o.adaptive == 2 ? 1 : 2;
+        r.launches += 1;
         ra.active = r.ad_active.as<int32_t>();
     }
-    PA_CUDA(c, pa::launch_rs_rest(ra, st));
-    r.launches += 2;
+    PA_CUDA(c, pa::launch_rs_step(ra, st));
+    r.launches += 1;
 
     pa::SweepArgs sa{};
     sa.g = g;
@@ -923,6 +919,11 @@ int enqueue_step(pa_ctx *c, int32_t k, cudaStream_t st, bool time_sweep) {
     sa.best_cfg = r.best_cfg.as<int8_t>();
     sa.accepts = r.rec_acc.as<unsigned long long>();
     sa.sweep_emin = r.rec_sweep.as<int32_t>();
+    // The sweep leaves the minimum that the next step's weights need, unless
+    // non-local moves change the energies after it.
+    const bool nlm = o.nlm_period > 0 && k > 0 && k % o.nlm_period == 0;
+    r.have_emin = !nlm && k + 1 < r.K;
+    sa.emin_next = r.have_emin ? r.rec_emin.as<int32_t>() + (k + 1) : nullptr;
     cudaEvent_t s0 = nullptr, s1 = nullptr;
     if (time_sweep) {
         PA_CUDA(c, cudaEventCreate(&s0));
@@ -947,7 +948,7 @@ int enqueue_step(pa_ctx *c, int32_t k, cudaStream_t st, bool time_sweep) {
     r.launches += 1;
     r.sweep_launches += 1;
     r.cur = nxt;
-    if (o.nlm_period > 0 && k > 0 && k % o.nlm_period == 0) {
+    if (nlm) {
         pa::NlmArgs na{};
         na.g = g;
         na.pos = c->d_pos.as<int32_t>();
@@ -1258,6 +1259,10 @@ int pa_set_state(pa_ctx *c, const int8_t *spins, int32_t steps_done) {
                                      r.E[r.cur].as<int32_t>(), r.Rpad, st));
     r.launches += 1;
     r.k_done = steps_done;
+    // Minima that the replaced population's run left for the steps to come.
+    if (steps_done < r.K)
+        PA_CUDA(c, cudaMemsetAsync(r.rec_emin.as<int32_t>() + steps_done, 0x7F, 4 * (size_t)(r.K - steps_done), st));
+    r.have_emin = false;
     return pa_sync(c);
 }
 

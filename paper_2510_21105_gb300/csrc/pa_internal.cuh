@@ -102,7 +102,7 @@ static __device__ __forceinline__ int32_t systematic_count_m(unsigned long long 
 }
 
 constexpr int32_t EMIN_SENTINEL = 0x7F7F7F7F;  // byte-fillable "+infinity"
-constexpr int RS_CHUNK = 256;                   // slots per resampling CTA (power of two)
+constexpr int RS_CHUNK = 256;                   // slots per CTA of the ESS partials and the minimum
 
 struct GraphDev {
     int32_t n, np, ncol, mmax, maxcls;   // maxcls: largest colour class
@@ -158,6 +158,7 @@ struct SweepArgs {
     int8_t *best_cfg;            // [nblk][np] configuration of that record
     unsigned long long *accepts; // [K] accepted flips per step
     int32_t *sweep_emin;         // [K][S] minimum energy per sweep end
+    int32_t *emin_next;          // minimum energy entering the next step, or nullptr
 };
 
 struct ResampleArgs {
@@ -168,10 +169,6 @@ struct ResampleArgs {
     const int32_t *qsel;         // adaptive: row of qpow for step k (nullptr: row k)
     const int32_t *active;       // [K] or nullptr
     int32_t *emin;               // [K]
-    double *partA;               // [nch]
-    unsigned long long *partT;   // [nch]
-    unsigned long long *tval;    // [Rpad]
-    unsigned long long *ploc;    // [Rpad]
     int32_t *parent;             // [Rpad]
     double *recA;                // [K]
     unsigned long long *recT;    // [K]
@@ -203,9 +200,9 @@ cudaError_t launch_rows_out(const GraphDev &g, const int32_t *pos, const int8_t 
 cudaError_t launch_rows_in(const GraphDev &g, const int8_t *raw, int8_t *rows, int32_t R, int32_t Rpad,
                            cudaStream_t st);
 cudaError_t launch_check(const int8_t *raw, size_t bytes, int32_t *bad, cudaStream_t st);
-// Minimum of the energies (and the step's start stamp), then weights + parents.
+// Minimum of the energies; the step's start stamp, weights and parents.
 cudaError_t launch_rs_min(const ResampleArgs &a, cudaStream_t st);
-cudaError_t launch_rs_rest(const ResampleArgs &a, cudaStream_t st);
+cudaError_t launch_rs_step(const ResampleArgs &a, cudaStream_t st);
 cudaError_t launch_stamp(unsigned long long *stamp, cudaStream_t st);
 
 struct SweepConfig {

@@ -54,7 +54,7 @@ struct AdaptArgs {
     double rhoR, delta;
     const double *qpow;            // [2^J][32]: row dn-1 = squarings of exp(-dn delta)
     double *part;                  // [J+1][2][nch] chunk tree sums of w and w*w
-    int32_t *state;                // [0] = n_prev, [1] = current level (mode 2)
+    int32_t *state;                // [0] = n_prev, [1] = current level (mode 2), [3] = CTAs done (mode 1)
     int32_t *qsel, *active, *tidx, *jsel;
     double *beta;
     int32_t mode;                  // 1 ESS rule, 2 acceptance-rate rule

@@ -46,16 +46,16 @@ __global__ void __launch_bounds__(pa::CL_THREADS) k_resample_noalloc(const int32
         e[i] = r0 + i < R ? E[r0 + i] : 0x7FFFFFFF;
         mn = min(mn, e[i]);
     }
-    pa::cluster_table(sh, qp);
+    pa::cluster_table(sh, qp.v);
     const int32_t emin = pa::cluster_min(sh, mn);
     double w[K];
     unsigned long long t[K];
 #pragma unroll
     for (int i = 0; i < K; ++i) {
-        w[i] = r0 + i < R ? pa::cluster_weight(sh, qp, (uint32_t)(e[i] - emin)) : 0.0;
+        w[i] = r0 + i < R ? pa::cluster_weight(sh, qp.v, (uint32_t)(e[i] - emin)) : 0.0;
         t[i] = (unsigned long long)__dmul_rn(w[i], 4294967296.0);
     }
-    unsigned long long P = pa::cluster_sums<K>(sh, w, t);
+    unsigned long long P = pa::cluster_sums<pa::CL_THREADS, K>(sh, w, t);
     const unsigned long long T = sh.T, m = ~0ull / T;
     const uint32_t o = pa::philox10(make_uint4(0u, 0u, k, pa::TAG_RESAMPLE), key0, key1).x;
     int32_t lo = pa::systematic_count_m(P, R, T, m, o);
@@ -65,8 +65,8 @@ __global__ void __launch_bounds__(pa::CL_THREADS) k_resample_noalloc(const int32
         const int32_t hi = pa::systematic_count_m(P, R, T, m, o);
         if (r0 + i < R) {
             if (counts) counts[r0 + i] = hi - lo;
-            for (int q = lo; q < hi; ++q) parent[q] = r0 + i;
         }
+        pa::fill_parents(parent, lo, r0 + i < R ? hi : lo, r0 + i);
         lo = hi;
     }
     if (r0 == 0) {
@@ -116,9 +116,9 @@ extern "C" int pa_resample_noalloc(const int32_t *energies, int32_t R, double be
         qp.v[b] = sq;
         sq = sq * sq;
     }
-    const pa::ClusterShape shape = pa::cluster_shape(R);
+    const pa::ClusterShape shape = pa::cluster_shape(R, pa::CL_THREADS);
     auto *kernel = shape.k == 1 ? &k_resample_noalloc<1> : shape.k == 2 ? &k_resample_noalloc<2> : &k_resample_noalloc<4>;
-    if (pa::launch_cluster(kernel, shape, st, energies, R, qp, (uint32_t)seed, (uint32_t)(seed >> 32), (uint32_t)k, parent,
+    if (pa::launch_cluster(kernel, shape, pa::CL_THREADS, st, energies, R, qp, (uint32_t)seed, (uint32_t)(seed >> 32), (uint32_t)k, parent,
                            counts, result) != cudaSuccess) {
         cudaGetLastError();
         return PA_ECUDA;

@@ -91,16 +91,16 @@ __global__ void __launch_bounds__(pa::CL_THREADS) k_shard_partials(const int32_t
     namespace cg = cooperative_groups;
     __shared__ pa::ClusterShared sh;
     const int r0 = ((int)cg::this_cluster().block_rank() * pa::CL_THREADS + (int)threadIdx.x) * K;
-    pa::cluster_table(sh, qp);
+    pa::cluster_table(sh, qp.v);
     __syncthreads();
     double w[K];
     unsigned long long t[K];
 #pragma unroll
     for (int i = 0; i < K; ++i) {
-        w[i] = r0 + i < n ? pa::cluster_weight(sh, qp, (uint32_t)(E[r0 + i] - emin)) : 0.0;
+        w[i] = r0 + i < n ? pa::cluster_weight(sh, qp.v, (uint32_t)(E[r0 + i] - emin)) : 0.0;
         t[i] = (unsigned long long)__dmul_rn(w[i], 4294967296.0);
     }
-    unsigned long long P = pa::cluster_sums<K>(sh, w, t);
+    unsigned long long P = pa::cluster_sums<pa::CL_THREADS, K>(sh, w, t);
 #pragma unroll
     for (int i = 0; i < K; ++i) {
         if (r0 + i < n) {
@@ -223,12 +223,12 @@ int pa_shard_partials(const int32_t *energies, int32_t n, int32_t emin, double b
         sq = sq * sq;
     }
     const ShardScratch s = scratch_view(scratch, n);
-    const pa::ClusterShape shape = pa::cluster_shape(n);
+    const pa::ClusterShape shape = pa::cluster_shape(n, pa::CL_THREADS);
     auto *kernel = shape.k == 1   ? &k_shard_partials<1>
                    : shape.k == 2 ? &k_shard_partials<2>
                    : shape.k == 4 ? &k_shard_partials<4>
                                   : &k_shard_partials<8>;
-    if (pa::launch_cluster(kernel, shape, st, energies, n, emin, qp, s) != cudaSuccess) {
+    if (pa::launch_cluster(kernel, shape, pa::CL_THREADS, st, energies, n, emin, qp, s) != cudaSuccess) {
         cudaGetLastError();
         return PA_ECUDA;
     }
