@@ -1137,6 +1137,18 @@ __device__ __forceinline__ uint32_t lop3(uint32_t a, uint32_t b, uint32_t c) {
 }
 constexpr int L_MAJ = 0xE8, L_XOR = 0x96, L_SEL = 0xCA;   // a b + b c + c a; a ^ b ^ c; a ? b : c
 
+// philox10 with the round keys of the kernel arguments.
+__device__ __forceinline__ uint4 philox10_keys(uint4 c, const uint32_t (&rk0)[10], const uint32_t (&rk1)[10]) {
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        uint32_t lo0, hi0, lo1, hi1;
+        mul_wide(0xD2511F53u, c.x, lo0, hi0);
+        mul_wide(0xCD9E8D57u, c.z, lo1, hi1);
+        c = make_uint4(hi1 ^ c.y ^ rk0[r], lo1, hi0 ^ c.w ^ rk1[r], lo0);
+    }
+    return c;
+}
+
 // Full adder of the planes a, b, c: returns the carry, a becomes the sum.
 __device__ __forceinline__ uint32_t msc_fa(uint32_t &a, uint32_t b, uint32_t c) {
     const uint32_t k = lop3<L_MAJ>(a, b, c);
@@ -1489,7 +1501,9 @@ __device__ __forceinline__ void msc_drain_ties(const SweepArgs &a, const uint32_
             for (int b = 0; b < N - 1; ++b) e |= ((q[3 + b] >> bit) & 1u) << b;
             const int m = 2 * (int)e + 2 - odd;
             const int rep = 4 * (bit & 7) + (bit >> 3);
-            if (sweep_tail_bits(vid, 32u * blk + rep, (uint32_t)a.k, c3, a.key0, a.key1) < (Tt[m] & 0xFFFFFFu)) {
+            const uint4 u = philox10_keys(make_uint4(vid, (32u * blk + rep) >> 2, (uint32_t)a.k, TAG_TAIL | c3), a.rk0,
+                                          a.rk1);
+            if ((word_of(u, rep & 3u) >> 8) < (Tt[m] & 0xFFFFFFu)) {
                 W.flip(p, 1u << bit);
                 atomicAdd(&Eacc[rep], 2 * m);
                 nacc += (vmask >> bit) & 1u;
