@@ -148,11 +148,14 @@ __global__ void __launch_bounds__(256) k_nlm_pair(NlmArgs a, const int32_t *orde
     const int gl = tid & (G - 1), grp = tid / G, NG = NT / G;
     const int m = blockIdx.x;
     const int sa = order[2 * m], sb = order[2 * m + 1];
-    int8_t *ga = a.spins + (size_t)sa * np;
+    int8_t *ga = a.spins + (size_t)sa * np;   // int8 rows; layouts without fields have bit rows
     int8_t *gb = a.spins + (size_t)sb * np;
+    uint32_t *wa = reinterpret_cast<uint32_t *>(a.spins) + (size_t)sa * a.g.nbw;
+    uint32_t *wb = reinterpret_cast<uint32_t *>(a.spins) + (size_t)sb * a.g.nbw;
     int nd_part = 0;
     for (int w = tid; w < nw; w += NT) {
-        const uint32_t xa = nlm_row_bits(ga, w, np), xb = nlm_row_bits(gb, w, np);
+        const uint32_t xa = a.fields ? nlm_row_bits(ga, w, np) : wa[w];
+        const uint32_t xb = a.fields ? nlm_row_bits(gb, w, np) : wb[w];
         const int rem = n - 32 * w;   // positions of this word below n
         const uint32_t live = rem >= 32 ? 0xFFFFFFFFu : (rem <= 0 ? 0u : (1u << rem) - 1u);
         Sa[w] = xa;
@@ -249,6 +252,11 @@ __global__ void __launch_bounds__(256) k_nlm_pair(NlmArgs a, const int32_t *orde
         const uint32_t c = D[w] & ~cand[w];
         if (!c) continue;
         Sa[w] ^= c;
+        if (!a.fields) {
+            wa[w] ^= c;
+            wb[w] ^= c;
+            continue;
+        }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int p0 = 32 * w + 16 * h;
@@ -358,9 +366,23 @@ __global__ void __launch_bounds__(256) k_nlm_block(NlmArgs a) {
     const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31;
     const int r = blockIdx.x;
     {
-        const uint4 *gx = reinterpret_cast<const uint4 *>(a.spins + (size_t)r * np);
         uint4 *lx = reinterpret_cast<uint4 *>(x);
-        for (int i = tid; i < (np >> 4); i += NT) lx[i] = gx[i];
+        if (a.fields) {
+            const uint4 *gx = reinterpret_cast<const uint4 *>(a.spins + (size_t)r * np);
+            for (int i = tid; i < (np >> 4); i += NT) lx[i] = gx[i];
+        } else {   // bit row: 16 bits to 16 spin bytes (positions past n are never read)
+            const uint16_t *gb = reinterpret_cast<const uint16_t *>(reinterpret_cast<const uint32_t *>(a.spins) + (size_t)r * a.g.nbw);
+            for (int i = tid; i < (np >> 4); i += NT) {
+                const uint32_t b = gb[i];
+                uint32_t v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t d = (((b >> (4 * q)) & 0xFu) * 0x00204081u) & 0x01010101u;
+                    v[q] = ~(d * 0xFEu);   // 0x01 or 0xFF
+                }
+                lx[i] = make_uint4(v[0], v[1], v[2], v[3]);
+            }
+        }
         for (int i = tid; i < nw; i += NT) {
             inB[i] = 0u;
             aff[i] = 0u;
@@ -438,7 +460,12 @@ __global__ void __launch_bounds__(256) k_nlm_block(NlmArgs a) {
     __syncthreads();
     if (!sh_acc) return;
     int8_t *gx = a.spins + (size_t)r * np;
-    for (int t = tid; t < cnt; t += NT) {
+    if (!a.fields) {   // bit row: the block's positions are the bits of inB
+        uint32_t *gw = reinterpret_cast<uint32_t *>(a.spins) + (size_t)r * a.g.nbw;
+        for (int w = tid; w < nw; w += NT)
+            if (inB[w]) gw[w] ^= inB[w];
+    }
+    for (int t = tid; a.fields && t < cnt; t += NT) {
         const int p = Bl[t];
         const int8_t v = (int8_t)-x[p];
         x[p] = v;

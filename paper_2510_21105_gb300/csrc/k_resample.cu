@@ -152,35 +152,52 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_step(ResampleArgs a) {
 // 16 ms each way.
 constexpr int ROWS_THREADS = 256;
 
-__global__ void __launch_bounds__(ROWS_THREADS) k_rows_out(int32_t n, int32_t np, const int32_t *__restrict__ pos,
+template <bool BITS>
+__global__ void __launch_bounds__(ROWS_THREADS) k_rows_out(int32_t n, int32_t np, int32_t nbw,
+                                                           const int32_t *__restrict__ pos,
                                                            const int8_t *__restrict__ rows, int8_t *__restrict__ raw) {
-    extern __shared__ __align__(16) int8_t x[];   // [np]
-    const uint4 *row = reinterpret_cast<const uint4 *>(rows + (size_t)blockIdx.x * np);
-    for (int i = threadIdx.x; i < (np >> 4); i += ROWS_THREADS) reinterpret_cast<uint4 *>(x)[i] = row[i];
+    extern __shared__ __align__(16) int8_t x[];   // the row: [np] bytes or [nbw] words
+    const uint32_t *xw = reinterpret_cast<const uint32_t *>(x);
+    const int units = BITS ? nbw >> 2 : np >> 4;
+    const uint4 *row = reinterpret_cast<const uint4 *>(rows) + (size_t)blockIdx.x * units;
+    for (int i = threadIdx.x; i < units; i += ROWS_THREADS) reinterpret_cast<uint4 *>(x)[i] = row[i];
     __syncthreads();
+    auto spin = [&](int p) {
+        return BITS ? (uint8_t)((xw[p >> 5] >> (p & 31)) & 1u ? 0x01 : 0xFF) : (uint8_t)x[p];
+    };
     int8_t *out = raw + (size_t)blockIdx.x * n;
     // Rows start at any byte: whole words at word boundaries, bytes at the ends.
     const int head = min(n, (int)((4 - (reinterpret_cast<uintptr_t>(out) & 3)) & 3)), words = (n - head) >> 2;
     for (int c = threadIdx.x; c < words; c += ROWS_THREADS) {
         uint32_t v = 0u;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) v |= (uint32_t)(uint8_t)x[__ldg(&pos[head + 4 * c + j])] << (8 * j);
+        for (int j = 0; j < 4; ++j) v |= (uint32_t)spin(__ldg(&pos[head + 4 * c + j])) << (8 * j);
         *reinterpret_cast<uint32_t *>(out + head + 4 * c) = v;
     }
     const int rest = n - 4 * words;   // head and tail bytes
     for (int t = threadIdx.x; t < rest; t += ROWS_THREADS) {
         const int i = t < head ? t : 4 * words + t;
-        out[i] = x[__ldg(&pos[i])];
+        out[i] = (int8_t)spin(__ldg(&pos[i]));
     }
 }
 
-__global__ void __launch_bounds__(ROWS_THREADS) k_rows_in(int32_t n, int32_t np, const uint32_t *__restrict__ vid,
+template <bool BITS>
+__global__ void __launch_bounds__(ROWS_THREADS) k_rows_in(int32_t n, int32_t np, int32_t nbw,
+                                                          const uint32_t *__restrict__ vid,
                                                           const int8_t *__restrict__ raw, int8_t *__restrict__ rows,
                                                           int32_t R) {
     extern __shared__ __align__(16) int8_t x[];   // [n]
     const int8_t *in = raw + (size_t)min((int)blockIdx.x, R - 1) * n;
     for (int i = threadIdx.x; i < n; i += ROWS_THREADS) x[i] = in[i];
     __syncthreads();
+    if (BITS) {
+        uint32_t *out = reinterpret_cast<uint32_t *>(rows) + (size_t)blockIdx.x * nbw;
+        for (int p = threadIdx.x; p < 32 * nbw; p += ROWS_THREADS) {   // whole warps
+            const uint32_t w = __ballot_sync(0xFFFFFFFFu, p < n && x[__ldg(&vid[min(p, n - 1)])] == 1);
+            if ((p & 31) == 0) out[p >> 5] = w;
+        }
+        return;
+    }
     uint32_t *out = reinterpret_cast<uint32_t *>(rows + (size_t)blockIdx.x * np);
     for (int c = threadIdx.x; c < (np >> 2); c += ROWS_THREADS) {
         uint32_t v = 0u;
@@ -220,17 +237,19 @@ cudaError_t allow_row(const void *fn, int32_t np) {
 }
 }  // namespace
 
-cudaError_t launch_rows_out(const GraphDev &g, const int32_t *pos, const int8_t *rows, int8_t *raw, int32_t R,
-                            cudaStream_t st) {
-    if (cudaError_t e = allow_row(reinterpret_cast<const void *>(&k_rows_out), g.np)) return e;
-    k_rows_out<<<R, ROWS_THREADS, g.np, st>>>(g.n, g.np, pos, rows, raw);
+cudaError_t launch_rows_out(const GraphDev &g, const int32_t *pos, const int8_t *rows, bool bits, int8_t *raw,
+                            int32_t R, cudaStream_t st) {
+    auto *fn = bits ? &k_rows_out<true> : &k_rows_out<false>;
+    if (cudaError_t e = allow_row(reinterpret_cast<const void *>(fn), g.np)) return e;
+    fn<<<R, ROWS_THREADS, bits ? 4 * g.nbw : g.np, st>>>(g.n, g.np, g.nbw, pos, rows, raw);
     return cudaGetLastError();
 }
 
-cudaError_t launch_rows_in(const GraphDev &g, const int8_t *raw, int8_t *rows, int32_t R, int32_t Rpad,
+cudaError_t launch_rows_in(const GraphDev &g, const int8_t *raw, int8_t *rows, bool bits, int32_t R, int32_t Rpad,
                            cudaStream_t st) {
-    if (cudaError_t e = allow_row(reinterpret_cast<const void *>(&k_rows_in), g.np)) return e;
-    k_rows_in<<<Rpad, ROWS_THREADS, g.np, st>>>(g.n, g.np, g.vid, raw, rows, R);
+    auto *fn = bits ? &k_rows_in<true> : &k_rows_in<false>;
+    if (cudaError_t e = allow_row(reinterpret_cast<const void *>(fn), g.np)) return e;
+    fn<<<Rpad, ROWS_THREADS, g.np, st>>>(g.n, g.np, g.nbw, g.vid, raw, rows, R);
     return cudaGetLastError();
 }
 

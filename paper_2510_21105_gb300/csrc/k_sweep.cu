@@ -1025,47 +1025,46 @@ __device__ __forceinline__ int msc_bit(int r) {   // bit of replica r = 4g + q i
     return 8 * (r & 3) + (r >> 2);
 }
 
-// Rows <-> bit words for 4 positions 4c .. 4c+3. A spin byte is 0x01 (+1) or
-// 0xFF (-1), 0 on padding. Load: per group g the four rows 4g + q give a word
-// y whose byte j holds, in bit q, replica 4g + q at position 4c + j; the
-// multiply by 0x00204081 spreads that nibble so that bit q lands on bit 8q
-// (the four shifted copies do not overlap, so nothing carries), and the shift
-// by g puts it on bit 8q + g of the position's word. Store: the inverse, with
-// byte j of the row word = 0x01 or 0xFF from the spread bit d (0xFF ^ 0xFE d)
-// and 0 on padding positions.
-__device__ __forceinline__ void msc_pack_rows(const int8_t *spins_in, const int32_t *PS, int np, int c,
-                                              uint32_t (&w4)[4]) {
+// 32 x 32 bit transpose over a warp: bit b of lane l goes to bit l of lane b.
+__device__ __forceinline__ uint32_t msc_transpose32(uint32_t x, int lane) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) w4[j] = 0u;
+    for (int s = 16; s; s >>= 1) {
+        const uint32_t m = 0xFFFFFFFFu / ((1u << s) + 1u);   // bits b with (b & s) == 0
+        const bool hi = lane & s;
+        const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x, s);
+        const uint32_t keep = hi ? ~m : m, rot = __funnelshift_l(y, y, hi ? 32 - s : s);
+        x = (keep & x) | (~keep & rot);
+    }
+    return x;
+}
+
+// Bit rows <-> words: a warp takes 128 positions of the word's 32 replicas, lane
+// l the row of the replica at bit l (msc_bit), 16 bytes of it, and transposes
+// them. Against int8 rows (32 loads and about 800 instructions per 4 positions
+// of a thread and step) a step without sweeps went from 50 to 22 us (G63-
+// shaped, R = 16384) and from 167 to 48 us (torus, R = 32768).
+__device__ __forceinline__ int msc_lane_replica(int lane) { return 4 * (lane & 7) + (lane >> 3); }
+
+// row: this lane's row; group of 128 positions q.
+__device__ __forceinline__ void msc_load_words(const uint32_t *row, uint32_t *Wsm, int np, int q, int lane) {
+    const uint4 v = __ldg(reinterpret_cast<const uint4 *>(row) + q);
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int g = 0; g < 8; ++g) {
-        uint32_t y = 0u;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t v = __ldg(reinterpret_cast<const uint32_t *>(spins_in + (size_t)PS[4 * g + q] * np + 4 * c));
-            y |= (v & ~(v >> 1) & 0x01010101u) << q;   // bit 0 of each byte set and bit 1 clear: +1
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) w4[j] |= ((((y >> (8 * j)) & 0xFu) * 0x00204081u) & 0x01010101u) << g;
+    for (int j = 0; j < 4; ++j) {
+        const uint32_t t = msc_transpose32(w[j], lane);
+        const int p = 128 * q + 32 * j + lane;
+        if (p < np) Wsm[p] = t;
     }
 }
 
-__device__ __forceinline__ void msc_unpack_rows(const uint32_t (&w4)[4], int8_t *spins_out, int slot0, int np, int n,
-                                                int c) {
-    uint32_t real = 0u;
+__device__ __forceinline__ void msc_store_words(const uint32_t *Wsm, uint32_t *row, int np, int q, int lane) {
+    uint32_t w[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) real |= (4 * c + j < n ? 0xFFu : 0u) << (8 * j);
-#pragma unroll
-    for (int g = 0; g < 8; ++g) {
-        uint32_t e = 0u;   // byte q, bit j: replica 4g + q at position 4c + j
-#pragma unroll
-        for (int j = 0; j < 4; ++j) e |= ((w4[j] >> g) & 0x01010101u) << j;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t d = (((e >> (8 * q)) & 0xFu) * 0x00204081u) & 0x01010101u;
-            *reinterpret_cast<uint32_t *>(spins_out + (size_t)(slot0 + 4 * g + q) * np + 4 * c) = ~(d * 0xFEu) & real;
-        }
+    for (int j = 0; j < 4; ++j) {
+        const int p = 128 * q + 32 * j + lane;
+        w[j] = msc_transpose32(p < np ? Wsm[p] : 0u, lane);
     }
+    reinterpret_cast<uint4 *>(row)[q] = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
 // Philox4x32-10 for the counters (c0, c1_g, c2, c3) of one item, which differ
@@ -1589,12 +1588,10 @@ __global__ void __launch_bounds__(256, 4) k_sweep_msc(const SweepArgs a) {
         }
         __syncthreads();
         if (tid < 32 && rank == 0) Eacc[tid] = a.E_in[PS[tid]];
-        // Load: 32 int8 spin rows -> one bit word per position.
-        for (int c = tid; c < (np >> 2); c += NT) {
-            uint32_t w4[4];
-            msc_pack_rows(a.spins_in, PS, np, c, w4);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) Wsm[4 * c + j] = w4[j];
+        {   // bit rows of the parents -> one word per position
+            const uint32_t *row = reinterpret_cast<const uint32_t *>(a.spins_in) +
+                                  (size_t)PS[msc_lane_replica(lane)] * a.g.nbw;
+            for (int q = warp; 4 * q < a.g.nbw; q += NT / 32) msc_load_words(row, Wsm, np, q, lane);
         }
         barrier();   // all copies loaded, energies in place
         const MscLevels L{misc[6], misc[7]};
@@ -1706,13 +1703,11 @@ __global__ void __launch_bounds__(256, 4) k_sweep_msc(const SweepArgs a) {
             }
             if (CL) barrier();   // the copy reads CTA 0's words before the next sweep changes them
         }
-        // Store: bit words -> int8 spin rows (fields are not kept by this
-        // layout); the CTAs of a cluster share the columns.
-        for (int c = csize * tid + rank; c < (np >> 2); c += csize * NT) {
-            uint32_t w4[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) w4[j] = Wsm[4 * c + j];
-            msc_unpack_rows(w4, a.spins_out, slot0, np, n, c);
+        {   // words -> bit rows; the CTAs of a cluster share the columns
+            uint32_t *row = reinterpret_cast<uint32_t *>(a.spins_out) +
+                            (size_t)(slot0 + msc_lane_replica(lane)) * a.g.nbw;
+            for (int q = warp * csize + rank; 4 * q < a.g.nbw; q += (NT / 32) * csize)
+                msc_store_words(Wsm, row, np, q, lane);
         }
         if (rank == 0) {
             if (warp == 0) {
@@ -1733,8 +1728,8 @@ __global__ void __launch_bounds__(256, 4) k_sweep_msc(const SweepArgs a) {
 // position are counted as in the sweep (7 planes for any degree) and summed in
 // bit-sliced accumulators; E = (stored entries / 2) - sum of the counts. SRC:
 //   WORDS_INIT  spins of the initial population: +1 iff bit 31 of its Philox
-//               word is set; written to the population rows
-//   WORDS_POP   rows of a population (position order, np bytes)
+//               word is set; written to the population's bit rows
+//   WORDS_POP   bit rows of a population
 //   WORDS_RAW   configurations in vertex order (n bytes each, any alignment);
 //               a byte other than +1 / -1 sets *bad
 // Against a byte per neighbour and replica from global memory the rows are read
@@ -1776,26 +1771,28 @@ __global__ void __launch_bounds__(256, 3) k_word_energy(GraphDev g, const int8_t
         }
         if (wrong) *bad = 1;
     } else {
-        for (int c = tid; c < (g.np >> 2); c += NT) {
-            uint32_t w4[4];
+        uint32_t *row = reinterpret_cast<uint32_t *>(rows) + (size_t)(slot0 + msc_lane_replica(lane)) * g.nbw;
+        for (int q = warp; 4 * q < g.nbw; q += NT / 32) {
             if (SRC == WORDS_POP) {
-                msc_pack_rows(in, PS, g.np, c, w4);
-            } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    w4[j] = 0u;
-                    if (4 * c + j >= g.n) continue;
-                    const uint32_t vid = __ldg(&g.vid[4 * c + j]);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const uint4 u = philox10(make_uint4(vid, (uint32_t)(slot0 >> 2) + q, 0u, TAG_INIT), key0, key1);
-                        w4[j] |= ((u.x >> 31) | (u.y >> 31) << 8 | (u.z >> 31) << 16 | (u.w >> 31) << 24) << q;
-                    }
-                }
-                msc_unpack_rows(w4, rows, slot0, g.np, g.n, c);
+                msc_load_words(row, Wsm, g.np, q, lane);
+                continue;
             }
 #pragma unroll
-            for (int j = 0; j < 4; ++j) Wsm[4 * c + j] = w4[j];
+            for (int j = 0; j < 4; ++j) {
+                const int p = 128 * q + 32 * j + lane;
+                uint32_t w = 0u;
+                if (p < g.n) {
+                    const uint32_t vid = __ldg(&g.vid[p]);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const uint4 u = philox10(make_uint4(vid, (uint32_t)(slot0 >> 2) + i, 0u, TAG_INIT), key0, key1);
+                        w |= ((u.x >> 31) | (u.y >> 31) << 8 | (u.z >> 31) << 16 | (u.w >> 31) << 24) << i;
+                    }
+                }
+                if (p < g.np) Wsm[p] = w;
+            }
+            __syncwarp();
+            msc_store_words(Wsm, row, g.np, q, lane);
         }
     }
     __syncthreads();
@@ -2052,7 +2049,7 @@ cudaError_t launch_init_words(const GraphDev &g, int8_t *spins, int32_t *E, int3
 }
 
 cudaError_t launch_energy_words(const GraphDev &g, const int8_t *spins, int32_t *E, int32_t Rpad, cudaStream_t st) {
-    return launch_word_energy(WORDS_POP, g, spins, nullptr, nullptr, E, Rpad, Rpad / 32, 0u, 0u, nullptr, st);
+    return launch_word_energy(WORDS_POP, g, nullptr, nullptr, const_cast<int8_t *>(spins), E, Rpad, Rpad / 32, 0u, 0u, nullptr, st);
 }
 
 cudaError_t launch_energy_raw(const GraphDev &g, const int8_t *raw, const int32_t *pos, int32_t *E, int32_t R,

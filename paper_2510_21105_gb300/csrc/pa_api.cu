@@ -164,6 +164,7 @@ struct pa_ctx {
         g.ncol = ncol;
         g.mmax = maxdeg;
         g.m2 = m2;
+        g.nbw = ((np + 127) / 128) * 4;
         g.maxcls = maxcls;
         g.rp = d_rp.as<uint32_t>();
         g.col = d_col.as<uint16_t>();
@@ -734,8 +735,9 @@ int pa_anneal_begin(pa_ctx *c, const double *betas, int32_t K, int32_t R, int32_
     const size_t npR = (size_t)c->np * r.Rpad;
     const int32_t Kc = std::max(K, 1);
     const int32_t Sc = std::max(sweeps, 1);
-    // The multi-spin-coded layouts keep no fields.
-    bool ok = r.spins[0].alloc(npR, ST) && r.spins[1].alloc(npR, ST) &&
+    // The multi-spin-coded layouts keep bit rows and no fields.
+    const size_t row = msc ? 4 * (size_t)g.nbw : (size_t)c->np;
+    bool ok = r.spins[0].alloc(row * r.Rpad, ST) && r.spins[1].alloc(row * r.Rpad, ST) &&
               (msc || (r.fields[0].alloc(2 * npR, ST) && r.fields[1].alloc(2 * npR, ST))) && r.E[0].alloc(4 * (size_t)r.Rpad, ST) &&
               r.E[1].alloc(4 * (size_t)r.Rpad, ST) && r.parent.alloc(4 * (size_t)r.Rpad, ST) &&
               r.d_tables.alloc(4 * r.tables.size(), ST) && r.d_tidx.alloc(4 * (size_t)Kc, ST) &&
@@ -1053,6 +1055,20 @@ int pa_anneal(pa_ctx *c, const double *betas, int32_t K, int32_t R, int32_t swee
 }  // extern "C"
 
 namespace {
+// Population rows: bit rows in the multi-spin-coded layouts, else int8.
+bool bit_rows(const RunState &r) { return r.variant == PA_VARIANT_MSC || r.variant == PA_VARIANT_MSC_PAIR; }
+size_t row_bytes(const pa_ctx *c) { return bit_rows(c->run) ? 4 * (size_t)c->gdev().nbw : (size_t)c->np; }
+
+// Configurations in vertex order on their way to or from the host pass through
+// the buffer the next step will write, `chunk` of them at a time.
+struct RawRows {
+    int8_t *p;
+    int32_t chunk;
+    explicit RawRows(const pa_ctx *c)
+        : p(c->run.spins[1 - c->run.cur].as<int8_t>()),
+          chunk((int32_t)std::min<size_t>((size_t)c->run.R, row_bytes(c) * c->run.Rpad / c->n)) {}
+};
+
 // Lexicographic minimum of the per-block records; returns the block or -1.
 int best_block(pa_ctx *c, int4 *rec) {
     RunState &r = c->run;
@@ -1220,11 +1236,17 @@ int pa_get_state(pa_ctx *c, int8_t *spins, int32_t *energies) {
     RunState &r = c->run;
     if (!r.begun) return fail(c, PA_ESTATE, "no anneal");
     if (int rc = pa_sync(c)) return rc;
-    if (spins) {   // vertex order, through the buffer the next step will write
-        int8_t *raw = r.spins[1 - r.cur].as<int8_t>();
-        PA_CUDA(c, pa::launch_rows_out(c->gdev(), c->d_pos.as<int32_t>(), r.spins[r.cur].as<int8_t>(), raw, r.R,
-                                       c->stream()));
-        PA_CUDA(c, copy(c, spins, raw, (size_t)r.R * c->n, cudaMemcpyDeviceToHost, c->stream(), true));
+    if (spins) {   // vertex order, some rows at a time
+        const RawRows raw(c);
+        const bool bits = bit_rows(r);
+        for (int32_t s0 = 0; s0 < r.R; s0 += raw.chunk) {
+            const int32_t cnt = std::min(raw.chunk, r.R - s0);
+            PA_CUDA(c, pa::launch_rows_out(c->gdev(), c->d_pos.as<int32_t>(),
+                                           r.spins[r.cur].as<int8_t>() + row_bytes(c) * s0, bits, raw.p,
+                                           cnt, c->stream()));
+            PA_CUDA(c, copy(c, spins + (size_t)s0 * c->n, raw.p, (size_t)cnt * c->n, cudaMemcpyDeviceToHost,
+                            c->stream(), true));
+        }
         PA_CUDA(c, cudaStreamSynchronize(c->stream()));
     }
     if (energies)
@@ -1238,21 +1260,32 @@ int pa_set_state(pa_ctx *c, const int8_t *spins, int32_t steps_done) {
     if (!r.begun) return fail(c, PA_ESTATE, "pa_anneal_begin has not run");
     if (steps_done < 0 || steps_done > r.K) return fail(c, PA_EINVAL, "steps_done out of range");
     if (int rc = pa_sync(c)) return rc;
-    // The configurations go to the buffer the next step will write, are checked
-    // there, and only then replace the population.
+    // All configurations are checked before any replaces a row of the population.
     cudaStream_t st = c->stream();
     const pa::GraphDev g = c->gdev();
-    int8_t *raw = r.spins[1 - r.cur].as<int8_t>();
+    const RawRows raw(c);
     int32_t *bad = r.parent.as<int32_t>();   // written by the next step before it is read
     int32_t wrong = 0;
-    PA_CUDA(c, copy(c, raw, spins, (size_t)r.R * c->n, cudaMemcpyHostToDevice, st, true));
     PA_CUDA(c, cudaMemsetAsync(bad, 0, 4, st));
-    PA_CUDA(c, pa::launch_check(raw, (size_t)r.R * c->n, bad, st));
-    PA_CUDA(c, cudaMemcpyAsync(&wrong, bad, 4, cudaMemcpyDeviceToHost, st));
-    PA_CUDA(c, cudaStreamSynchronize(st));
-    if (wrong) return fail(c, PA_EINVAL, "spins must be +1/-1");
-    PA_CUDA(c, pa::launch_rows_in(g, raw, r.spins[r.cur].as<int8_t>(), r.R, r.Rpad, st));
-    if (r.variant == PA_VARIANT_MSC || r.variant == PA_VARIANT_MSC_PAIR)
+    for (int pass = 0; pass < 2; ++pass) {   // check, then take over
+        for (int32_t s0 = 0; s0 < r.R; s0 += raw.chunk) {
+            const int32_t cnt = std::min(raw.chunk, r.R - s0);
+            if (pass == 0 || raw.chunk < r.R)   // one chunk: it is still there
+                PA_CUDA(c, copy(c, raw.p, spins + (size_t)s0 * c->n, (size_t)cnt * c->n, cudaMemcpyHostToDevice, st,
+                                true));
+            if (pass == 0)
+                PA_CUDA(c, pa::launch_check(raw.p, (size_t)cnt * c->n, bad, st));
+            else
+                PA_CUDA(c, pa::launch_rows_in(g, raw.p, r.spins[r.cur].as<int8_t>() + row_bytes(c) * s0,
+                                              bit_rows(r), cnt, s0 + cnt == r.R ? r.Rpad - s0 : cnt, st));
+        }
+        if (pass == 0) {
+            PA_CUDA(c, cudaMemcpyAsync(&wrong, bad, 4, cudaMemcpyDeviceToHost, st));
+            PA_CUDA(c, cudaStreamSynchronize(st));
+            if (wrong) return fail(c, PA_EINVAL, "spins must be +1/-1");
+        }
+    }
+    if (bit_rows(r))
         PA_CUDA(c, pa::launch_energy_words(g, r.spins[r.cur].as<int8_t>(), r.E[r.cur].as<int32_t>(), r.Rpad, st));
     else
         PA_CUDA(c, pa::launch_fields(g, r.spins[r.cur].as<int8_t>(), r.fields[r.cur].as<int16_t>(),
@@ -1290,7 +1323,7 @@ int pa_energies(pa_ctx *c, const int8_t *spins, int32_t R, int32_t *energies, in
         PA_CUDA(c, pa::launch_energy_raw(g, dx.as<int8_t>(), c->d_pos.as<int32_t>(), dE.as<int32_t>(), R, bad, st));
     } else {
         PA_CUDA(c, pa::launch_check(dx.as<int8_t>(), raw, bad, st));
-        PA_CUDA(c, pa::launch_rows_in(g, dx.as<int8_t>(), dr.as<int8_t>(), R, R, st));
+        PA_CUDA(c, pa::launch_rows_in(g, dx.as<int8_t>(), dr.as<int8_t>(), false, R, R, st));
         PA_CUDA(c, pa::launch_fields(g, dr.as<int8_t>(), dh.as<int16_t>(), dE.as<int32_t>(), R, st));
     }
     PA_CUDA(c, copy(c, E.data(), dE.p, 4 * ((size_t)R + 1), cudaMemcpyDeviceToHost, st, true));

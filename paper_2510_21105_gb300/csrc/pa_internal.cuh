@@ -2,7 +2,9 @@
 //
 // Device layout of one anneal (vertices renumbered by colour; "position" p
 // is a vertex's index in that order, np = n rounded up to 16):
-//   spins  int8  [Rpad][np]   +1/-1, ping-pong pair (cur / next)
+//   spins  ping-pong pair (cur / next): int8 [Rpad][np], +1/-1, in the layouts
+//          with fields; bit rows uint32 [Rpad][nbw], bit p set for +1, in the
+//          multi-spin-coded ones (fields absent)
 //   fields int16 [Rpad][np]   h_p = sum_j w_pj x_j, ping-pong pair
 //   E      int32 [Rpad]       Ising energy of each replica, ping-pong pair
 //   parent int32 [Rpad]       new slot -> old slot of the current step
@@ -107,6 +109,7 @@ constexpr int RS_CHUNK = 256;                   // slots per CTA of the ESS part
 struct GraphDev {
     int32_t n, np, ncol, mmax, maxcls;   // maxcls: largest colour class
     int32_t m2;           // stored entries (twice the edges)
+    int32_t nbw;          // words of a bit row: np bits rounded up to 16 bytes
     const uint32_t *rp;   // [n+1] row pointers, position order
     const uint16_t *col;  // [2M] neighbour positions
     const int8_t *wt;     // [2M] weights or nullptr (all +1)
@@ -139,7 +142,7 @@ struct GraphDev {
 
 struct SweepArgs {
     GraphDev g;
-    const int8_t *spins_in;
+    const int8_t *spins_in;      // multi-spin coded: bit rows
     const int16_t *fields_in;
     const int32_t *E_in;
     int8_t *spins_out;
@@ -192,12 +195,13 @@ cudaError_t launch_init_words(const GraphDev &g, int8_t *spins, int32_t *E, int3
 cudaError_t launch_energy_words(const GraphDev &g, const int8_t *spins, int32_t *E, int32_t Rpad, cudaStream_t st);
 cudaError_t launch_energy_raw(const GraphDev &g, const int8_t *raw, const int32_t *pos, int32_t *E, int32_t R,
                               int32_t *bad, cudaStream_t st);
-// Population rows (position order, np bytes) <-> configurations in vertex order
-// (n bytes each): out writes R of them; in reads R of them into Rpad rows, the
-// padding rows repeating the last one; check sets *bad if a byte is not +1 / -1.
-cudaError_t launch_rows_out(const GraphDev &g, const int32_t *pos, const int8_t *rows, int8_t *raw, int32_t R,
-                            cudaStream_t st);
-cudaError_t launch_rows_in(const GraphDev &g, const int8_t *raw, int8_t *rows, int32_t R, int32_t Rpad,
+// Population rows (position order, np bytes or bit rows) <-> configurations in
+// vertex order (n bytes each): out writes R of them; in reads R of them into Rpad
+// rows, the padding rows repeating the last one; check sets *bad if a byte is
+// not +1 / -1.
+cudaError_t launch_rows_out(const GraphDev &g, const int32_t *pos, const int8_t *rows, bool bits, int8_t *raw,
+                            int32_t R, cudaStream_t st);
+cudaError_t launch_rows_in(const GraphDev &g, const int8_t *raw, int8_t *rows, bool bits, int32_t R, int32_t Rpad,
                            cudaStream_t st);
 cudaError_t launch_check(const int8_t *raw, size_t bytes, int32_t *bad, cudaStream_t st);
 // Minimum of the energies; the step's start stamp, weights and parents.
