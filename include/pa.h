@@ -59,14 +59,17 @@ typedef struct pa_ctx pa_ctx;
 #define PA_VARIANT_I8 0   /* int8 spins + int16/int8 local fields in shared memory */
 #define PA_VARIANT_MSC 1  /* multi-spin coded: 32 replicas per 32-bit word */
 #define PA_VARIANT_AUTO 2 /* chosen per graph and population: multi-spin coded
-                             when the 32-replica words give every SM a word,
-                             the CTA-pair kernel when they cover at least 40%
-                             of the SMs, else the first of the packed byte
-                             layout, int16 fields and multi-spin coding that
-                             fits the graph in shared memory */
-#define PA_VARIANT_MSC_PAIR 3 /* multi-spin coded, one thread-block cluster of two
-                                 CTAs per 32-replica word (distributed shared
-                                 memory); same results as PA_VARIANT_MSC */
+                             when the 32-replica words give every SM a word;
+                             with fewer words the cluster kernel when they cover
+                             at least 40% of the SMs or the graph's colour
+                             classes are large enough; else the first of the
+                             packed byte layout, int16 fields and multi-spin
+                             coding that fits the graph in shared memory */
+#define PA_VARIANT_MSC_PAIR 3 /* multi-spin coded, each 32-replica word spread
+                                 over a thread-block cluster of two to eight CTAs
+                                 (distributed shared memory) as far as the colour
+                                 classes keep them busy; same results as
+                                 PA_VARIANT_MSC */
 
 typedef struct {
     int32_t variant;          /* PA_VARIANT_*; default PA_VARIANT_AUTO */

@@ -1512,8 +1512,8 @@ __device__ __forceinline__ void msc_drain_ties(const SweepArgs &a, const uint32_
     __syncwarp();
 }
 
-// Sweeps of multi-spin-coded words. CL: a thread-block cluster of two CTAs
-// shares a word. Every CTA keeps a full copy of the word array; inside a
+// Sweeps of multi-spin-coded words. CL: a thread-block cluster (2, 4 or
+// 8 CTAs) shares a word. Every CTA keeps a full copy of the word array; inside a
 // colour class the CTAs take the positions in turns of 32, every changed word
 // is stored into all copies (the others' through distributed shared memory),
 // and a cluster barrier closes each class. The 32 energies live in CTA 0,
@@ -1918,8 +1918,32 @@ size_t sweep_smem_bytes(const GraphDev &g, int G, int field_bits, int threads) {
            (size_t)((g.ncol + 1 + 3) & ~3) * 4 + (size_t)(8 * G + 8) * 4;
 }
 
+// CTAs per word of the cluster kernel: as many as the largest class keeps busy
+// (eight warps each, rounded up) while all clusters stay resident at about 2.6
+// CTAs per SM. us per step of 4 sweeps with 2 / 4 / 8 CTAs: G63-shaped (largest
+// class 47 slices) R = 1024 147 / 121 / 118, R = 2048 148 / 139 / 144, R = 3072
+// 179 / 161 / 239, R = 4096 180 / 186 / 266; torus N = 10000 R = 1024 99 / 65 /
+// 65, R = 3072 138 / 115 / 148; 18,000-vertex planar (two CTAs per SM) R = 1024
+// 214 / 147 / 142, R = 1536 214 / 189 / 241. One CTA is better where a class fits
+// it: n = 2000, degree 12, R = 1024 82 against 90 / 92 / 98. With less than five
+// rounds in the largest class the cluster barriers only pay on idle SMs: N = 2500
+// torus (39 slices) R = 1024 44 / 31, R = 3072 44 / 51 with 1 / 2.
+int msc_cluster(const GraphDev &g, int words, int sms) {
+    int limit = 0, per_sm = 0, dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    const size_t smem = sweep_smem_bytes(g, 8, 2, 256);
+    const int resident = (int)std::min<size_t>(4, (size_t)per_sm / (smem + 1024));
+    limit = std::min(13 * sms / 5, resident * sms);
+    const int busy = (g.maxcls + 31) / 32 / 8;
+    if (busy < 5) limit = std::min(limit, sms);
+    int c = 1;
+    while (c < 8 && c < busy && 2 * c * words <= limit) c *= 2;
+    return c;
+}
+
 cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int threads,
-                            bool weighted, SweepConfig *cfg) {
+                            bool weighted, SweepConfig *cfg, int cluster) {
     int dev = 0, sms = 0, occ = 0, limit = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1946,8 +1970,12 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
         const int per = ((R + 4 * G - 1) / (4 * G) + sms - 1) / sms;
         threads = per <= 2 ? 512 : per <= 4 ? 256 : 128;
     }
+    if (field_bits == 2) {
+        if (!cluster) cluster = msc_cluster(g, (R + 31) / 32, sms);
+        if (cluster == 1) field_bits = 1;
+    }
     size_t smem = sweep_smem_bytes(g, G, field_bits, threads);
-    if (field_bits == 1 || field_bits == 2) {
+    if (msc) {
         // Tie queues: 64 entries per warp, 40 where 64 would cost a resident
         // block, and what the reserved words leave when the graph fills shared
         // memory.
@@ -1984,14 +2012,15 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
     if (cudaError_t e = raise_smem(fn, smem)) return e;
     const int nblk = (R + 4 * G - 1) / (4 * G);
     if (field_bits == 2) {
-        // One cluster of two CTAs per word; the hardware schedules them as slots free up.
+        // One cluster per word; the hardware schedules them as slots free up.
+        cfg->cluster = cluster;
         cudaLaunchConfig_t lc = {};
-        lc.gridDim = dim3(2 * nblk);
+        lc.gridDim = dim3(cfg->cluster * nblk);
         lc.blockDim = dim3(threads);
         lc.dynamicSmemBytes = smem;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 2;
+        at[0].val.clusterDim.x = cfg->cluster;
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         lc.attrs = at;
         lc.numAttrs = 1;
@@ -2003,7 +2032,7 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
         cfg->field_bits = field_bits;
         cfg->threads = threads;
         cfg->smem = smem;
-        cfg->grid = 2 * nblk;
+        cfg->grid = cfg->cluster * nblk;
         return cudaSuccess;
     }
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem);
@@ -2029,7 +2058,7 @@ cudaError_t launch_sweep(const SweepConfig &cfg, const SweepArgs &a, cudaStream_
     lc.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.x = cfg.cluster;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     lc.attrs = at;
     lc.numAttrs = cfg.field_bits == 2 ? 1 : 0;

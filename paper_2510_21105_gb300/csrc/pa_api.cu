@@ -594,19 +594,22 @@ int pa_anneal_begin(pa_ctx *c, const double *betas, int32_t K, int32_t R, int32_
     const bool packed_fits = c->maxdeg <= 127 && c->packed_ok && fits(7, 1, o.threads_per_cta ? o.threads_per_cta : 128);
     const bool int16_fits = fits(16, o.replicas_per_cta == 8 ? 2 : 1, 512);
     if (o.variant == PA_VARIANT_AUTO) {
-        // Multi-spin coding is fastest once its 32-replica words give every SM
-        // at least one block (the words past the largest SM multiple run in the
-        // CTA-pair kernel, see below). With fewer words, down to about 40% of
-        // the SM count, the CTA-pair kernel (two CTAs per word) still beats the
-        // 4-replica packed layout; below that the packed layout's smaller
-        // blocks win. Measured (G attempts/s, packed / MSC / MSC pair):
-        // G63-shaped R = 2048: 251 / 196 / 255; R = 4096: 357 / 388 / 413;
-        // R = 8192: 362 / 558 / 533; torus 100x100 R = 2048: 281 / 265 / 445.
+        // Multi-spin coding once its 32-replica words give every SM a block (the
+        // words past the largest SM multiple run in CTA pairs, see below). With
+        // fewer words each is spread over a cluster (msc_cluster); that beats the
+        // 4-replica packed layout from a number of words that falls with the
+        // slices of 32 positions in the largest class, which keep the CTAs busy.
+        // us per step of 4 sweeps, packed / multi-spin coded: 18,000-vertex planar
+        // (139 slices) R = 64 163 / 115, torus N = 4900 (77) R = 64 50 / 39; G63-
+        // shaped (47) R = 512 98 / 114, R = 768 143 / 117; n = 2000, degree 12 (14)
+        // R = 1024 70 / 82, R = 1536 77 / 82, R = 2048 91 / 82.
         const bool msc_ok = msc_fits && o.field_bits == 0 && (o.threads_per_cta == 0 || o.threads_per_cta <= 256);
-        const int32_t words = (R + 31) / 32;
+        const int32_t words = (R + 31) / 32, slices = (c->maxcls + 31) / 32;
+        const bool spread = 5 * words >= 2 * sms ||
+                            (packed_fits && words >= (slices >= 64 ? 1 : slices >= 24 ? 24 : slices >= 12 ? 48 : sms));
         if (msc_ok && words >= sms)
             o.variant = PA_VARIANT_MSC;
-        else if (msc_ok && 5 * words >= 2 * sms)
+        else if (msc_ok && spread)
             o.variant = PA_VARIANT_MSC_PAIR;
         else if ((o.field_bits == 0 || o.field_bits == 7) && packed_fits)
             o.variant = PA_VARIANT_I8;
@@ -673,7 +676,7 @@ int pa_anneal_begin(pa_ctx *c, const double *betas, int32_t K, int32_t R, int32_
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const int32_t words = r.nblk, wm = sms > 0 ? (words / sms) * sms : 0;
         if (wm > 0 && wm < words) {
-            ce = pa::sweep_configure(g, R - 32 * wm, 8, 2, 256, c->weighted, &r.sweep2);
+            ce = pa::sweep_configure(g, R - 32 * wm, 8, 2, 256, c->weighted, &r.sweep2, 2);
             if (ce != cudaSuccess) return cuda_fail(c, ce, "sweep_configure (tail)");
             ce = pa::sweep_configure(g, 32 * wm, 8, 1, threads, c->weighted, &r.sweep);
             if (ce != cudaSuccess) return cuda_fail(c, ce, "sweep_configure (head)");
