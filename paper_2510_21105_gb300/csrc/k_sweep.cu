@@ -2043,6 +2043,7 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
     cfg->threads = threads;
     cfg->smem = smem;
     cfg->grid = nblk < occ * sms ? nblk : occ * sms;
+    cfg->occ = occ;
     return cudaSuccess;
 }
 

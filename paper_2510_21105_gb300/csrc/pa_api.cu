@@ -269,6 +269,22 @@ void collect_events(RunState &r) {
     free_run_events(r);
 }
 
+// Whether the words past the largest SM multiple run in CTA pairs beside the
+// others. It evens out the last wave of blocks (occ per SM) where the rest fills
+// at most half of the SMs with pairs, and costs cluster barriers, which classes
+// of few slices cannot carry. us per step of 4 sweeps, pairs / all words in
+// one-CTA blocks, on 152 SMs: G63-shaped 200 words 206 / 236, 270 words 254 / 237,
+// 512 words 364 / 401, 560 words 439 / 400, 1024 words 710 / 787, 1200 words 838 /
+// 791; torus N = 10000 200 words 171 / 211, 620 words 434 / 474, 1024 words 729 /
+// 763; n = 2000, degree 12 (14 slices) 200 words 115 / 101, 512 words 164 / 157;
+// 18,000-vertex planar 200 words 362 / 451, 270 words 631 / 451.
+bool pair_tail(int32_t words, int sms, int occ, int32_t slices) {
+    const int32_t cap = occ * sms, rem = words % cap, q = rem / sms, r = rem % sms;
+    if (r == 0 || slices < 24 || words < sms) return false;
+    if (words < cap) return 2 * r <= sms;
+    return q == 0 ? 8 * r <= sms : q >= 2 && 4 * r <= 3 * sms;
+}
+
 int validate_opts(pa_ctx *c, const pa_anneal_opts &o) {
     if (o.variant < 0 || o.variant > 3) return fail(c, PA_EINVAL, "variant");
     if (o.field_bits != 16 && o.field_bits != 8 && o.field_bits != 7)
@@ -674,8 +690,8 @@ int pa_anneal_begin(pa_ctx *c, const double *betas, int32_t K, int32_t R, int32_
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int32_t words = r.nblk, wm = sms > 0 ? (words / sms) * sms : 0;
-        if (wm > 0 && wm < words) {
+        const int32_t words = r.nblk, wm = (words / sms) * sms;
+        if (pair_tail(words, sms, r.sweep.occ, (c->maxcls + 31) / 32)) {
             ce = pa::sweep_configure(g, R - 32 * wm, 8, 2, 256, c->weighted, &r.sweep2, 2);
             if (ce != cudaSuccess) return cuda_fail(c, ce, "sweep_configure (tail)");
             ce = pa::sweep_configure(g, 32 * wm, 8, 1, threads, c->weighted, &r.sweep);

@@ -217,6 +217,7 @@ struct SweepConfig {
     size_t smem;
     bool small = false;   // the small-graph kernel of the layout
     int cluster = 0;      // multi-spin coded in clusters: CTAs per word
+    int occ = 0;          // resident blocks per SM (no cluster)
     int qcap = 0;   // multi-spin coded: tie-queue entries per warp; other layouts: entries of the block's queue (0: none)
 };
 // Dynamic shared memory of one sweep CTA (G: 4-replica groups of the int8/int16 layouts;
