@@ -129,9 +129,9 @@ struct GraphDev {
     // A unit holds four bonds of each lane, lane after lane, so a warp reads it
     // in one contiguous piece and all lanes run the slice's largest unit count
     // (positions are sorted by degree). Entries are byte offsets of the
-    // neighbours' words (4 * position): 16 bits up to np = 16384, with the signs
-    // of entries 2j and 2j + 1 (weight -1) in bits 0 and 1 of entry 2j, else
-    // (mbig) 32 bits with the sign in bit 0. Padding entries point at the lane's
+    // neighbours' words (4 * position): 16 bits on signed graphs up to np = 16384,
+    // with the signs of entries 2j and 2j + 1 (weight -1) in bits 0 and 1 of entry
+    // 2j, else (mbig) 32 bits with the sign in bit 0. Padding entries point at the lane's
     // own position (its word XOR itself counts nothing).
     const uint2 *msl;
     const int32_t *csl;      // [ncol+1]
