@@ -4,8 +4,8 @@ Candidates are the kernel shapes the library offers: the spin encoding (packed
 byte of spin + 7-bit field, int8 spin + int8 or int16 field, multi-spin coded
 32 replicas per word), the replicas per CTA (4 or 8 for the int8/int16
 layouts) and the threads per CTA (the colour-block width: positions of one
-colour updated in parallel per pass; the multi-spin-coded kernels always run
-256 threads, which measured fastest against 192, 320 and 384). Each feasible
+colour updated in parallel per pass; the multi-spin-coded kernels choose 256
+or 512 threads themselves, by the CTAs that share an SM). Each feasible
 candidate anneals a
 short slice of the instance's own schedule (from its middle, where the
 acceptance rate is typical of most of a run) with per-launch CUDA-event

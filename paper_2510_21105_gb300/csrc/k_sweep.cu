@@ -1531,7 +1531,7 @@ __device__ __forceinline__ void msc_drain_ties(const SweepArgs &a, const uint32_
 // remotely. Halving the work unit lets the SMs balance the words that do not
 // divide over them.
 template <int N, bool WEIGHTED, bool BIG, bool CL>
-__global__ void __launch_bounds__(256, 4) k_sweep_msc(const SweepArgs a) {
+__global__ void __launch_bounds__(512, 2) k_sweep_msc(const SweepArgs a) {
     namespace cg = cooperative_groups;
     using Sh = MscShape<N>;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1547,7 +1547,7 @@ __global__ void __launch_bounds__(256, 4) k_sweep_msc(const SweepArgs a) {
     int32_t *Eacc = cls + csz;      // [32] (in a cluster: CTA 0's)
     int32_t *PS = Eacc + 32;        // [32]
     int32_t *misc = PS + 32;        // best E, step, sweep, slot, copy-from (r+1), changed, level bounds
-    constexpr int NT = 256;
+    const int NT = blockDim.x;   // 256 or 512
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     uint32_t *TQ = reinterpret_cast<uint32_t *>(misc + 8) + (size_t)warp * a.qcap * Sh::entry;   // this warp's tie queue
     int rank = 0, csize = 1;
@@ -1612,7 +1612,7 @@ __global__ void __launch_bounds__(256, 4) k_sweep_msc(const SweepArgs a) {
 #pragma unroll
         for (int b = 0; b < Sh::acc_planes; ++b) S[b] = 0u;
         int cnt = 0;   // items per lane in S
-        const int w0 = warp * csize + rank, nw = (NT / 32) * csize;
+        const int w0 = warp * csize + rank, nw = (NT >> 5) * csize;
         // Descriptor and vertices of the warp's next slice, read one slice ahead.
         uint2 d = make_uint2(0u, 0u);
         uint32_t vd = 0u;
@@ -1928,32 +1928,54 @@ size_t sweep_smem_bytes(const GraphDev &g, int G, int field_bits, int threads) {
            (size_t)((g.ncol + 1 + 3) & ~3) * 4 + (size_t)(8 * G + 8) * 4;
 }
 
+static size_t msc_fixed_bytes(const GraphDev &g) {
+    return ((size_t)g.np + msc_table_words(g.mmax) + 72 + ((g.ncol + 1 + 3) & ~3)) * 4;
+}
+
+// Threads of an MSC block: 512 where an SM would otherwise hold too few warps, 256
+// elsewhere and where a class has no more slices than eight warps. That is where
+// the launch has at most one CTA for an SM (us per step of 4 sweeps with 256 / 512
+// threads, 140 words of one CTA: G63-shaped 168 / 139, 100 x 100 torus 138 / 111,
+// n = 2000 83 / 74; 32 words in clusters of four: 112 / 100, 99 / 58 (the torus
+// with 8 slices per CTA 64 / 58), 18,000-vertex planar 137 / 120; five slices per
+// class, n = 3000 and degree 48, 140 words: 213 / 216) and where shared memory
+// holds at most two CTAs (140 x 140 torus, 18,000-vertex planar and n = 16,272 at
+// 64 to 512 words: 1.03 to 1.34 times faster; one CTA, n = 30,000: 1.28). With
+// three or four of 256 resident those win, the barrier after a class holds up
+// fewer warps (G63-shaped 500 words 376 / 427, 2048 words 1264 / 1475).
+static int msc_threads(const GraphDev &g, int ctas, int sms, int per_sm, int limit, bool clusters) {
+    const size_t fixed = msc_fixed_bytes(g), entry = (size_t)msc_entry_words(g.mmax) * 4;
+    auto fit = [&](int threads) { return (int)std::min<size_t>(1024 / threads, (size_t)per_sm / (fixed + 40 * entry * (threads / 32) + 1024)); };
+    if (g.maxcls <= 256 || fixed + 40 * entry * 16 > (size_t)limit) return 256;
+    const bool few = ctas <= sms || fit(256) <= (clusters ? 1 : 2);
+    return few && fit(512) >= std::min(fit(256), (ctas + sms - 1) / sms) ? 512 : 256;
+}
+
 // CTAs per word of the cluster kernel: as many as the largest class keeps busy
-// (eight warps each, rounded up) while all clusters stay resident at about 2.6
-// CTAs per SM. us per step of 4 sweeps with 2 / 4 / 8 CTAs: G63-shaped (largest
-// class 47 slices) R = 1024 147 / 121 / 118, R = 2048 148 / 139 / 144, R = 3072
-// 179 / 161 / 239, R = 4096 180 / 186 / 266; torus N = 10000 R = 1024 99 / 65 /
-// 65, R = 3072 138 / 115 / 148; 18,000-vertex planar (two CTAs per SM) R = 1024
-// 214 / 147 / 142, R = 1536 214 / 189 / 241. One CTA is better where a class fits
-// it: n = 2000, degree 12, R = 1024 82 against 90 / 92 / 98. With less than five
-// rounds in the largest class the cluster barriers only pay on idle SMs: N = 2500
-// torus (39 slices) R = 1024 44 / 31, R = 3072 44 / 51 with 1 / 2.
+// (eight warps each, rounded up) while each has an SM of its own. us per step of 4
+// sweeps with 1 / 2 / 4 / 8 CTAs of 512 threads: G63-shaped (largest class 47
+// slices) 14 words 138 / 120 / 99 / 98, 25 words 139 / 121 / 100 / 113, 70 words
+// 139 / 121 / 126 / 220; torus N = 10000 (157) 14 words 110 / 79 / 57 / 48, 32
+// words 111 / 79 / 58 / 72, 98 words 111 / 129 / 131 / -; 18,000-vertex planar
+// (139) 14 words 223 / 160 / 119 / 101, 98 words 224 / 255 / 269 / -. One CTA is
+// better where a class fits it: n = 2000, degree 12 (14), 14 words 74 / 85 / 87 /
+// 92. With a word and more for each SM, pairs of 256 threads still even out the
+// last wave where four fit an SM: torus N = 10000 170 words 207 / 183, G63-shaped
+// 220 / 203.
 int msc_cluster(const GraphDev &g, int words, int sms) {
-    int limit = 0, per_sm = 0, dev = 0;
+    int dev = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    const size_t smem = sweep_smem_bytes(g, 8, 2, 256);
-    const int resident = (int)std::min<size_t>(4, (size_t)per_sm / (smem + 1024));
-    limit = std::min(13 * sms / 5, resident * sms);
+    const int resident = (int)std::min<size_t>(4, (size_t)per_sm / (sweep_smem_bytes(g, 8, 2, 256) + 1024));
     const int busy = (g.maxcls + 31) / 32 / 8;
-    if (busy < 5) limit = std::min(limit, sms);
+    const int limit = words > sms && busy >= 5 ? std::min(13 * sms / 5, resident * sms) : sms;
     int c = 1;
     while (c < 8 && c < busy && 2 * c * words <= limit) c *= 2;
     return c;
 }
 
 cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int threads,
-                            bool weighted, SweepConfig *cfg, int cluster) {
+                            bool weighted, SweepConfig *cfg, int cluster, int all_words) {
     int dev = 0, sms = 0, occ = 0, limit = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1963,7 +1985,12 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
     bool small = false;
     if (msc) {
         G = 8;
-        threads = 256;
+        if (field_bits == 2) {
+            if (!cluster) cluster = msc_cluster(g, (R + 31) / 32, sms);
+            if (cluster == 1) field_bits = 1;
+        }
+        const int ctas = all_words ? all_words : (R + 31) / 32 * (field_bits == 2 ? cluster : 1);
+        threads = msc_threads(g, ctas, sms, per_sm, limit, field_bits == 2);
     } else if (field_bits == 7) {
         G = 1;
         // Few blocks: more threads each, so that an SM has about 1024 whatever the
@@ -1980,18 +2007,14 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
         const int per = ((R + 4 * G - 1) / (4 * G) + sms - 1) / sms;
         threads = per <= 2 ? 512 : per <= 4 ? 256 : 128;
     }
-    if (field_bits == 2) {
-        if (!cluster) cluster = msc_cluster(g, (R + 31) / 32, sms);
-        if (cluster == 1) field_bits = 1;
-    }
     size_t smem = sweep_smem_bytes(g, G, field_bits, threads);
     if (msc) {
         // Tie queues: 64 entries per warp, 40 where 64 would cost a resident
         // block, and what the reserved words leave when the graph fills shared
         // memory.
-        const size_t fixed = ((size_t)g.np + msc_table_words(g.mmax) + 72 + ((g.ncol + 1 + 3) & ~3)) * 4;
+        const size_t fixed = msc_fixed_bytes(g);
         const size_t per_entry = (size_t)(threads / 32) * msc_entry_words(g.mmax) * 4;
-        auto resident = [&](int cap) { return std::min<size_t>(4, (size_t)per_sm / (fixed + cap * per_entry + 1024)); };
+        auto resident = [&](int cap) { return std::min<size_t>(1024 / threads, (size_t)per_sm / (fixed + cap * per_entry + 1024)); };
         cfg->qcap = resident(64) < resident(40) ? 40 : 64;
         if (fixed + cfg->qcap * per_entry > (size_t)limit) cfg->qcap = (int)((smem - fixed) / per_entry);
         if (cfg->qcap < 1) return cudaErrorInvalidConfiguration;

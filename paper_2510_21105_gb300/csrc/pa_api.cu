@@ -273,11 +273,11 @@ void collect_events(RunState &r) {
 // others. It evens out the last wave of blocks (occ per SM) where the rest fills
 // at most half of the SMs with pairs, and costs cluster barriers, which classes
 // of few slices cannot carry. us per step of 4 sweeps, pairs / all words in
-// one-CTA blocks, on 152 SMs: G63-shaped 200 words 206 / 236, 270 words 254 / 237,
-// 512 words 364 / 401, 560 words 439 / 400, 1024 words 710 / 787, 1200 words 838 /
-// 791; torus N = 10000 200 words 171 / 211, 620 words 434 / 474, 1024 words 729 /
-// 763; n = 2000, degree 12 (14 slices) 200 words 115 / 101, 512 words 164 / 157;
-// 18,000-vertex planar 200 words 362 / 451, 270 words 631 / 451.
+// one-CTA blocks, on 152 SMs: G63-shaped 200 words 193 / 221, 270 words 254 / 237,
+// 470 words 341 / 376, 560 words 439 / 400, 1000 words 672 / 740, 1200 words 838 /
+// 791; torus N = 10000 200 words 168 / 207, 470 words 338 / 378, 1000 words 687 /
+// 750; n = 2000, degree 12 (14 slices) 200 words 115 / 101, 512 words 164 / 157;
+// 18,000-vertex planar 200 words 359 / 399, 270 words 631 / 451.
 bool pair_tail(int32_t words, int sms, int occ, int32_t slices) {
     const int32_t cap = occ * sms, rem = words % cap, q = rem / sms, r = rem % sms;
     if (r == 0 || slices < 24 || words < sms) return false;
@@ -618,9 +618,9 @@ int pa_anneal_begin(pa_ctx *c, const double *betas, int32_t K, int32_t R, int32_
         // 4-replica packed layout from a number of words that falls with the
         // slices of 32 positions in the largest class, which keep the CTAs busy.
         // us per step of 4 sweeps, packed / multi-spin coded: 18,000-vertex planar
-        // (139 slices) R = 64 163 / 115, torus N = 4900 (77) R = 64 50 / 39; G63-
-        // shaped (47) R = 512 98 / 114, R = 768 143 / 117; n = 2000, degree 12 (14)
-        // R = 1024 70 / 82, R = 1536 77 / 82, R = 2048 91 / 82.
+        // (139 slices) R = 32 159 / 100, torus N = 4900 (77) R = 32 49 / 34; G63-
+        // shaped (47) R = 448 96 / 98, R = 800 138 / 100; n = 2000, degree 12 (14)
+        // R = 1216 68 / 74, R = 1472 75 / 75, R = 2240 89 / 75.
         const bool msc_ok = msc_fits && o.field_bits == 0 && (o.threads_per_cta == 0 || o.threads_per_cta <= 256);
         const int32_t words = (R + 31) / 32, slices = (c->maxcls + 31) / 32;
         const bool spread = 5 * words >= 2 * sms ||
@@ -694,9 +694,9 @@ int pa_anneal_begin(pa_ctx *c, const double *betas, int32_t K, int32_t R, int32_
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const int32_t words = r.nblk, wm = (words / sms) * sms;
         if (pair_tail(words, sms, r.sweep.occ, (c->maxcls + 31) / 32)) {
-            ce = pa::sweep_configure(g, R - 32 * wm, 8, 2, 256, c->weighted, &r.sweep2, 2);
+            ce = pa::sweep_configure(g, R - 32 * wm, 8, 2, 256, c->weighted, &r.sweep2, 2, words);
             if (ce != cudaSuccess) return cuda_fail(c, ce, "sweep_configure (tail)");
-            ce = pa::sweep_configure(g, 32 * wm, 8, 1, threads, c->weighted, &r.sweep);
+            ce = pa::sweep_configure(g, 32 * wm, 8, 1, threads, c->weighted, &r.sweep, 0, words);
             if (ce != cudaSuccess) return cuda_fail(c, ce, "sweep_configure (head)");
             if (!r.st2 && cudaStreamCreateWithFlags(&r.st2, cudaStreamNonBlocking) != cudaSuccess)
                 return fail(c, PA_ECUDA, "stream create");

@@ -54,3 +54,17 @@ def test_row_encodings_and_short_queues(n, maxdeg, m):
     gpu = run_gpu(g, betas, 33, 1, seed=5, variant=1)
     orc = run_oracle(g, betas, 33, 1, seed=5)
     assert_parity(gpu, orc, g, 33, 1)
+
+
+@pytest.mark.parametrize("n,R,variant", [
+    (8001, 33, 3), (8001, 700, 3), (8001, 1300, 3), (8001, 2500, 3), (8001, 5000, 3),   # 8, 4, 2, 1 CTAs per word; pairs past one word per SM
+    (8001, 33, 1), (250, 40, 1),                                                        # one CTA: 512 threads, and 256 for a short class
+    (18000, 4870, 1), (40000, 33, 3)])                                                  # two CTAs, one CTA in an SM's shared memory
+def test_threads_and_clusters(n, R, variant):
+    """Each block size and cluster size of the launch rule."""
+    require_gpu()
+    g = _hub_graph(n, 9, 2 * n, n, True)
+    betas = np.array([0.3, 1.5])
+    gpu = run_gpu(g, betas, R, 1, seed=R, variant=variant)
+    orc = run_oracle(g, betas, R, 1, seed=R)
+    assert_parity(gpu, orc, g, R, 1)
