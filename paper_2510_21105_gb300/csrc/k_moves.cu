@@ -541,6 +541,8 @@ __device__ __forceinline__ void ad_take(const AdaptArgs &a, int n_prev, int j) {
 // butterflies; zero padding adds exact zeros), ESS_j = A^2 / B, and the smallest
 // j with ESS_j >= rho R is taken (else J).
 __global__ void __launch_bounds__(RS_CHUNK) k_ad_partials(AdaptArgs a) {
+    wait_previous();
+    ready_for_next();
     const int n_prev = a.state[0];
     if (n_prev >= a.nmax) {
         if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) a.active[a.k] = 0;
@@ -743,10 +745,20 @@ cudaError_t launch_nonlocal(const NlmArgs &a, void *scratch, cudaStream_t st, in
     return cudaGetLastError();
 }
 
-cudaError_t launch_adapt(const AdaptArgs &a, cudaStream_t st) {
-    if (a.mode == 2) k_ad_accept<<<1, 1, 0, st>>>(a);
-    else k_ad_partials<<<dim3(a.nch, a.J + 1), RS_CHUNK, 0, st>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_adapt(const AdaptArgs &a, cudaStream_t st, bool early) {
+    if (a.mode == 2) {
+        k_ad_accept<<<1, 1, 0, st>>>(a);
+        return cudaGetLastError();
+    }
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(a.nch, a.J + 1);
+    lc.blockDim = dim3(RS_CHUNK);
+    lc.stream = st;
+    cudaLaunchAttribute at[1];
+    early_attribute(at[0]);
+    lc.attrs = at;
+    lc.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&lc, k_ad_partials, a);
 }
 
 }  // namespace pa

@@ -105,6 +105,8 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_step(ResampleArgs a) {
     __shared__ ClusterShared sh;
     __shared__ double qs[32];
     const int rank = (int)cg::this_cluster().block_rank();
+    wait_previous();
+    ready_for_next();
     if (rank == 0 && threadIdx.x == 0) a.stamp[a.k] = gtimer();
     if (a.active && !a.active[a.k]) return;   // the whole cluster
     const int row = a.qsel ? a.qsel[a.k] : a.k;
@@ -280,7 +282,7 @@ cudaError_t launch_rs_min(const ResampleArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_rs_step(const ResampleArgs &a, cudaStream_t st) {
+cudaError_t launch_rs_step(const ResampleArgs &a, cudaStream_t st, bool early) {
     const ClusterShape shape = cluster_shape(a.R, RS_THREADS);
     auto *kernel = shape.k == 1   ? &k_rs_step<1>
                    : shape.k == 2 ? &k_rs_step<2>
@@ -288,7 +290,7 @@ cudaError_t launch_rs_step(const ResampleArgs &a, cudaStream_t st) {
                    : shape.k == 8 ? &k_rs_step<8>
                    : shape.k == 16 ? &k_rs_step<16>
                                    : &k_rs_step<32>;
-    return launch_cluster(kernel, shape, RS_THREADS, st, a);
+    return launch_cluster(kernel, shape, RS_THREADS, st, early, a);
 }
 
 cudaError_t launch_stamp(unsigned long long *stamp, cudaStream_t st) {

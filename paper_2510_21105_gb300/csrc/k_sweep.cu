@@ -190,6 +190,7 @@ __device__ __forceinline__ bool sweep_item(uint32_t *__restrict__ Ssm, const uin
 template <int G, int FB, bool WEIGHTED>
 __global__ void __launch_bounds__(1024) k_sweep(const SweepArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
+    wait_previous();
     // A step after the adaptive schedule has ended only carries the population over.
     const bool act = !a.active || a.active[a.k];
     const int nsweeps = act ? a.S : 0;
@@ -233,8 +234,8 @@ __global__ void __launch_bounds__(1024) k_sweep(const SweepArgs a) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const size_t row = (size_t)PS[4 * g + q] * np + 4 * c;
-                w[q] = __ldg(reinterpret_cast<const uint32_t *>(a.spins_in + row));
-                f[q] = __ldg(reinterpret_cast<const uint2 *>(a.fields_in + row));
+                w[q] = __ldcg(reinterpret_cast<const uint32_t *>(a.spins_in + row));
+                f[q] = __ldcg(reinterpret_cast<const uint2 *>(a.fields_in + row));
             }
             uint32_t o[4];
             transpose4x4_bytes(w[0], w[1], w[2], w[3], o);
@@ -517,6 +518,7 @@ __device__ __forceinline__ void pk_round(uint32_t *__restrict__ Bsm, const uint2
 template <bool WEIGHTED, int NTB, int MINB>
 __global__ void __launch_bounds__(NTB, MINB) k_sweep_packed(const SweepArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
+    wait_previous();
     const bool act = !a.active || a.active[a.k];
     const int nsweeps = act ? a.S : 0;
     const int np = a.g.np;
@@ -555,8 +557,8 @@ __global__ void __launch_bounds__(NTB, MINB) k_sweep_packed(const SweepArgs a) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const size_t row = (size_t)PS[q] * np + 4 * c;
-                w[q] = __ldg(reinterpret_cast<const uint32_t *>(a.spins_in + row));
-                f[q] = __ldg(reinterpret_cast<const uint2 *>(a.fields_in + row));
+                w[q] = __ldcg(reinterpret_cast<const uint32_t *>(a.spins_in + row));
+                f[q] = __ldcg(reinterpret_cast<const uint2 *>(a.fields_in + row));
             }
             uint32_t o[4];
             transpose4x4_bytes(w[0], w[1], w[2], w[3], o);
@@ -723,8 +725,6 @@ template <int FB, bool WEIGHTED, int NH>
 __global__ void __launch_bounds__(2 * NH) k_sweep_small(const SweepArgs a) {
     constexpr int NT = 2 * NH;
     extern __shared__ __align__(16) unsigned char smem[];
-    const bool act = !a.active || a.active[a.k];
-    const int nsweeps = act ? a.S : 0;
     const int np = a.g.np, n = a.g.n, ncol = a.g.ncol;
     uint32_t *U = reinterpret_cast<uint32_t *>(smem);              // [np][4] uniforms of the sweep
     uint32_t *Bsm = U + 4 * np;                                    // FB 7: [np + 32] bytes; FB 16: [2 (np + 32)] fields
@@ -739,12 +739,15 @@ __global__ void __launch_bounds__(2 * NH) k_sweep_small(const SweepArgs a) {
     uint32_t *Psm = reinterpret_cast<uint32_t *>(misc + 8);        // FB 7: degree parity bits
     const int tid = threadIdx.x, lane = tid & 31, ht = tid & (NH - 1);   // ht: thread of its half
     const bool decides = tid < NH;
-    const uint32_t *tab = a.tables + (size_t)a.tidx[a.k] * (a.g.mmax + 1);
-    for (int i = tid; i <= a.g.mmax; i += NT) T[i] = tab[i];
     for (int i = tid; i <= n; i += NT) rows[i] = a.g.prp[i];
     if (FB == 7)
         for (int i = tid; i < (np + 31) >> 5; i += NT) Psm[i] = a.g.parity[i];
     for (int i = tid; i <= ncol; i += NT) cls[i] = a.g.cls[i];
+    wait_previous();
+    const bool act = !a.active || a.active[a.k];
+    const int nsweeps = act ? a.S : 0;
+    const uint32_t *tab = a.tables + (size_t)a.tidx[a.k] * (a.g.mmax + 1);
+    for (int i = tid; i <= a.g.mmax; i += NT) T[i] = tab[i];
 
     for (int blk = blockIdx.x; blk < a.nblk; blk += gridDim.x) {
         const int slot0 = blk * 4;
@@ -762,8 +765,8 @@ __global__ void __launch_bounds__(2 * NH) k_sweep_small(const SweepArgs a) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const size_t row = (size_t)PS[q] * np + 4 * c;
-                w[q] = __ldg(reinterpret_cast<const uint32_t *>(a.spins_in + row));
-                f[q] = __ldg(reinterpret_cast<const uint2 *>(a.fields_in + row));
+                w[q] = __ldcg(reinterpret_cast<const uint32_t *>(a.spins_in + row));
+                f[q] = __ldcg(reinterpret_cast<const uint2 *>(a.fields_in + row));
             }
             uint32_t o[4];
             transpose4x4_bytes(w[0], w[1], w[2], w[3], o);
@@ -944,6 +947,7 @@ __global__ void __launch_bounds__(2 * NH) k_sweep_small(const SweepArgs a) {
             }
             if (decides) first(0);
         }
+        if (blk + (int)gridDim.x >= a.nblk) ready_for_next();
         // Store to the next population buffers.
         for (int c = tid; c < (np >> 2); c += NT) {
             uint32_t sp[4] = {0u, 0u, 0u, 0u}, fx[4] = {0u, 0u, 0u, 0u}, fy[4] = {0u, 0u, 0u, 0u};
@@ -1047,7 +1051,7 @@ __device__ __forceinline__ int msc_lane_replica(int lane) { return 4 * (lane & 7
 
 // row: this lane's row; group of 128 positions q.
 __device__ __forceinline__ void msc_load_words(const uint32_t *row, uint32_t *Wsm, int np, int q, int lane) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4 *>(row) + q);
+    const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(row) + q);
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -1535,6 +1539,7 @@ __global__ void __launch_bounds__(512, 2) k_sweep_msc(const SweepArgs a) {
     namespace cg = cooperative_groups;
     using Sh = MscShape<N>;
     extern __shared__ __align__(16) unsigned char smem[];
+    wait_previous();
     const bool act = !a.active || a.active[a.k];
     const int nsweeps = act ? a.S : 0;
     const int np = a.g.np, n = a.g.n;
@@ -1713,6 +1718,7 @@ __global__ void __launch_bounds__(512, 2) k_sweep_msc(const SweepArgs a) {
             }
             if (CL) barrier();   // the copy reads CTA 0's words before the next sweep changes them
         }
+        if (lb + nunits >= a.nblk) ready_for_next();
         {   // words -> bit rows; the CTAs of a cluster share the columns
             uint32_t *row = reinterpret_cast<uint32_t *>(a.spins_out) +
                             (size_t)(slot0 + msc_lane_replica(lane)) * a.g.nbw;
@@ -2080,7 +2086,7 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
     return cudaSuccess;
 }
 
-cudaError_t launch_sweep(const SweepConfig &cfg, const SweepArgs &a, cudaStream_t st) {
+cudaError_t launch_sweep(const SweepConfig &cfg, const SweepArgs &a, cudaStream_t st, bool early) {
     void *fn = select_kernel(cfg.G, cfg.field_bits, a.g.wt != nullptr, cfg.threads, a.g.mmax, a.g.mbig != 0, cfg.small);
     SweepArgs b = a;
     b.qcap = cfg.qcap;
@@ -2090,12 +2096,13 @@ cudaError_t launch_sweep(const SweepConfig &cfg, const SweepArgs &a, cudaStream_
     lc.blockDim = dim3(cfg.threads);
     lc.dynamicSmemBytes = cfg.smem;
     lc.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = cfg.cluster;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    lc.attrs = at;
-    lc.numAttrs = cfg.field_bits == 2 ? 1 : 0;
+    cudaLaunchAttribute at[2];
+    early_attribute(at[0]);
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cfg.cluster;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    lc.attrs = early ? at : at + 1;
+    lc.numAttrs = (early ? 1 : 0) + (cfg.field_bits == 2 ? 1 : 0);
     return cudaLaunchKernelExC(&lc, fn, args);
 }
 

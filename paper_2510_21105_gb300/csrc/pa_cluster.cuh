@@ -184,19 +184,20 @@ __device__ __forceinline__ void fill_parents(int32_t *__restrict__ parent, int32
     }
 }
 
-// Launches a cluster kernel of `shape` on st.
+// Launches a cluster kernel of `shape` on st; early: see wait_previous.
 template <class... P, class... A>
-cudaError_t launch_cluster(void (*kernel)(P...), const ClusterShape &shape, int threads, cudaStream_t st, A... args) {
+cudaError_t launch_cluster(void (*kernel)(P...), const ClusterShape &shape, int threads, cudaStream_t st, bool early, A... args) {
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(shape.ctas);
     lc.blockDim = dim3(threads);
     lc.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = shape.ctas;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    early_attribute(at[1]);
     lc.attrs = at;
-    lc.numAttrs = 1;
+    lc.numAttrs = early ? 2 : 1;
     return cudaLaunchKernelEx(&lc, kernel, args...);
 }
 

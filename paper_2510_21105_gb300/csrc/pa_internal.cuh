@@ -206,7 +206,7 @@ cudaError_t launch_rows_in(const GraphDev &g, const int8_t *raw, int8_t *rows, b
 cudaError_t launch_check(const int8_t *raw, size_t bytes, int32_t *bad, cudaStream_t st);
 // Minimum of the energies; the step's start stamp, weights and parents.
 cudaError_t launch_rs_min(const ResampleArgs &a, cudaStream_t st);
-cudaError_t launch_rs_step(const ResampleArgs &a, cudaStream_t st);
+cudaError_t launch_rs_step(const ResampleArgs &a, cudaStream_t st, bool early = false);
 cudaError_t launch_stamp(unsigned long long *stamp, cudaStream_t st);
 
 struct SweepConfig {
@@ -220,6 +220,20 @@ struct SweepConfig {
     int occ = 0;          // resident blocks per SM (no cluster)
     int qcap = 0;   // multi-spin coded: tie-queue entries per warp; other layouts: entries of the block's queue (0: none)
 };
+// Launches that begin while the kernel before them in the stream ends ("early").
+// Every kernel launched so runs wait_previous before it touches what a step
+// writes, all threads, so that a kernel that has ended implies that all before it
+// have; tables of the graph are older than the chain and may be read ahead. Data
+// that a step writes is read past the read-only cache. ready_for_next lets the
+// next kernel's CTAs take free slots; no CTA of this one is then unscheduled.
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void ready_for_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+inline void early_attribute(cudaLaunchAttribute &at) {
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+}
+
 // Dynamic shared memory of one sweep CTA (G: 4-replica groups of the int8/int16 layouts;
 // field_bits 1/2 multi-spin coded, 7 packed, 8/16 int8/int16 fields).
 size_t sweep_smem_bytes(const GraphDev &g, int G, int field_bits, int threads);
@@ -229,6 +243,6 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
                             bool weighted, SweepConfig *cfg, int cluster = 0, int all_words = 0);
 // CTAs per word that the multi-spin-coded layout should use for `words` words (1: no cluster).
 int msc_cluster(const GraphDev &g, int words, int sms);
-cudaError_t launch_sweep(const SweepConfig &cfg, const SweepArgs &a, cudaStream_t st);
+cudaError_t launch_sweep(const SweepConfig &cfg, const SweepArgs &a, cudaStream_t st, bool early = false);
 
 }  // namespace pa

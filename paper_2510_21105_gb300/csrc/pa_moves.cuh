@@ -65,7 +65,7 @@ struct AdaptArgs {
 // j = 0; a previous step that accepted fewer than acc_lo n R S flips moves j
 // one level finer (j + 1, at most J), more than acc_hi n R S one level
 // coarser (j - 1, at least 0); dn = min(2^(J-j), nmax - n_prev).
-cudaError_t launch_adapt(const AdaptArgs &a, cudaStream_t st);
+cudaError_t launch_adapt(const AdaptArgs &a, cudaStream_t st, bool early = false);
 
 // Stagnation reheating (an alternative reading of the adaptive control):
 // at the start of step k > 0 the lowest sweep-end energy of step k-1 updates

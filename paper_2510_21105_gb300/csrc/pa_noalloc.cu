@@ -118,7 +118,7 @@ extern "C" int pa_resample_noalloc(const int32_t *energies, int32_t R, double be
     }
     const pa::ClusterShape shape = pa::cluster_shape(R, pa::CL_THREADS);
     auto *kernel = shape.k == 1 ? &k_resample_noalloc<1> : shape.k == 2 ? &k_resample_noalloc<2> : &k_resample_noalloc<4>;
-    if (pa::launch_cluster(kernel, shape, pa::CL_THREADS, st, energies, R, qp, (uint32_t)seed, (uint32_t)(seed >> 32), (uint32_t)k, parent,
+    if (pa::launch_cluster(kernel, shape, pa::CL_THREADS, st, false, energies, R, qp, (uint32_t)seed, (uint32_t)(seed >> 32), (uint32_t)k, parent,
                            counts, result) != cudaSuccess) {
         cudaGetLastError();
         return PA_ECUDA;

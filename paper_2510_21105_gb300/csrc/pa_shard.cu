@@ -228,7 +228,7 @@ int pa_shard_partials(const int32_t *energies, int32_t n, int32_t emin, double b
                    : shape.k == 2 ? &k_shard_partials<2>
                    : shape.k == 4 ? &k_shard_partials<4>
                                   : &k_shard_partials<8>;
-    if (pa::launch_cluster(kernel, shape, pa::CL_THREADS, st, energies, n, emin, qp, s) != cudaSuccess) {
+    if (pa::launch_cluster(kernel, shape, pa::CL_THREADS, st, false, energies, n, emin, qp, s) != cudaSuccess) {
         cudaGetLastError();
         return PA_ECUDA;
     }

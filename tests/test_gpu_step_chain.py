@@ -58,3 +58,23 @@ def test_replaced_population_forgets_the_old_minimum(opts):
         (s2, e2), m2, A2, c2 = got[1]
         assert np.array_equal(s1, s2) and np.array_equal(e1, e2)
         assert np.array_equal(m1, m2) and np.array_equal(A1, A2) and np.array_equal(c1, c2)
+
+
+ESS = dict(adaptive=1, rho=0.6, adapt_J=5, adapt_dbeta_max=0.25, beta_max=2.0)
+ACC = dict(adaptive=2, adapt_J=4, adapt_dbeta_max=0.4, beta_max=3.0, acc_lo=0.12, acc_hi=0.3)
+
+
+@pytest.mark.parametrize("opts", [dict(), dict(variant=1), dict(variant=3), dict(field_bits=16), dict(field_bits=8),
+                                  dict(field_bits=7, threads_per_cta=128), ESS, dict(variant=3, **ESS), ACC,
+                                  dict(reheat_after=4, reheat_back=2), dict(variant=1, nlm_period=3)])
+@pytest.mark.parametrize("R", [70, 2500])
+def test_many_short_steps(opts, R):
+    """Steps of a few microseconds, each launched while the one before it ends."""
+    require_gpu()
+    g = wl.gnm(300, 900, seed=3)
+    betas = None if "adaptive" in opts else wl.linear_betas(0.05, 3.0, 60)
+    K = 80 if betas is None else None
+    kw = {k: v for k, v in opts.items() if k not in ("variant", "field_bits", "threads_per_cta")}
+    gpu = run_gpu(g, betas, R, 1, seed=R, K=K, **opts)
+    orc = run_oracle(g, betas, R, 1, seed=R, K=K, **kw)
+    assert_parity(gpu, orc, g, R, 1)
