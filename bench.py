@@ -391,7 +391,7 @@ def run_ours(args, rank, world, dist):
             layout += f"; {words // sms * sms} words in one-CTA blocks + {words % sms} in CTA pairs, concurrently"
             kernel = ("k_sweep_msc+pair", args.threads or 256)
     elif variant_run == 3:
-        layout = "multi-spin coded, a cluster of two CTAs per 32-replica word"
+        layout = "multi-spin coded, a thread-block cluster per 32-replica word"
         kernel = ("k_sweep_msc_pair", 256)
     else:
         fb = args.field_bits if args.field_bits else (7 if g.maxdeg <= 127 else 16)
@@ -405,10 +405,14 @@ def run_ours(args, rank, world, dist):
     stats_acc = {"sweep_ms": 0.0, "sweep_launches": 0, "kernel_launches": 0}
     if dist:
         dist.barrier()
+    # The bit rows of a population fit L2: a larger buffer is written before every anneal.
+    flush = torch.zeros(512 << 20, dtype=torch.uint8, device="cuda")
     torch.cuda.synchronize()
     with ClockSampler(local) as clk:
         ev0.record(stream)
         for _ in range(args.steps):
+            with torch.cuda.stream(stream):
+                flush.zero_()
             one(time_kernels=1)
             st = ann.stats()
             for key in stats_acc:
@@ -439,6 +443,7 @@ def run_ours(args, rank, world, dist):
         lib = B.lib()
         times, h2d, d2h = [], 0, 0
         for it in range(args.steps + 1):
+            flush.zero_()
             torch.cuda.synchronize()
             t0 = time.perf_counter()
             ctx = B.C.c_void_p()
@@ -486,7 +491,7 @@ def run_ours(args, rank, world, dist):
             "data": "synthetic",
             "config": {"workload": f"{args.config}: G63-shaped N={g.n} M={g.m} R={R} K={K} S={S} "
                                    f"beta {c['beta'][0]}->{c['beta'][1]} nlm_period={c['nlm_period']}",
-                       "l2": "inputs larger than L2 (population 688 MB per buffer pair)",
+                       "l2": "flushed before every step (a 512 MB buffer is written, inside the timed region)",
                        "seed": c["seed"]},
             "layout": layout,
             "accept_rate": acc_rate,

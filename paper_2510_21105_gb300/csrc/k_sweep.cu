@@ -1019,7 +1019,9 @@ __global__ void __launch_bounds__(2 * NH) k_sweep_small(const SweepArgs a) {
 // Bound: the ALU pipe (three-input logic and shifts) and, with few large
 // colour classes' worth of warps per SM, latency. Measured per step of 10
 // sweeps, means over beta 0.2 .. 3.6, R = 16384: G63-shaped (N = 7000) 0.981 ->
-// 0.872 ms, signed torus (N = 10000) 1.030 -> 0.843 ms.
+// 0.872 ms, signed torus (N = 10000) 1.030 -> 0.843 ms; with bit rows, round
+// keys for the ties and narrower accumulators since, whole anneals of 200 steps
+// G63-shaped 199 -> 161 ms and, R = 32768, 80 steps of 8 sweeps, torus 140 -> 110.
 //
 // A tie (probability 1/256 per uncertain attempt) is queued with its counter
 // planes, and the ties of a warp's items are settled by all 32 lanes together
