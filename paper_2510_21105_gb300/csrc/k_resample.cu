@@ -49,6 +49,8 @@ __global__ void k_init_spins(GraphDev g, int8_t *spins, int32_t Rpad, uint32_t k
     }
 }
 
+constexpr int ROW_STATIC = 256;   // bytes of static shared memory a kernel may use beside a row
+
 // One CTA per replica: h_p = sum_j w_pj x_j and E = 1/2 sum_p x_p h_p. The
 // replica's row is read once into shared memory, where the neighbours' spins are
 // gathered (N = 18001, R = 1024: 89 us; gathered from global memory 162 us).
@@ -72,7 +74,7 @@ __global__ void k_fields_energy(GraphDev g, const int8_t *spins, int16_t *fields
         }
         h[p] = (int16_t)hp;
     }
-    __shared__ long long red[32];
+    __shared__ long long red[ROW_STATIC / 8];
     for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, off);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
@@ -233,9 +235,10 @@ __global__ void k_stamp(unsigned long long *stamp) { *stamp = gtimer(); }
 }  // namespace
 
 namespace {
-// A row in dynamic shared memory: up to 65,536 bytes.
+// A row in dynamic shared memory: up to 65,536 bytes. Without the attribute the
+// 48 KB hold the kernel's static part as well.
 cudaError_t allow_row(const void *fn, int32_t np) {
-    return np <= 48 * 1024 ? cudaSuccess : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 65536);
+    return np + ROW_STATIC <= 48 * 1024 ? cudaSuccess : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 65536);
 }
 }  // namespace
 
