@@ -694,7 +694,7 @@ cudaError_t launch_nonlocal(const NlmArgs &a, void *scratch, cudaStream_t st, in
         if (a.R < 1) return cudaSuccess;
         const size_t smem = nlm_block_smem_bytes(a.g.np, a.block);
         static std::mutex mu;
-        static size_t raised = 48 * 1024;
+        static size_t raised = 0;   // the 48 KB without it hold the static part as well
         {
             std::lock_guard<std::mutex> lock(mu);
             if (smem > raised) {   // per-function attribute: only ever raise it

@@ -32,6 +32,26 @@ with B.Annealer.from_graph(g) as a:
 np.testing.assert_array_equal(E, [oracle.energy(g.rp, g.col, g.w, row) for row in x])
 """
 
+# Block moves hold the row, two bitsets and the block beside their sums.
+BLOCKS = """
+import sys
+import numpy as np
+import oracle
+from paper_2510_21105_gb300 import binding as B, workloads as wl
+n = int(sys.argv[1])
+g = wl.gnm(n, n, seed=n)
+betas = wl.linear_betas(0.2, 1.5, 3)
+o = dict(nlm_period=1, nlm_kind=1, nlm_block=32)
+with B.Annealer.from_graph(g) as a:
+    a.anneal(betas, 33, 1, 3, **o)
+    spins, E = a.state()
+    rec = a.step_stats()
+ref = oracle.anneal(g.rp, g.col, g.w, betas, R=33, S=1, seed=3, **o)
+np.testing.assert_array_equal(spins, ref.spins)
+np.testing.assert_array_equal(E, ref.E)
+np.testing.assert_array_equal(rec["nlm_flips"], ref.step_nlm_flips)
+"""
+
 
 def _run(script, *args):
     env = dict(os.environ, PYTHONPATH=ROOT)
@@ -44,3 +64,9 @@ def _run(script, *args):
 def test_energies_of_rows_around_48_kb(n):
     require_gpu()
     _run(ENERGIES, n)
+
+
+@pytest.mark.parametrize("n", [39152, 39153, 39216, 39217])
+def test_block_moves_around_48_kb(n):
+    require_gpu()
+    _run(BLOCKS, n)
