@@ -150,6 +150,21 @@ typedef struct {
     int64_t d2h_bytes;        /* device-to-host bytes copied by this context */
 } pa_stats_t;
 
+/* Shape of the sweep launches of a context's current anneal. A block is what
+ * one CTA, or one cluster of CTAs, anneals: `replicas` replicas of one word or
+ * group. tail_*: the words that run beside the others on a second stream
+ * (all 0 without such a launch). */
+typedef struct {
+    int32_t variant;          /* PA_VARIANT_* that runs */
+    int32_t replicas;         /* replicas per block */
+    int32_t blocks;           /* blocks of the sweep (without the tail) */
+    int32_t threads;          /* threads per CTA */
+    int32_t ctas;             /* CTAs per block: 1, or the size of the cluster */
+    int32_t small_graph;      /* 1: the kernel for graphs whose colour classes
+                                 each fit one round of a CTA */
+    int32_t tail_blocks, tail_threads, tail_ctas;
+} pa_sweep_shape_t;
+
 /* Per-step records; each pointer may be NULL, arrays hold steps_run entries
  * (sweep_emin: steps_run * sweeps, counts: steps_run * R). */
 typedef struct {
@@ -271,6 +286,10 @@ int pa_run_info(pa_ctx *ctx, int32_t *R, int32_t *K, int32_t *sweeps, int32_t *s
 
 /* Totals and timings of the anneal (waits for pending work). */
 int pa_stats(pa_ctx *ctx, pa_stats_t *out);
+
+/* How the current anneal's sweeps are launched (does not wait). Errors:
+ * PA_ESTATE before pa_anneal_begin. */
+int pa_sweep_shape(pa_ctx *ctx, pa_sweep_shape_t *out);
 
 /* Per-step records (waits for pending work). */
 int pa_step_stats(pa_ctx *ctx, pa_step_arrays *out);

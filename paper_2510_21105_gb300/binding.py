@@ -48,6 +48,12 @@ class pa_stats_t(C.Structure):
                 ("h2d_bytes", C.c_int64), ("d2h_bytes", C.c_int64)]
 
 
+class pa_sweep_shape_t(C.Structure):
+    _fields_ = [(name, C.c_int32) for name in
+                ("variant", "replicas", "blocks", "threads", "ctas", "small_graph", "tail_blocks", "tail_threads",
+                 "tail_ctas")]
+
+
 class pa_step_arrays(C.Structure):
     _fields_ = [(name, C.c_void_p) for name in
                 ("beta", "emin", "A", "T", "o", "accepts", "lnZ", "sweep_emin", "nlm_pairs",
@@ -130,6 +136,7 @@ def lib():
                 "pa_save": ([vp, C.c_char_p], C.c_int),
                 "pa_load": ([vp, C.c_char_p], C.c_int),
                 "pa_stats": ([vp, C.POINTER(pa_stats_t)], C.c_int),
+                "pa_sweep_shape": ([vp, C.POINTER(pa_sweep_shape_t)], C.c_int),
                 "pa_run_info": ([vp, C.POINTER(i32), C.POINTER(i32), C.POINTER(i32), C.POINTER(i32)],
                                 C.c_int),
                 "pa_step_stats": ([vp, C.POINTER(pa_step_arrays)], C.c_int),
@@ -169,7 +176,7 @@ def exported_symbols():
     return ["pa_version", "pa_strerror", "pa_last_error", "pa_default_opts", "pa_create",
             "pa_destroy", "pa_anneal", "pa_anneal_begin", "pa_anneal_run", "pa_sync", "pa_best",
             "pa_best_record", "pa_get_state", "pa_set_state", "pa_energies", "pa_save", "pa_load", "pa_stats",
-            "pa_step_stats", "pa_tables", "pa_colouring", "pa_set_allocator", "pa_run_info",
+            "pa_sweep_shape", "pa_step_stats", "pa_tables", "pa_colouring", "pa_set_allocator", "pa_run_info",
             "pa_resample_noalloc", "pa_batch_anneal", "pa_server_start", "pa_server_submit",
             "pa_server_poll", "pa_server_result", "pa_server_stats", "pa_server_stop",
             "pa_server_release", "pa_server_hold", "pa_probe_peaks", "pa_shard_scratch_bytes", "pa_shard_min",
@@ -301,6 +308,12 @@ def pa_stats(ctx) -> dict:
     st = pa_stats_t()
     _check(lib().pa_stats(ctx, C.byref(st)), "pa_stats", ctx)
     return {name: getattr(st, name) for name, _ in pa_stats_t._fields_}
+
+
+def pa_sweep_shape(ctx) -> dict:
+    sh = pa_sweep_shape_t()
+    _check(lib().pa_sweep_shape(ctx, C.byref(sh)), "pa_sweep_shape", ctx)
+    return {name: getattr(sh, name) for name, _ in pa_sweep_shape_t._fields_}
 
 
 def pa_step_stats(ctx, steps: int, R: int, S: int, counts: bool = False) -> dict:
@@ -559,6 +572,9 @@ class Annealer:
 
     def stats(self):
         return pa_stats(self.ctx)
+
+    def sweep_shape(self):
+        return pa_sweep_shape(self.ctx)
 
     def step_stats(self, counts=False):
         st = self.stats()

@@ -1983,7 +1983,7 @@ int msc_cluster(const GraphDev &g, int words, int sms) {
 }
 
 cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int threads,
-                            bool weighted, SweepConfig *cfg, int cluster, int all_words) {
+                            bool weighted, SweepConfig *cfg, int cluster, int whole_threads) {
     int dev = 0, sms = 0, occ = 0, limit = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1997,8 +1997,8 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
             if (!cluster) cluster = msc_cluster(g, (R + 31) / 32, sms);
             if (cluster == 1) field_bits = 1;
         }
-        const int ctas = all_words ? all_words : (R + 31) / 32 * (field_bits == 2 ? cluster : 1);
-        threads = msc_threads(g, ctas, sms, per_sm, limit, field_bits == 2);
+        threads = whole_threads ? whole_threads
+                                : msc_threads(g, (R + 31) / 32 * (field_bits == 2 ? cluster : 1), sms, per_sm, limit, field_bits == 2);
     } else if (field_bits == 7) {
         G = 1;
         // Few blocks: more threads each, so that an SM has about 1024 whatever the

@@ -95,10 +95,9 @@ struct RunState {
     bool begun = false;
     int32_t R = 0, Rpad = 0, K = 0, S = 0, nblk = 0, nch = 0, k_done = 0;
     int32_t nrec = 0;                    // replica blocks in all (one best record each)
-    // Multi-spin coding with a word count that the SM count does not divide:
-    // the first (words / SMs) * SMs words run in the one-CTA kernel and the
-    // rest in the CTA-pair kernel on a second stream, concurrently, so every
-    // SM carries the same share.
+    // Multi-spin coding with words past the largest SM multiple that pay as CTA
+    // pairs (pair_tail): the first (words / SMs) * SMs words run in the one-CTA
+    // kernel and the rest in pairs on a second stream, concurrently.
     bool split = false;
     // Adaptive runs end on the device (the controller reaches beta_max); the
     // host reads the active flag of a step behind the ones it enqueues, through
@@ -694,9 +693,16 @@ int pa_anneal_begin(pa_ctx *c, const double *betas, int32_t K, int32_t R, int32_
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const int32_t words = r.nblk, wm = (words / sms) * sms;
         if (pair_tail(words, sms, r.sweep.occ, (c->maxcls + 31) / 32)) {
-            ce = pa::sweep_configure(g, R - 32 * wm, 8, 2, 256, c->weighted, &r.sweep2, 2, words);
+            // Both parts with the threads chosen for the whole: with 512 in the head and
+            // 256 in the tail the launches ran one after the other or badly side by side
+            // (us per step of 4 sweeps, 200 words: torus N = 10000 338 against 167 with
+            // 256 in both, G63-shaped 382 against 196; where two blocks fit an SM, 512 /
+            // 256, 256 / 256, 512 / 512: 18,000-vertex planar 363, 342, 335; torus
+            // N = 19600 329, 307, 296; n = 16272 and degree 12 393, 384, 361).
+            const int whole = r.sweep.threads;
+            ce = pa::sweep_configure(g, R - 32 * wm, 8, 2, 0, c->weighted, &r.sweep2, 2, whole);
             if (ce != cudaSuccess) return cuda_fail(c, ce, "sweep_configure (tail)");
-            ce = pa::sweep_configure(g, 32 * wm, 8, 1, threads, c->weighted, &r.sweep, 0, words);
+            ce = pa::sweep_configure(g, 32 * wm, 8, 1, 0, c->weighted, &r.sweep, 0, whole);
             if (ce != cudaSuccess) return cuda_fail(c, ce, "sweep_configure (head)");
             if (!r.st2 && cudaStreamCreateWithFlags(&r.st2, cudaStreamNonBlocking) != cudaSuccess)
                 return fail(c, PA_ECUDA, "stream create");
@@ -1375,6 +1381,25 @@ int pa_run_info(pa_ctx *c, int32_t *R, int32_t *K, int32_t *sweeps, int32_t *ste
     if (K) *K = r.K;
     if (sweeps) *sweeps = r.S;
     if (steps_done) *steps_done = r.k_done;
+    return PA_OK;
+}
+
+int pa_sweep_shape(pa_ctx *c, pa_sweep_shape_t *out) {
+    if (!c || !out) return PA_EINVAL;
+    const RunState &r = c->run;
+    if (!r.begun) return fail(c, PA_ESTATE, "no anneal");
+    *out = pa_sweep_shape_t{};
+    out->variant = r.variant;
+    out->replicas = 4 * r.sweep.G;
+    out->blocks = r.nblk;
+    out->threads = r.sweep.threads;
+    out->ctas = r.sweep.field_bits == 2 ? r.sweep.cluster : 1;
+    out->small_graph = r.sweep.small ? 1 : 0;
+    if (r.split) {
+        out->tail_blocks = r.nblk2;
+        out->tail_threads = r.sweep2.threads;
+        out->tail_ctas = r.sweep2.cluster;
+    }
     return PA_OK;
 }
 

@@ -237,10 +237,10 @@ inline void early_attribute(cudaLaunchAttribute &at) {
 // Dynamic shared memory of one sweep CTA (G: 4-replica groups of the int8/int16 layouts;
 // field_bits 1/2 multi-spin coded, 7 packed, 8/16 int8/int16 fields).
 size_t sweep_smem_bytes(const GraphDev &g, int G, int field_bits, int threads);
-// threads = 0, cluster = 0: chosen here; all_words: words of the whole sweep where this launch is
-// one part of it (0: it is all).
+// threads = 0, cluster = 0: chosen here (multi-spin coded: always); whole_threads: threads of the
+// whole multi-spin-coded sweep where this launch is one part of it (0: it is all).
 cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int threads,
-                            bool weighted, SweepConfig *cfg, int cluster = 0, int all_words = 0);
+                            bool weighted, SweepConfig *cfg, int cluster = 0, int whole_threads = 0);
 // CTAs per word that the multi-spin-coded layout should use for `words` words (1: no cluster).
 int msc_cluster(const GraphDev &g, int words, int sms);
 cudaError_t launch_sweep(const SweepConfig &cfg, const SweepArgs &a, cudaStream_t st, bool early = false);
