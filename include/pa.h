@@ -162,6 +162,8 @@ typedef struct {
     int32_t ctas;             /* CTAs per block: 1, or the size of the cluster */
     int32_t small_graph;      /* 1: the kernel for graphs whose colour classes
                                  each fit one round of a CTA */
+    int32_t row_queue;        /* 1: accepted items of the int8/int16 kernel go
+                                 through a queue of the block */
     int32_t tail_blocks, tail_threads, tail_ctas;
 } pa_sweep_shape_t;
 

@@ -187,7 +187,7 @@ __device__ __forceinline__ bool sweep_item(uint32_t *__restrict__ Ssm, const uin
     return true;
 }
 
-template <int G, int FB, bool WEIGHTED>
+template <int G, int FB, bool WEIGHTED, bool QUEUED>
 __global__ void __launch_bounds__(1024) k_sweep(const SweepArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     wait_previous();
@@ -207,13 +207,12 @@ __global__ void __launch_bounds__(1024) k_sweep(const SweepArgs a) {
     int32_t *misc = PS + 4 * G;         // best E, step, sweep, slot, copy-from (q+1), changed
     SweepQueue Q{reinterpret_cast<uint4 *>(misc + 8), nullptr, 0};
     Q.count = reinterpret_cast<int32_t *>(Q.ent + 2 * blockDim.x);
-    const bool queued = a.qcap != 0;   // room for the queue
 
     const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31;
     const uint32_t *tab = a.tables + (size_t)a.tidx[a.k] * (a.g.mmax + 1);
     for (int i = tid; i <= a.g.mmax; i += NT) Tt[i] = tab[i];
     for (int i = tid; i <= a.g.ncol; i += NT) cls[i] = a.g.cls[i];
-    if (queued && tid < 3) Q.count[tid] = 0;
+    if (QUEUED && tid < 3) Q.count[tid] = 0;
     const int gthr = tid % G;   // NT is a multiple of 32, so each thread keeps one group
 
     for (int blk = blockIdx.x; blk < a.nblk; blk += gridDim.x) {
@@ -269,55 +268,63 @@ __global__ void __launch_bounds__(1024) k_sweep(const SweepArgs a) {
         for (int q = 0; q < 4; ++q) vmask |= (slot0 + 4 * gthr + q < a.R) ? (1u << q) : 0u;
         const uint32_t c1 = (uint32_t)(blk * G + gthr);
         uint32_t nacc = 0;
-        // The uniforms of a thread's first item of the next class are drawn while
-        // the present class is finished (they depend on no spin).
+        // With the queue the uniforms of a thread's first item of the next class are
+        // drawn while the present class is finished (they depend on no spin).
         uint32_t vid = 0, uw = 0;
         auto draw = [&](int p, uint32_t c3) {
             vid = __ldg(&a.g.vid[p]);
             uw = group_uniforms(a, vid, c1, c3);
         };
-        if (nsweeps && tid < cls[1] * G) draw(tid / G, TAG_SWEEP);
+        if (QUEUED && nsweeps && tid < cls[1] * G) draw(tid / G, TAG_SWEEP);
         for (int s = 0; s < nsweeps; ++s) {
             const uint32_t c3 = TAG_SWEEP | (uint32_t)s;
             int dE[4] = {0, 0, 0, 0};
             for (int c = 0; c < a.g.ncol; ++c) {
                 const int p0 = cls[c], cnt = (cls[c + 1] - p0) * G;
-                for (int base = 0; base < cnt; base += NT) {   // uniform over the block
-                    const int idx = base + tid;
-                    bool have = false;
-                    uint4 ent = make_uint4(0u, 0u, 0u, 0u);
-                    if (idx < cnt) {
-                        const int p = p0 + idx / G;
-                        if (base) draw(p, c3);
-                        have = sweep_item<G, FB>(Ssm, Hsm, Tt, a, p, gthr, vid, uw, c1, c3, vmask, dE, nacc, ent.y, ent.z);
-                        ent.x = (uint32_t)p | (uint32_t)gthr << 16;
-                    }
-                    auto walk = [&](const uint4 &e, int sub, int lanes) {
-                        const uint32_t pe = e.x & 0xFFFFu, ge = e.x >> 16;
-                        const uint32_t e1 = __ldg(&a.g.rp[pe + 1]);
-                        for (uint32_t i = __ldg(&a.g.rp[pe]) + sub; i < e1; i += lanes) {
-                            const int j = __ldg(&a.g.col[i]);
-                            uint32_t s0 = e.y, s1 = e.z;
-                            if (WEIGHTED && __ldg(&a.g.wt[i]) < 0) {
-                                s0 = 0u - s0;
-                                s1 = 0u - s1;
-                            }
-                            if (FB == 16) {
-                                atomicAdd(&Hsm[2 * (j * G + ge)], s0);
-                                atomicAdd(&Hsm[2 * (j * G + ge) + 1], s1);
-                            } else {
-                                atomicAdd(&Hsm[j * G + ge], s0);
-                            }
+                auto walk = [&](const uint4 &e, int sub, int lanes) {
+                    const uint32_t pe = e.x & 0xFFFFu, ge = e.x >> 16;
+                    const uint32_t e1 = __ldg(&a.g.rp[pe + 1]);
+                    for (uint32_t i = __ldg(&a.g.rp[pe]) + sub; i < e1; i += lanes) {
+                        const int j = __ldg(&a.g.col[i]);
+                        uint32_t s0 = e.y, s1 = e.z;
+                        if (WEIGHTED && __ldg(&a.g.wt[i]) < 0) {
+                            s0 = 0u - s0;
+                            s1 = 0u - s1;
                         }
-                    };
-                    if (queued) Q.push(have, ent, lane);
-                    else if (have) walk(ent, 0, 1);
-                    if (base + NT >= cnt) {
-                        const int cn = c + 1 < a.g.ncol ? c + 1 : 0;
-                        if (tid < (cls[cn + 1] - cls[cn]) * G)
-                            draw(cls[cn] + tid / G, TAG_SWEEP | (uint32_t)(cn ? s : s + 1));
+                        if (FB == 16) {
+                            atomicAdd(&Hsm[2 * (j * G + ge)], s0);
+                            atomicAdd(&Hsm[2 * (j * G + ge) + 1], s1);
+                        } else {
+                            atomicAdd(&Hsm[j * G + ge], s0);
+                        }
                     }
-                    if (queued) Q.drain(walk);
+                };
+                if (QUEUED) {
+                    for (int base = 0; base < cnt; base += NT) {   // uniform over the block
+                        const int idx = base + tid;
+                        bool have = false;
+                        uint4 ent = make_uint4(0u, 0u, 0u, 0u);
+                        if (idx < cnt) {
+                            const int p = p0 + idx / G;
+                            if (base) draw(p, c3);
+                            have = sweep_item<G, FB>(Ssm, Hsm, Tt, a, p, gthr, vid, uw, c1, c3, vmask, dE, nacc, ent.y, ent.z);
+                            ent.x = (uint32_t)p | (uint32_t)gthr << 16;
+                        }
+                        Q.push(have, ent, lane);
+                        if (base + NT >= cnt) {
+                            const int cn = c + 1 < a.g.ncol ? c + 1 : 0;
+                            if (tid < (cls[cn + 1] - cls[cn]) * G)
+                                draw(cls[cn] + tid / G, TAG_SWEEP | (uint32_t)(cn ? s : s + 1));
+                        }
+                        Q.drain(walk);
+                    }
+                } else {
+                    for (int idx = tid; idx < cnt; idx += NT) {
+                        const int p = p0 + idx / G;
+                        uint4 ent = make_uint4((uint32_t)p | (uint32_t)gthr << 16, 0u, 0u, 0u);
+                        draw(p, c3);
+                        if (sweep_item<G, FB>(Ssm, Hsm, Tt, a, p, gthr, vid, uw, c1, c3, vmask, dE, nacc, ent.y, ent.z)) walk(ent, 0, 1);
+                    }
                 }
                 __syncthreads();
             }
@@ -1901,11 +1908,11 @@ void *packed_kernel(int threads) {
 }
 
 template <int G, int FB, bool W>
-void *kernel_ptr() {
-    return reinterpret_cast<void *>(&k_sweep<G, FB, W>);
+void *kernel_ptr(bool queued) {
+    return queued ? reinterpret_cast<void *>(&k_sweep<G, FB, W, true>) : reinterpret_cast<void *>(&k_sweep<G, FB, W, false>);
 }
 
-void *select_kernel(int G, int fb, bool weighted, int threads, int mmax, bool big, bool small) {
+void *select_kernel(int G, int fb, bool weighted, int threads, int mmax, bool big, bool small, bool queued) {
     if (fb == 1 || fb == 2) {
         if (big) return weighted ? msc_kernel<true, true>(mmax, fb == 2) : msc_kernel<false, true>(mmax, fb == 2);
         return weighted ? msc_kernel<true, false>(mmax, fb == 2) : msc_kernel<false, false>(mmax, fb == 2);
@@ -1916,11 +1923,11 @@ void *select_kernel(int G, int fb, bool weighted, int threads, int mmax, bool bi
     }
     if (fb == 7) return weighted ? packed_kernel<true>(threads) : packed_kernel<false>(threads);
     if (G == 1) {
-        if (fb == 16) return weighted ? kernel_ptr<1, 16, true>() : kernel_ptr<1, 16, false>();
-        return weighted ? kernel_ptr<1, 8, true>() : kernel_ptr<1, 8, false>();
+        if (fb == 16) return weighted ? kernel_ptr<1, 16, true>(queued) : kernel_ptr<1, 16, false>(queued);
+        return weighted ? kernel_ptr<1, 8, true>(queued) : kernel_ptr<1, 8, false>(queued);
     }
-    if (fb == 16) return weighted ? kernel_ptr<2, 16, true>() : kernel_ptr<2, 16, false>();
-    return weighted ? kernel_ptr<2, 8, true>() : kernel_ptr<2, 8, false>();
+    if (fb == 16) return weighted ? kernel_ptr<2, 16, true>(queued) : kernel_ptr<2, 16, false>(queued);
+    return weighted ? kernel_ptr<2, 8, true>(queued) : kernel_ptr<2, 8, false>(queued);
 }
 
 }  // namespace
@@ -1982,6 +1989,26 @@ int msc_cluster(const GraphDev &g, int words, int sms) {
     return c;
 }
 
+// The int8/int16 kernels: blocks of the launch for each SM, and blocks of t threads
+// and smem bytes that an SM holds (at least one).
+static int int_blocks_per_sm(int R, int G, int sms) { return ((R + 4 * G - 1) / (4 * G) + sms - 1) / sms; }
+static int int_resident(int t, size_t smem, int per_sm) {
+    return std::max(1, std::min(1024 / t, (int)((size_t)per_sm / (smem + 1024))));
+}
+
+// Whether the int8/int16 kernels queue their accepted items: the block's lanes for
+// each position of a class, times the neighbours of a row, from 96. Below that a
+// thread is done with its own rows before the queue's barrier pays. us per step of 4
+// sweeps without / with the queue (512 threads; that figure in brackets): 18,001-
+// vertex planar 259 / 340 (5), n = 7000, degree 12 140 / 169 (8), n = 2000, degree 12
+// 69 / 75 (28), n = 7000, degree 48 271 / 279 (70), n = 2000, degree 24 104 / 101 (80),
+// n = 2000, degree 48 192 / 157 (233), n = 7000, degree 100 574 / 466 (234), n = 500,
+// degree 250 874 / 375 (19,200); groups of 8 replicas, n = 2000, degree 48 189 / 189
+// (117), n = 7000, degree 100 750 / 654 (117).
+static bool row_queue_pays(const GraphDev &g, int G, int threads) {
+    return (double)g.m2 * threads * g.ncol >= 96.0 * g.n * g.n * G;
+}
+
 cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int threads,
                             bool weighted, SweepConfig *cfg, int cluster, int whole_threads) {
     int dev = 0, sms = 0, occ = 0, limit = 0, per_sm = 0;
@@ -2011,9 +2038,23 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
             threads = per <= 1 ? 1024 : per == 2 ? 512 : per <= 4 ? 256 : 128;
             while (threads > 128 && threads / 2 >= g.maxcls) threads /= 2;
         }
-    } else if (automatic) {   // as above; n = 500, degree 250, R = 4096: 404 us with 128 threads, 1375 with 512
-        const int per = ((R + 4 * G - 1) / (4 * G) + sms - 1) / sms;
-        threads = per <= 2 ? 512 : per <= 4 ? 256 : 128;
+    } else if (automatic) {
+        // 512 threads, and half as many as long as that saves a wave of blocks (an
+        // SM holds 1024 threads of these kernels, and what its shared memory has
+        // room for) and the classes leave many of the threads idle. us per step of 4
+        // sweeps with 512 / 256 / 128 threads: int16, n = 300, degree 24, R = 5000
+        // (9 blocks per SM) 334 / 205 / 146; int8, n = 2000, degree 6, 4 blocks per SM
+        // 119 / 93 / 112, 9 blocks 251 / 206 / 179. Large classes and few blocks in
+        // shared memory keep 512: int8, 18,001-vertex planar 265 / 444 / 808, int16,
+        // N = 4900 torus (three fit, 4 per SM) 181 / 261 / 449.
+        const int per = int_blocks_per_sm(R, G, sms);
+        const size_t block = sweep_smem_bytes(g, G, field_bits, 0);
+        auto waves = [&](int t) {
+            const int res = int_resident(t, block, per_sm);
+            return (per + res - 1) / res;
+        };
+        threads = 512;
+        while (threads > 128 && waves(threads / 2) < waves(threads) && (size_t)g.n * G < (size_t)2 * threads * g.ncol) threads /= 2;
     }
     size_t smem = sweep_smem_bytes(g, G, field_bits, threads);
     if (msc) {
@@ -2042,14 +2083,20 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
             cfg->small = true;
             threads = 2 * half;
             smem = need;
-        } else if (field_bits != 7 && smem + sweep_queue_bytes(threads) <= (size_t)limit) {
+        } else if (field_bits != 7 && row_queue_pays(g, G, threads)) {
             // int8/int16: the block's queue of accepted items, where shared memory
-            // has room for it (without it each thread walks its own rows).
-            smem += sweep_queue_bytes(threads);
-            cfg->qcap = threads;
+            // has room for it without costing a resident block (without it each
+            // thread walks its own rows).
+            const size_t with = smem + sweep_queue_bytes(threads);
+            const int all = int_blocks_per_sm(R, G, sms);
+            if (with <= (size_t)limit &&
+                std::min(all, int_resident(threads, with, per_sm)) == std::min(all, int_resident(threads, smem, per_sm))) {
+                smem = with;
+                cfg->qcap = threads;
+            }
         }
     }
-    void *fn = select_kernel(G, field_bits, weighted, threads, g.mmax, g.mbig != 0, small);
+    void *fn = select_kernel(G, field_bits, weighted, threads, g.mmax, g.mbig != 0, small, cfg->qcap != 0);
     if (cudaError_t e = raise_smem(fn, smem)) return e;
     const int nblk = (R + 4 * G - 1) / (4 * G);
     if (field_bits == 2) {
@@ -2089,7 +2136,7 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
 }
 
 cudaError_t launch_sweep(const SweepConfig &cfg, const SweepArgs &a, cudaStream_t st, bool early) {
-    void *fn = select_kernel(cfg.G, cfg.field_bits, a.g.wt != nullptr, cfg.threads, a.g.mmax, a.g.mbig != 0, cfg.small);
+    void *fn = select_kernel(cfg.G, cfg.field_bits, a.g.wt != nullptr, cfg.threads, a.g.mmax, a.g.mbig != 0, cfg.small, cfg.qcap != 0);
     SweepArgs b = a;
     b.qcap = cfg.qcap;
     void *args[] = {&b};

@@ -1395,6 +1395,7 @@ int pa_sweep_shape(pa_ctx *c, pa_sweep_shape_t *out) {
     out->threads = r.sweep.threads;
     out->ctas = r.sweep.field_bits == 2 ? r.sweep.cluster : 1;
     out->small_graph = r.sweep.small ? 1 : 0;
+    out->row_queue = r.variant == PA_VARIANT_I8 && r.sweep.qcap > 0 ? 1 : 0;
     if (r.split) {
         out->tail_blocks = r.nblk2;
         out->tail_threads = r.sweep2.threads;
