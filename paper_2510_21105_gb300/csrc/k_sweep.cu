@@ -1756,12 +1756,12 @@ __global__ void __launch_bounds__(512, 2) k_sweep_msc(const SweepArgs a) {
 //               word is set; written to the population's bit rows
 //   WORDS_POP   bit rows of a population
 //   WORDS_RAW   configurations in vertex order (n bytes each, any alignment);
-//               a byte other than +1 / -1 sets *bad
+//               a byte other than +1 / -1 sets *bad (null: checked already)
 // Against a byte per neighbour and replica from global memory the rows are read
 // once per 32 replicas. Torus, N = 10000, R = 32768: initial spins, fields and
 // energies took 1320 us, spins and energies alone (the multi-spin-coded layouts
 // read no fields) take 287 us; bound by the Philox calls.
-inline size_t word_energy_smem(const GraphDev &g) { return ((size_t)g.np + 32 + 64) * 4; }
+inline size_t word_energy_smem(const GraphDev &g) { return ((size_t)g.np + 32 + 32) * 4; }
 
 constexpr int WORDS_INIT = 0, WORDS_POP = 1, WORDS_RAW = 2;
 
@@ -1774,27 +1774,35 @@ __global__ void __launch_bounds__(256, 3) k_word_energy(GraphDev g, const int8_t
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t *Wsm = reinterpret_cast<uint32_t *>(smem);             // [np]
     int32_t *Eacc = reinterpret_cast<int32_t *>(Wsm + g.np + 32);   // [32]; the 32 words before are read past a class
-    int32_t *PS = Eacc + 32;                                        // [32]
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     const int slot0 = (int)blockIdx.x * 32;
-    if (tid < 32) {
-        Eacc[tid] = 0;
-        PS[tid] = min(slot0 + tid, R - 1);
-    }
-    __syncthreads();
+    if (tid < 32) Eacc[tid] = 0;
     if (SRC == WORDS_RAW) {
+        // Four positions a thread at a time, and of a ragged word only the
+        // configurations that exist (the bits of the others stay 0, their energies
+        // are not written). us of a call, against one position at a time and 32 loads
+        // for it whatever R: n = 57,000, R = 1 403 -> 191, R = 33 608 -> 347; N = 7000,
+        // R = 300 136 -> 113.
+        const int live = min(32, R - slot0);
         bool wrong = false;
-        for (int i = tid; i < g.n; i += NT) {
-            uint32_t w = 0u;
+        for (int i0 = tid; i0 < g.n; i0 += 4 * NT) {
+            uint32_t w[4] = {0u, 0u, 0u, 0u};
 #pragma unroll 8
-            for (int r = 0; r < 32; ++r) {
-                const int v = __ldg(&in[(size_t)PS[r] * g.n + i]);
-                w |= (uint32_t)(v == 1) << msc_bit(r);
-                wrong |= v != 1 && v != -1;
+            for (int r = 0; r < live; ++r) {
+                const int8_t *x = in + (size_t)(slot0 + r) * g.n;
+                const int b = msc_bit(r);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int v = i0 + j * NT < g.n ? __ldg(&x[i0 + j * NT]) : 1;
+                    w[j] |= (uint32_t)(v == 1) << b;
+                    wrong |= v != 1 && v != -1;
+                }
             }
-            Wsm[pos[i]] = w;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (i0 + j * NT < g.n) Wsm[pos[i0 + j * NT]] = w[j];
         }
-        if (wrong) *bad = 1;
+        if (wrong && bad) *bad = 1;
     } else {
         uint32_t *row = reinterpret_cast<uint32_t *>(rows) + (size_t)(slot0 + msc_lane_replica(lane)) * g.nbw;
         for (int q = warp; 4 * q < g.nbw; q += NT / 32) {

@@ -1106,6 +1106,20 @@ struct RawRows {
           chunk((int32_t)std::min<size_t>((size_t)c->run.R, row_bytes(c) * c->run.Rpad / c->n)) {}
 };
 
+bool all_spins(const int8_t *x, size_t count) {   // eight bytes at a time: odd, and the upper seven bits equal
+    constexpr uint64_t ones = 0x0101010101010101ull;
+    uint64_t wrong = 0;
+    size_t t = 0;
+    for (; t + 8 <= count; t += 8) {
+        uint64_t v;
+        std::memcpy(&v, x + t, 8);
+        wrong |= (v & ones) ^ ones;
+        wrong |= (v & ~ones) ^ ((v >> 7) & ones) * 0xFEu;
+    }
+    for (; t < count; ++t) wrong |= x[t] != 1 && x[t] != -1;
+    return wrong == 0;
+}
+
 // Lexicographic minimum of the per-block records; returns the block or -1.
 int best_block(pa_ctx *c, int4 *rec) {
     RunState &r = c->run;
@@ -1343,6 +1357,9 @@ int pa_energies(pa_ctx *c, const int8_t *spins, int32_t R, int32_t *energies, in
     cudaStream_t st = c->stream();
     const pa::GraphDev g = c->gdev();
     const size_t raw = (size_t)R * c->n;
+    // Few spins are checked here, which costs less than clearing a flag for the kernel.
+    const bool host = raw <= 16384;
+    if (host && !all_spins(spins, raw)) return fail(c, PA_EINVAL, "spins must be +1/-1");
     const bool words = pa::word_energy_fits(g);   // else rows and fields, as at the start of an anneal
     DevBuf dx, dr, dh, dE;
     struct Drain {   // runs before the buffers are freed, on every return path
@@ -1353,17 +1370,17 @@ int pa_energies(pa_ctx *c, const int8_t *spins, int32_t R, int32_t *energies, in
         (!words && (!dr.alloc((size_t)R * c->np, st) || !dh.alloc(2 * (size_t)R * c->np, st))))
         return fail(c, PA_ENOMEM, "device allocation failed");
     std::vector<int32_t> E((size_t)R + 1);   // the last entry: a byte other than +1 / -1 was found
-    int32_t *bad = dE.as<int32_t>() + R;
+    int32_t *bad = host ? nullptr : dE.as<int32_t>() + R;
     PA_CUDA(c, copy(c, dx.p, spins, raw, cudaMemcpyHostToDevice, st, true));
-    PA_CUDA(c, cudaMemsetAsync(bad, 0, 4, st));
+    if (bad) PA_CUDA(c, cudaMemsetAsync(bad, 0, 4, st));
     if (words) {
         PA_CUDA(c, pa::launch_energy_raw(g, dx.as<int8_t>(), c->d_pos.as<int32_t>(), dE.as<int32_t>(), R, bad, st));
     } else {
-        PA_CUDA(c, pa::launch_check(dx.as<int8_t>(), raw, bad, st));
+        if (bad) PA_CUDA(c, pa::launch_check(dx.as<int8_t>(), raw, bad, st));
         PA_CUDA(c, pa::launch_rows_in(g, dx.as<int8_t>(), dr.as<int8_t>(), false, R, R, st));
         PA_CUDA(c, pa::launch_fields(g, dr.as<int8_t>(), dh.as<int16_t>(), dE.as<int32_t>(), R, st));
     }
-    PA_CUDA(c, copy(c, E.data(), dE.p, 4 * ((size_t)R + 1), cudaMemcpyDeviceToHost, st, true));
+    PA_CUDA(c, copy(c, E.data(), dE.p, 4 * ((size_t)R + (bad ? 1 : 0)), cudaMemcpyDeviceToHost, st, true));
     PA_CUDA(c, cudaStreamSynchronize(st));
     if (E[R]) return fail(c, PA_EINVAL, "spins must be +1/-1");
     for (int32_t s = 0; s < R; ++s) {
