@@ -1106,6 +1106,17 @@ struct RawRows {
           chunk((int32_t)std::min<size_t>((size_t)c->run.R, row_bytes(c) * c->run.Rpad / c->n)) {}
 };
 
+// Populations so small that the host permutes them faster than the device does,
+// which takes one to three launches, a wait for the check, and with bit rows a copy
+// for every eighth of the configurations. us of a call, device / host: set, N = 96,
+// R = 1 46 / 29, N = 300, R = 31 60 / 43, N = 96, R = 500 52 / 63; get, N = 96, R = 1
+// 41 / 30, N = 300, R = 31 40 / 39, N = 96, R = 500 44 / 64; with bit rows N = 96,
+// R = 33 set 83 / 28, get 74 / 30.
+bool by_host(const pa_ctx *c) {
+    const int32_t chunk = RawRows(c).chunk, copies = (c->run.R + chunk - 1) / chunk;
+    return (size_t)c->run.R * c->n <= 16384u * (size_t)std::min(copies, 6);
+}
+
 bool all_spins(const int8_t *x, size_t count) {   // eight bytes at a time: odd, and the upper seven bits equal
     constexpr uint64_t ones = 0x0101010101010101ull;
     uint64_t wrong = 0;
@@ -1287,9 +1298,21 @@ int pa_get_state(pa_ctx *c, int8_t *spins, int32_t *energies) {
     RunState &r = c->run;
     if (!r.begun) return fail(c, PA_ESTATE, "no anneal");
     if (int rc = pa_sync(c)) return rc;
-    if (spins) {   // vertex order, some rows at a time
+    const bool bits = bit_rows(r);
+    if (spins && by_host(c)) {
+        const size_t row = row_bytes(c);
+        std::vector<uint8_t> buf((size_t)r.R * row);
+        PA_CUDA(c, copy(c, buf.data(), r.spins[r.cur].p, buf.size(), cudaMemcpyDeviceToHost));
+        for (int32_t s = 0; s < r.R; ++s) {
+            const uint8_t *x = buf.data() + (size_t)s * row;
+            int8_t *out = spins + (size_t)s * c->n;
+            for (int32_t i = 0; i < c->n; ++i) {
+                const int32_t p = c->pos[i];
+                out[i] = bits ? (int8_t)(2 * ((x[p >> 3] >> (p & 7)) & 1) - 1) : (int8_t)x[p];
+            }
+        }
+    } else if (spins) {   // vertex order, some rows at a time
         const RawRows raw(c);
-        const bool bits = bit_rows(r);
         for (int32_t s0 = 0; s0 < r.R; s0 += raw.chunk) {
             const int32_t cnt = std::min(raw.chunk, r.R - s0);
             PA_CUDA(c, pa::launch_rows_out(c->gdev(), c->d_pos.as<int32_t>(),
@@ -1310,33 +1333,56 @@ int pa_set_state(pa_ctx *c, const int8_t *spins, int32_t steps_done) {
     RunState &r = c->run;
     if (!r.begun) return fail(c, PA_ESTATE, "pa_anneal_begin has not run");
     if (steps_done < 0 || steps_done > r.K) return fail(c, PA_EINVAL, "steps_done out of range");
+    // Up to 256 KB the host checks faster than the device, which takes a launch and a
+    // wait, and with bit rows a second upload (N = 4900, R = 31: 129 us of a call
+    // against 184).
+    const bool bits = bit_rows(r), host = by_host(c), checked = (size_t)r.R * c->n <= 262144u;
+    if (checked && !all_spins(spins, (size_t)r.R * c->n)) return fail(c, PA_EINVAL, "spins must be +1/-1");
     if (int rc = pa_sync(c)) return rc;
     // All configurations are checked before any replaces a row of the population.
     cudaStream_t st = c->stream();
     const pa::GraphDev g = c->gdev();
-    const RawRows raw(c);
-    int32_t *bad = r.parent.as<int32_t>();   // written by the next step before it is read
-    int32_t wrong = 0;
-    PA_CUDA(c, cudaMemsetAsync(bad, 0, 4, st));
-    for (int pass = 0; pass < 2; ++pass) {   // check, then take over
-        for (int32_t s0 = 0; s0 < r.R; s0 += raw.chunk) {
-            const int32_t cnt = std::min(raw.chunk, r.R - s0);
-            if (pass == 0 || raw.chunk < r.R)   // one chunk: it is still there
-                PA_CUDA(c, copy(c, raw.p, spins + (size_t)s0 * c->n, (size_t)cnt * c->n, cudaMemcpyHostToDevice, st,
-                                true));
-            if (pass == 0)
-                PA_CUDA(c, pa::launch_check(raw.p, (size_t)cnt * c->n, bad, st));
-            else
-                PA_CUDA(c, pa::launch_rows_in(g, raw.p, r.spins[r.cur].as<int8_t>() + row_bytes(c) * s0,
-                                              bit_rows(r), cnt, s0 + cnt == r.R ? r.Rpad - s0 : cnt, st));
+    std::vector<uint8_t> buf;   // pageable: lives until the stream has been waited for
+    if (host) {
+        const size_t row = row_bytes(c);
+        buf.assign((size_t)r.Rpad * row, 0);
+        for (int32_t s = 0; s < r.R; ++s) {
+            const int8_t *in = spins + (size_t)s * c->n;
+            uint8_t *x = buf.data() + (size_t)s * row;
+            for (int32_t i = 0; i < c->n; ++i) {
+                const int32_t p = c->pos[i];
+                if (bits) x[p >> 3] |= (uint8_t)((in[i] > 0) << (p & 7));
+                else x[p] = (uint8_t)in[i];
+            }
         }
-        if (pass == 0) {
-            PA_CUDA(c, cudaMemcpyAsync(&wrong, bad, 4, cudaMemcpyDeviceToHost, st));
-            PA_CUDA(c, cudaStreamSynchronize(st));
-            if (wrong) return fail(c, PA_EINVAL, "spins must be +1/-1");
+        for (int32_t s = r.R; s < r.Rpad; ++s)   // the padding rows repeat the last one
+            std::memcpy(buf.data() + (size_t)s * row, buf.data() + (size_t)(r.R - 1) * row, row);
+        PA_CUDA(c, copy(c, r.spins[r.cur].p, buf.data(), buf.size(), cudaMemcpyHostToDevice, st, true));
+    } else {
+        const RawRows raw(c);
+        int32_t *bad = r.parent.as<int32_t>();   // written by the next step before it is read
+        int32_t wrong = 0;
+        if (!checked) PA_CUDA(c, cudaMemsetAsync(bad, 0, 4, st));
+        for (int pass = checked ? 1 : 0; pass < 2; ++pass) {   // check, then take over
+            for (int32_t s0 = 0; s0 < r.R; s0 += raw.chunk) {
+                const int32_t cnt = std::min(raw.chunk, r.R - s0);
+                if (pass == 0 || checked || raw.chunk < r.R)   // one chunk after its check: it is still there
+                    PA_CUDA(c, copy(c, raw.p, spins + (size_t)s0 * c->n, (size_t)cnt * c->n, cudaMemcpyHostToDevice, st,
+                                    true));
+                if (pass == 0)
+                    PA_CUDA(c, pa::launch_check(raw.p, (size_t)cnt * c->n, bad, st));
+                else
+                    PA_CUDA(c, pa::launch_rows_in(g, raw.p, r.spins[r.cur].as<int8_t>() + row_bytes(c) * s0,
+                                                  bits, cnt, s0 + cnt == r.R ? r.Rpad - s0 : cnt, st));
+            }
+            if (pass == 0) {
+                PA_CUDA(c, cudaMemcpyAsync(&wrong, bad, 4, cudaMemcpyDeviceToHost, st));
+                PA_CUDA(c, cudaStreamSynchronize(st));
+                if (wrong) return fail(c, PA_EINVAL, "spins must be +1/-1");
+            }
         }
     }
-    if (bit_rows(r))
+    if (bits)
         PA_CUDA(c, pa::launch_energy_words(g, r.spins[r.cur].as<int8_t>(), r.E[r.cur].as<int32_t>(), r.Rpad, st));
     else
         PA_CUDA(c, pa::launch_fields(g, r.spins[r.cur].as<int8_t>(), r.fields[r.cur].as<int16_t>(),
