@@ -138,22 +138,22 @@ __global__ void k_shard_parents(ShardScratch s, int32_t n, unsigned long long P_
     }
 }
 
-// Rows in new-slot order, one CTA per row: bound by the copy's bandwidth. VEC:
-// rows of whole 16-byte units at 16-byte boundaries move four units per thread
+// Rows in new-slot order, one CTA (short rows: one warp) per row: bound by the
+// copy's bandwidth. VEC: rows of whole 16-byte units at 16-byte boundaries move four units per thread
 // at a time, otherwise byte by byte where the start or the end of a row is not
 // at a word boundary and word by word in between (the source words shifted into
 // place). 16384 rows of 7008 bytes: 216 us byte by byte, 33 us in units (7.0 TB/s read and written).
 constexpr int GATHER_THREADS = 128;
 
-template <bool VEC>
+template <bool VEC, int NT>
 __global__ void __launch_bounds__(GATHER_THREADS) k_shard_gather(const int8_t *__restrict__ spins,
                                                                  const int32_t *__restrict__ E, int32_t ncols,
                                                                  const int32_t *__restrict__ src, int32_t nout,
                                                                  int8_t *__restrict__ spins_out,
                                                                  int32_t *__restrict__ E_out) {
-    constexpr int NT = GATHER_THREADS;
-    const int tid = threadIdx.x;
-    for (int j = blockIdx.x; j < nout; j += gridDim.x) {
+    constexpr int ROWS = GATHER_THREADS / NT;   // rows of the CTA at a time
+    const int tid = threadIdx.x % NT;
+    for (int j = (int)blockIdx.x * ROWS + (int)threadIdx.x / NT; j < nout; j += (int)gridDim.x * ROWS) {
         const int32_t r = src[j];
         const int8_t *in = spins + (size_t)r * ncols;
         int8_t *out = spins_out + (size_t)j * ncols;
@@ -292,12 +292,16 @@ int pa_shard_gather(const int8_t *spins, const int32_t *energies, int32_t ncols,
     if (nout == 0) return PA_OK;   // a rank whose parents fill no new slot sends nothing
     if (!spins || !src || !spins_out || ncols < 1 || nout < 0 || (energies && !energies_out)) return PA_EINVAL;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const int grid = nout < 65536 ? nout : 65536;
     const uintptr_t mis = reinterpret_cast<uintptr_t>(spins) | reinterpret_cast<uintptr_t>(spins_out) | (uintptr_t)ncols;
-    if ((mis & 15) == 0)
-        k_shard_gather<true><<<grid, GATHER_THREADS, 0, st>>>(spins, energies, ncols, src, nout, spins_out, energies_out);
-    else
-        k_shard_gather<false><<<grid, GATHER_THREADS, 0, st>>>(spins, energies, ncols, src, nout, spins_out, energies_out);
+    // Rows of less than 768 bytes: a warp each, four in a CTA, and no more CTAs than
+    // fill the GPU a few times; a CTA for each costs more than its copy. us of the
+    // call, 65,536 rows, a CTA each / a warp each: 1 byte 52 / 25, 90 bytes 53 / 28,
+    // 600 bytes 52 / 29.
+    const bool vec = (mis & 15) == 0, brief = ncols < 768;
+    const int ctas = brief ? (nout - 1) / 4 + 1 : nout, most = brief ? 4096 : 65536;
+    auto *kernel = brief ? (vec ? &k_shard_gather<true, 32> : &k_shard_gather<false, 32>)
+                         : (vec ? &k_shard_gather<true, GATHER_THREADS> : &k_shard_gather<false, GATHER_THREADS>);
+    kernel<<<ctas < most ? ctas : most, GATHER_THREADS, 0, st>>>(spins, energies, ncols, src, nout, spins_out, energies_out);
     return cudaGetLastError() == cudaSuccess ? PA_OK : PA_ECUDA;
 }
 
