@@ -150,7 +150,8 @@ struct pa_ctx {
     std::vector<uint32_t> rp_p;         // position-order CSR
     std::vector<uint16_t> col_p;
     std::vector<int8_t> w_p;
-    DevBuf d_rp, d_col, d_w, d_vid, d_cls, d_pos, d_parity, d_prp, d_pcol, d_msl, d_csl, d_mvd, d_mcol;
+    DevBuf d_rp, d_col, d_w, d_vid, d_cls, d_pos, d_parity, d_prp, d_pcol, d_slices;
+    size_t at_msl = 0, at_mvd = 0, at_csl = 0;   // word offsets in d_slices, which begins with the units
     bool packed_ok = false, msc_rows = false, msc_big = false;
     RunState run;
     std::string err;
@@ -174,10 +175,11 @@ struct pa_ctx {
         g.prp = d_prp.as<uint32_t>();
         g.pcol = d_pcol.as<uint2>();
         g.packed_ok = packed_ok ? 1 : 0;
-        g.msl = msc_rows ? d_msl.as<uint2>() : nullptr;
-        g.csl = msc_rows ? d_csl.as<int32_t>() : nullptr;
-        g.mvd = msc_rows ? d_mvd.as<uint32_t>() : nullptr;
-        g.mcol = msc_rows ? d_mcol.p : nullptr;
+        const uint32_t *sl = msc_rows ? d_slices.as<uint32_t>() : nullptr;
+        g.msl = sl ? reinterpret_cast<const uint2 *>(sl + at_msl) : nullptr;
+        g.csl = sl ? reinterpret_cast<const int32_t *>(sl + at_csl) : nullptr;
+        g.mvd = sl ? sl + at_mvd : nullptr;
+        g.mcol = sl;
         g.mbig = msc_big ? 1 : 0;
         return g;
     }
@@ -466,7 +468,10 @@ int pa_create(pa_ctx **out, int32_t n, const uint32_t *row_ptr, const uint16_t *
     if (m2) h = fnv1a(h, col, sizeof(uint16_t) * m2);
     if (w && m2) h = fnv1a(h, w, m2);
     c->graph_hash = h;
-    // Upload.
+    // Upload: one copy behind the other, and one wait for all. The sources are pageable
+    // and live until then.
+    std::vector<uint32_t> prp, slab, par((c->np + 31) / 32, 0u);
+    std::vector<uint16_t> pcol;
     if (!c->d_rp.alloc(sizeof(uint32_t) * (n + 1)) || !c->d_col.alloc(sizeof(uint16_t) * (m2 + 8)) ||
         !c->d_w.alloc(m2 + 16) || !c->d_vid.alloc(sizeof(uint32_t) * n) ||
         !c->d_cls.alloc(sizeof(int32_t) * (ncol + 1)) || !c->d_pos.alloc(sizeof(int32_t) * n) ||
@@ -474,22 +479,22 @@ int pa_create(pa_ctx **out, int32_t n, const uint32_t *row_ptr, const uint16_t *
         delete c;
         return PA_ENOMEM;
     }
-    cudaError_t e1 = copy(c, c->d_rp.p, c->rp_p.data(), sizeof(uint32_t) * (n + 1), cudaMemcpyHostToDevice);
+    cudaError_t e1 = copy(c, c->d_rp.p, c->rp_p.data(), sizeof(uint32_t) * (n + 1), cudaMemcpyHostToDevice, nullptr, true);
     if (e1 == cudaSuccess && m2)
-        e1 = copy(c, c->d_col.p, c->col_p.data(), sizeof(uint16_t) * m2, cudaMemcpyHostToDevice);
+        e1 = copy(c, c->d_col.p, c->col_p.data(), sizeof(uint16_t) * m2, cudaMemcpyHostToDevice, nullptr, true);
     if (e1 == cudaSuccess && m2)
-        e1 = copy(c, c->d_w.p, c->w_p.data(), m2, cudaMemcpyHostToDevice);
+        e1 = copy(c, c->d_w.p, c->w_p.data(), m2, cudaMemcpyHostToDevice, nullptr, true);
     if (e1 == cudaSuccess)
-        e1 = copy(c, c->d_vid.p, c->vid.data(), sizeof(uint32_t) * n, cudaMemcpyHostToDevice);
+        e1 = copy(c, c->d_vid.p, c->vid.data(), sizeof(uint32_t) * n, cudaMemcpyHostToDevice, nullptr, true);
     if (e1 == cudaSuccess)
-        e1 = copy(c, c->d_cls.p, c->cls.data(), sizeof(int32_t) * (ncol + 1), cudaMemcpyHostToDevice);
+        e1 = copy(c, c->d_cls.p, c->cls.data(), sizeof(int32_t) * (ncol + 1), cudaMemcpyHostToDevice, nullptr, true);
     if (e1 == cudaSuccess)
-        e1 = copy(c, c->d_pos.p, c->pos.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice);
+        e1 = copy(c, c->d_pos.p, c->pos.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, nullptr, true);
     c->packed_ok = c->np + 32 <= 32768;
     if (e1 == cudaSuccess && c->packed_ok) {
-        std::vector<uint32_t> prp(n + 1, 0u);
+        prp.assign(n + 1, 0u);
         for (int32_t p = 0; p < n; ++p) prp[p + 1] = prp[p] + (c->rp_p[p + 1] - c->rp_p[p] + 3) / 4;
-        std::vector<uint16_t> pcol((size_t)prp[n] * 4 + 4);
+        pcol.resize((size_t)prp[n] * 4 + 4);
         for (int32_t p = 0; p < n; ++p) {
             size_t o = (size_t)prp[p] * 4;
             for (uint32_t e = c->rp_p[p]; e < c->rp_p[p + 1]; ++e, ++o)
@@ -497,11 +502,12 @@ int pa_create(pa_ctx **out, int32_t n, const uint32_t *row_ptr, const uint16_t *
             for (; o < (size_t)prp[p + 1] * 4; ++o) pcol[o] = (uint16_t)(c->np + (p & 31));
         }
         if (!c->d_prp.alloc(4 * (size_t)(n + 1)) || !c->d_pcol.alloc(2 * pcol.size())) {
+            cudaStreamSynchronize(nullptr);   // copies into the other buffers
             delete c;
             return PA_ENOMEM;
         }
-        e1 = copy(c, c->d_prp.p, prp.data(), 4 * (size_t)(n + 1), cudaMemcpyHostToDevice);
-        if (e1 == cudaSuccess) e1 = copy(c, c->d_pcol.p, pcol.data(), 2 * pcol.size(), cudaMemcpyHostToDevice);
+        e1 = copy(c, c->d_prp.p, prp.data(), 4 * (size_t)(n + 1), cudaMemcpyHostToDevice, nullptr, true);
+        if (e1 == cudaSuccess) e1 = copy(c, c->d_pcol.p, pcol.data(), 2 * pcol.size(), cudaMemcpyHostToDevice, nullptr, true);
     }
     c->msc_rows = c->maxdeg <= 127;
     // 16-bit entries take two operations each to unpack, 32-bit ones with a sign
@@ -510,62 +516,67 @@ int pa_create(pa_ctx **out, int32_t n, const uint32_t *row_ptr, const uint16_t *
     if (e1 == cudaSuccess && c->msc_rows) {
         std::vector<uint2> msl;
         std::vector<int32_t> csl(ncol + 1, 0);
-        std::vector<uint32_t> mvd;
         uint32_t units = 0;
         for (int32_t k = 0; k < ncol; ++k) {
             for (int32_t p0 = c->cls[k]; p0 < c->cls[k + 1]; p0 += 32) {
-                const int32_t p1 = std::min(p0 + 32, c->cls[k + 1]);
-                uint32_t most = 1;   // at least one unit: lanes without neighbours count their own word
-                for (int32_t p = p0; p < p1; ++p) most = std::max(most, (c->rp_p[p + 1] - c->rp_p[p] + 3) / 4);
+                // Degrees fall within a class. At least one unit: lanes without
+                // neighbours count their own word.
+                const uint32_t most = std::max(1u, (c->rp_p[p0 + 1] - c->rp_p[p0] + 3) / 4);
                 msl.push_back(make_uint2(units | most << 24, (uint32_t)p0));
-                for (int32_t p = p0; p < p0 + 32; ++p)
-                    mvd.push_back(p < p1 ? c->vid[p] | (c->rp_p[p + 1] - c->rp_p[p]) << 16 : 0x80000000u);
                 units += most;
             }
             csl[k + 1] = (int32_t)msl.size();
         }
-        const size_t esz = c->msc_big ? 4 : 2;
-        std::vector<unsigned char> mcol((size_t)units * 128 * esz);
-        for (const uint2 &d : msl) {
-            const size_t k = (size_t)(&d - msl.data());
-            for (uint32_t u = 0; u < d.x >> 24; ++u)
+        // One allocation and one upload: units, descriptors, vertices, class bounds.
+        const size_t ns = msl.size(), words = (size_t)units * (c->msc_big ? 128 : 64);
+        c->at_msl = words;
+        c->at_mvd = words + 2 * ns;
+        c->at_csl = c->at_mvd + 32 * ns;
+        slab.resize(c->at_csl + ncol + 1);
+        for (int32_t k = 0; k < ncol; ++k)
+            for (int32_t t = csl[k]; t < csl[k + 1]; ++t) {
+                const uint2 d = msl[t];
+                const uint32_t most = d.x >> 24;
                 for (uint32_t lane = 0; lane < 32; ++lane) {
-                    const bool live = !(mvd[32 * k + lane] >> 31);
-                    const uint32_t p = d.y + (live ? lane : 0u);
-                    const uint32_t e0 = c->rp_p[p] + 4 * u, e1p = live ? c->rp_p[p + 1] : 0u;
-                    uint32_t off[4], neg[4];
-                    for (uint32_t j = 0; j < 4; ++j) {
-                        const bool real = e0 + j < e1p;
-                        off[j] = 4u * (real ? (uint32_t)c->col_p[e0 + j] : p);
-                        neg[j] = real && c->w_p[e0 + j] < 0 ? 1u : 0u;
-                    }
-                    const size_t at = ((size_t)((d.x & 0xFFFFFFu) + u) * 32 + lane) * 4;
-                    for (uint32_t j = 0; j < 4; ++j) {
-                        if (c->msc_big)
-                            reinterpret_cast<uint32_t *>(mcol.data())[at + j] = off[j] | neg[j];
-                        else
-                            reinterpret_cast<uint16_t *>(mcol.data())[at + j] =
-                                (uint16_t)(off[j] | ((j & 1u) ? 0u : neg[j] | neg[j + 1] << 1));
+                    const bool live = (int32_t)(d.y + lane) < c->cls[k + 1];
+                    const uint32_t p = d.y + (live ? lane : 0u), e0 = c->rp_p[p], deg = live ? c->rp_p[p + 1] - e0 : 0u;
+                    slab[c->at_mvd + 32 * (size_t)t + lane] = live ? c->vid[p] | deg << 16 : 0x80000000u;
+                    const uint16_t *col_p = c->col_p.data() + e0;
+                    const int8_t *w_p = c->w_p.data() + e0;
+                    // Entry e of the lane: byte offset of its word, sign in bit 0.
+                    auto entry = [&](uint32_t e) { return e < deg ? 4u * col_p[e] | (w_p[e] < 0 ? 1u : 0u) : 4u * p; };
+                    uint32_t *at = slab.data() + ((size_t)(d.x & 0xFFFFFFu) * 32 + lane) * (c->msc_big ? 4 : 2);
+                    if (c->msc_big) {
+                        for (uint32_t e = 0; e < 4 * most; e += 4, at += 128)
+                            for (uint32_t j = 0; j < 4; ++j) at[j] = entry(e + j);
+                    } else {   // both signs of a pair in the low bits of its first entry
+                        for (uint32_t e = 0; e < 4 * most; e += 4, at += 64)
+                            for (uint32_t j = 0; j < 2; ++j) {
+                                const uint32_t x = entry(e + 2 * j), y = entry(e + 2 * j + 1);
+                                at[j] = x | (y & 1u) << 1 | (y & 0xFFFCu) << 16;
+                            }
                     }
                 }
+            }
+        for (size_t t = 0; t < ns; ++t) {
+            slab[c->at_msl + 2 * t] = msl[t].x;
+            slab[c->at_msl + 2 * t + 1] = msl[t].y;
         }
-        if (!c->d_msl.alloc(8 * msl.size()) || !c->d_csl.alloc(4 * csl.size()) || !c->d_mvd.alloc(4 * mvd.size()) ||
-            !c->d_mcol.alloc(mcol.size())) {
+        std::copy(csl.begin(), csl.end(), slab.begin() + c->at_csl);
+        if (!c->d_slices.alloc(4 * slab.size())) {
+            cudaStreamSynchronize(nullptr);   // copies into the other buffers
             delete c;
             return PA_ENOMEM;
         }
-        e1 = copy(c, c->d_msl.p, msl.data(), 8 * msl.size(), cudaMemcpyHostToDevice);
-        if (e1 == cudaSuccess) e1 = copy(c, c->d_csl.p, csl.data(), 4 * csl.size(), cudaMemcpyHostToDevice);
-        if (e1 == cudaSuccess) e1 = copy(c, c->d_mvd.p, mvd.data(), 4 * mvd.size(), cudaMemcpyHostToDevice);
-        if (e1 == cudaSuccess) e1 = copy(c, c->d_mcol.p, mcol.data(), mcol.size(), cudaMemcpyHostToDevice);
+        e1 = copy(c, c->d_slices.p, slab.data(), 4 * slab.size(), cudaMemcpyHostToDevice, nullptr, true);
     }
     if (e1 == cudaSuccess) {
-        std::vector<uint32_t> par((c->np + 31) / 32, 0u);
         for (int32_t p = 0; p < n; ++p)
             if ((c->rp_p[p + 1] - c->rp_p[p]) & 1u) par[p >> 5] |= 1u << (p & 31);
-        e1 = copy(c, c->d_parity.p, par.data(), sizeof(uint32_t) * par.size(), cudaMemcpyHostToDevice);
+        e1 = copy(c, c->d_parity.p, par.data(), sizeof(uint32_t) * par.size(), cudaMemcpyHostToDevice, nullptr, true);
     }
-    if (e1 != cudaSuccess) {
+    const cudaError_t e2 = cudaStreamSynchronize(nullptr);   // also where a copy failed
+    if (e1 != cudaSuccess || e2 != cudaSuccess) {
         delete c;
         cudaGetLastError();
         return PA_ECUDA;
