@@ -366,7 +366,8 @@ typedef struct {
 
 typedef struct {
     int64_t submitted, admitted, completed, queued, running;
-    int64_t bytes_in_use;     /* estimated device bytes of admitted requests */
+    int64_t bytes_in_use;     /* device bytes of admitted requests (an estimate
+                                 while a request is being set up) */
     int64_t attempts;         /* attempts of completed requests */
     double elapsed_ms;
 } pa_server_stats_t;

@@ -185,6 +185,19 @@ struct pa_ctx {
     }
 };
 
+size_t pa::context_bytes(const pa_ctx *c) {
+    const RunState &r = c->run;
+    size_t b = 0;
+    for (const DevBuf *d : {&c->d_rp, &c->d_col, &c->d_w, &c->d_vid, &c->d_cls, &c->d_pos, &c->d_parity, &c->d_prp, &c->d_pcol,
+                            &c->d_slices, &r.spins[0], &r.spins[1], &r.fields[0], &r.fields[1], &r.E[0], &r.E[1], &r.parent,
+                            &r.d_tables, &r.d_tidx, &r.d_qpow, &r.d_qblk, &r.rec_emin, &r.rec_A, &r.rec_T, &r.rec_o,
+                            &r.rec_acc, &r.rec_sweep, &r.rec_stamp, &r.rec_counts, &r.rec_nlm_pairs, &r.rec_nlm_flips,
+                            &r.rec_jsel, &r.best_rec, &r.best_cfg, &r.nlm_scratch, &r.ad_state, &r.ad_qsel, &r.ad_active,
+                            &r.ad_beta, &r.ad_part, &r.d_betas})
+        b += d->bytes;
+    return b;
+}
+
 namespace {
 
 // cudaMemcpy / cudaMemcpyAsync with per-context byte accounting.

@@ -15,6 +15,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+struct pa_ctx;
+
 namespace pa {
 
 // Full 32x32 -> 64-bit product (both halves from one wide multiply).
@@ -102,6 +104,9 @@ static __device__ __forceinline__ int32_t systematic_count_m(unsigned long long 
     const unsigned __int128 rhs = (unsigned __int128)T * (0x100000000ull - (unsigned long long)o);
     return (int32_t)(q + (lhs >= rhs ? 1ull : 0ull));
 }
+
+// Device bytes of a context's buffers.
+size_t context_bytes(const pa_ctx *c);
 
 constexpr int32_t EMIN_SENTINEL = 0x7F7F7F7F;  // byte-fillable "+infinity"
 constexpr int RS_CHUNK = 256;                   // slots per CTA of the ESS partials and the minimum

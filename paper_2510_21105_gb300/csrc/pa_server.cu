@@ -4,7 +4,8 @@
 //   admission   (admission thread) requests wait in FIFO order until their estimated device
 //               memory fits under the HBM budget (the oldest request is
 //               always admitted when nothing else runs), then get a context
-//               (graph upload) and an initialised population;
+//               (graph upload) and an initialised population, and are charged
+//               what these hold;
 //   ticks       (tick thread) each active request (at most n_streams at once, each on its
 //               own stream) gets its next steps_per_tick temperature steps
 //               enqueued; a request keeps at most two ticks in flight, so
@@ -33,6 +34,7 @@
 #include <vector>
 
 #include "../../include/pa.h"
+#include "pa_internal.cuh"
 
 namespace {
 
@@ -89,19 +91,26 @@ double ms_since(const pa_server *s) {
     return std::chrono::duration<double, std::milli>(Clock::now() - s->t0).count();
 }
 
-// Device bytes a request will hold: two population buffers (int8 spins +
-// int16 fields), energies, parents, resampling scratch, tables and records.
+// Device bytes a request may hold: two population buffers with their energies,
+// parents, best records, tables, per-step records and the graph's copies. Rows
+// are bits in a multi-spin-coded layout, else int8 spins and int16 fields; the
+// automatic layout may turn out to be either, so it counts as the larger. What
+// the context really holds takes the figure's place once it has been set up.
 size_t estimate_bytes(const Request &q) {
     const size_t np = (size_t)((q.n + 15) & ~15);
     const size_t rpad = (size_t)((q.R + 31) & ~31);
     const size_t m2 = q.rp.empty() ? 0 : q.rp.back();
+    const bool words = q.opts.variant == PA_VARIANT_MSC || q.opts.variant == PA_VARIANT_MSC_PAIR;
     int32_t maxdeg = 0;
     for (int32_t i = 0; i < q.n; ++i) maxdeg = std::max<int32_t>(maxdeg, (int32_t)(q.rp[i + 1] - q.rp[i]));
     const size_t K = (size_t)std::max(q.K, 1);
-    size_t b = 2 * np * rpad * 3 + 4 * 4 * rpad + 16 * 2 * rpad;
-    b += (rpad / 4) * (np + 16);                    // best records and configurations
-    b += K * (size_t)(maxdeg + 1) * 4 + K * 32 * 8 + K * (64 + 4 * (size_t)std::max(q.S, 1));
-    b += m2 * 6 + np * 24;                          // graph copies
+    size_t b = 2 * rpad * (words ? (np + 127) / 128 * 16 : 3 * np) + 3 * 4 * rpad;
+    b += (rpad / (words ? 32 : 4)) * (np + 16);     // best records and configurations
+    b += K * (size_t)(maxdeg + 1) * 4 + K * 32 * 8 + K * (80 + 4 * (size_t)std::max(q.S, 1));
+    // Graph copies: entries, weights, padded rows, slices of 32 rows of up to the
+    // largest degree for each of at most maxdeg + 1 classes.
+    const size_t d = (size_t)std::min(maxdeg, 127);
+    b += m2 * 9 + np * 44 + 128 * (d + 5) * (d + 1);
     if (q.opts.nlm_period > 0) b += (size_t)q.R * 12 + 16384;
     return b + (1u << 20);
 }
@@ -177,7 +186,10 @@ bool admit_one(pa_server *s, const std::shared_ptr<Request> &q) {
         finish(s, *q, rc);
         return false;
     }
+    const size_t held = pa::context_bytes(q->ctx);
     std::lock_guard<std::mutex> lock(s->mu);
+    s->used = s->used - q->bytes + held;
+    q->bytes = held;
     q->status = 1;
     s->active.push_back(q);
     s->stats.admitted += 1;
