@@ -878,14 +878,17 @@ int enqueue_step(pa_ctx *c, int32_t k, cudaStream_t st, bool time_sweep, bool ch
     const pa_anneal_opts &o = r.opts;
     const int cur = r.cur, nxt = 1 - r.cur;
     // chained: the stream's previous launch is this anneal's previous step, and no
-    // other anneal waits for the slots that an early launch would hold. Not across
+    // other anneal that the library runs (a batch's, a server's) waits for the slots
+    // that an early launch would hold. Not across
     // a second stream's join or a timing event. Gaps of 3 to 4 us between launches
     // fall to about 2; whole anneals before / after: adaptive schedule, R = 2048,
     // 42.9 / 40.2 ms, n = 500 and degree 250 6.90 / 6.69 ms, n = 800 5.59 / 5.20,
     // 12 steps of a small graph 0.68 / 0.64. The resampling step lets the sweep
     // start only after its own wait: with the sweep's CTAs placed while the last
     // ones of the step before still ran, they stacked up on the SMs that were free
-    // (adaptive schedule 54 ms).
+    // (adaptive schedule 54 ms). Beside other anneals the waiting CTAs cost more than
+    // the gaps: batch of nine 48.7 ms without, 49.1 with; Poisson trace of 64 served
+    // requests 1.659 against 1.651e12 attempts/s (three runs each).
     const bool early = chained && !r.split && !time_sweep;
     pa::ResampleArgs ra{};
     ra.E = r.E[cur].as<int32_t>();
@@ -1038,9 +1041,7 @@ int enqueue_step(pa_ctx *c, int32_t k, cudaStream_t st, bool time_sweep, bool ch
 }
 }  // namespace
 
-extern "C" {
-
-int pa_anneal_run(pa_ctx *c, int32_t k_end) {
+int pa::anneal_run(pa_ctx *c, int32_t k_end, bool alone) {
     if (!c) return PA_EINVAL;
     RunState &r = c->run;
     if (!r.begun) return fail(c, PA_ESTATE, "pa_anneal_begin has not run");
@@ -1078,7 +1079,7 @@ int pa_anneal_run(pa_ctx *c, int32_t k_end) {
     for (int32_t k = r.k_done; k < k_end && !ended;) {
         const int32_t kc = poll ? std::min(k_end, k + END_CHUNK) : k_end;
         for (; k < kc; ++k)
-            if (int rc = enqueue_step(c, k, st, r.opts.time_kernels != 0, k > r.k_done)) return rc;
+            if (int rc = enqueue_step(c, k, st, r.opts.time_kernels != 0, alone && k > r.k_done)) return rc;
         if (!poll || k >= k_end) break;
         const int slot = chunk % END_WINDOW;
         if (chunk >= END_WINDOW) {   // the slot's earlier copy: wait for it, then read it
@@ -1095,6 +1096,10 @@ int pa_anneal_run(pa_ctx *c, int32_t k_end) {
     r.k_done = k_end;
     return PA_OK;
 }
+
+extern "C" {
+
+int pa_anneal_run(pa_ctx *c, int32_t k_end) { return pa::anneal_run(c, k_end, true); }
 
 int pa_sync(pa_ctx *c) {
     if (!c) return PA_EINVAL;

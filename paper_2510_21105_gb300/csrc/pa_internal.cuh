@@ -107,6 +107,8 @@ static __device__ __forceinline__ int32_t systematic_count_m(unsigned long long 
 
 // Device bytes of a context's buffers.
 size_t context_bytes(const pa_ctx *c);
+// pa_anneal_run; alone: no other anneal shares the device.
+int anneal_run(pa_ctx *c, int32_t k_end, bool alone);
 
 constexpr int32_t EMIN_SENTINEL = 0x7F7F7F7F;  // byte-fillable "+infinity"
 constexpr int RS_CHUNK = 256;                   // slots per CTA of the ESS partials and the minimum

@@ -276,7 +276,7 @@ void worker_loop(pa_server *s) {
             }
             if (held || q->k_enq >= q->K || q->inflight.size() >= 2) continue;
             const int32_t k_end = std::min(q->K, q->k_enq + s->steps_per_tick);
-            if (pa_anneal_run(q->ctx, k_end) != PA_OK) {
+            if (pa::anneal_run(q->ctx, k_end, act.size() == 1) != PA_OK) {
                 finish(s, *q, PA_ECUDA);
                 continue;
             }
