@@ -382,22 +382,21 @@ def run_ours(args, rank, world, dist):
 
     for _ in range(args.warmup):
         one()
-    variant_run = ann.stats()["variant"]
-    if variant_run == 1:
-        layout, kernel = "multi-spin coded (32 replicas per 32-bit word)", ("k_sweep_msc", args.threads or 256)
-        sms = torch.cuda.get_device_properties(0).multi_processor_count
-        words = (R + 31) // 32
-        if words > sms and words % sms:
-            layout += f"; {words // sms * sms} words in one-CTA blocks + {words % sms} in CTA pairs, concurrently"
-            kernel = ("k_sweep_msc+pair", args.threads or 256)
-    elif variant_run == 3:
-        layout = "multi-spin coded, a thread-block cluster per 32-replica word"
-        kernel = ("k_sweep_msc_pair", 256)
+    shape = ann.sweep_shape()
+    if shape["variant"] in (1, 3):
+        layout = "multi-spin coded (32 replicas per 32-bit word)"
+        kernel = ("k_sweep_msc", shape["threads"])
+        if shape["tail_blocks"]:
+            layout += f"; {shape['blocks']} words in one-CTA blocks + {shape['tail_blocks']} in CTA pairs, concurrently"
+            kernel = ("k_sweep_msc+pair", shape["threads"])
+        elif shape["ctas"] > 1:
+            layout += f", a cluster of {shape['ctas']} CTAs per word"
+            kernel = ("k_sweep_msc_pair", shape["threads"])
     else:
         fb = args.field_bits if args.field_bits else (7 if g.maxdeg <= 127 else 16)
         layout = {7: "packed byte (spin bit + 7-bit field)", 8: "int8 spin + int8 field",
                   16: "int8 spin + int16 field"}[fb]
-        kernel = ("k_sweep_packed" if fb == 7 else "k_sweep", args.threads or (128 if fb == 7 else 512))
+        kernel = ("k_sweep_small" if shape["small_graph"] else "k_sweep_packed" if fb == 7 else "k_sweep", shape["threads"])
     peaks, peaks_src = load_peaks()
     probe = B.probe_peaks(sh)   # integer, Philox and shared-memory peaks of this GPU (a few ms)
     # timed region: device-resident inputs, K anneals
