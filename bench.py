@@ -18,6 +18,7 @@ from __future__ import annotations
 import argparse
 import collections
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -252,9 +253,10 @@ def msc_planes(max_degree: int) -> int:
 def msc_ops_per_attempt(mean_degree: float, max_degree: int = 31) -> float:
     """Algorithmic integer instructions of one multi-spin-coded attempt: one
     item (one position of a 32-replica word) divided by its 32 attempts, in the
-    byte-per-replica formulation. The kernel now decides in bit planes; the
-    count stays that of the byte formulation, so that the reported fraction of
-    the integer peak compares across builds.
+    byte-per-replica formulation of earlier builds. The kernel decides in bit
+    planes now and executes none of the count bytes, look-ups and byte energies
+    below (msc_plane_ops_per_attempt counts what it does); this count stays, so
+    that "frac" compares across builds.
       bond counting   per 4 bonds, three-input logic ops of the carry-save
                       adders: 7 + 2 (NPL - 3) with the planes kept
                       complemented (NPL >= 4), 13 with plain adders from
@@ -279,6 +281,37 @@ def msc_ops_per_attempt(mean_degree: float, max_degree: int = 31) -> float:
     return per_item / 32.0
 
 
+def msc_uncertain_levels(beta: float, max_degree: int) -> int:
+    """Counter values e (m = 2e + 1 or 2e + 2, m at most the degree) that have a
+    threshold floor(2^32 exp(-2 beta m)) with a non-zero top byte."""
+    m = max_degree if beta <= 0 else min(max_degree, int(8 * math.log(2.0) / (2 * beta)))
+    return (m + 1) // 2
+
+
+def msc_plane_ops_per_attempt(mean_degree: float, max_degree: int, betas) -> float:
+    """Algorithmic integer instructions of one attempt in the bit-plane form that
+    the kernel runs, averaged over a schedule; per item of 32 attempts:
+      uniforms   two Philox4x32-10 calls of 10 rounds x (2 widening multiplies +
+                 2 three-input xors), less the products of rounds 1-3 that the
+                 two share (2 of them the same for the whole launch): 73
+      bonds      counter start and end N planes each; per 8 bonds 7 full adders
+                 of two operations and one carry to ripple (N = counter planes)
+      decision   L values of m with a threshold that has a top byte: one to
+                 select the replicas, 8 to or in its planes; transpose of the
+                 uniforms 12 swaps x 4, comparison of 8 planes x 2. L = 0: the
+                 fold of the bytes to "zero or not", 35. Acceptance and tie 2
+      energy     N + 6 (N + 7 up to 4 planes) accumulator planes, two each, and
+                 a mask per counter plane
+    Loads, addresses, loop control, barriers, ties, and rows at load and store
+    are not counted."""
+    n = msc_planes(max_degree)
+    acc = n + (6 if n > 4 else 7)
+    item = 73 + 2 * n + (13 + 2 * (n - 3)) / 8.0 * mean_degree + (n - 2) // 2 + 2 + (3 * n + 2 * (acc - n))
+    levels = [msc_uncertain_levels(float(b), max_degree) for b in betas]
+    item += sum(48 + 16 + 9 * L if L else 35 for L in levels) / len(levels)
+    return item / 32.0
+
+
 def packed_ops_per_attempt(mean_degree: float, accept_rate: float) -> float:
     """4-replica layouts: one Philox call per 4 attempts (40 ops), the
     decision (5) and the field updates of an accepted flip (2 per bond)."""
@@ -298,7 +331,7 @@ def smem_bytes_per_attempt(kernel, mean_degree, accept_rate):
 
 
 def sweep_roofline(stats, attempts_per_launch, probe, clk_mhz, kernel, mean_degree, accept_rate, sms=SMS,
-                   max_degree=31):
+                   max_degree=31, betas=None):
     """Roofline of the sweep (the dominant kernel): integer-issue bound.
     probe: pa_probe_peaks of the device (measured peaks) or None."""
     launches = max(stats["sweep_launches"], 1)
@@ -311,6 +344,7 @@ def sweep_roofline(stats, attempts_per_launch, probe, clk_mhz, kernel, mean_degr
     achieved = aps * ops / 1e12
     derived = sms * INT_LANES_PER_SM * clk_mhz * 1e6 / 1e12
     peak = probe["int_ops_per_s"] / 1e12 if probe else derived
+    planes = msc_plane_ops_per_attempt(mean_degree, max_degree, betas) if msc and betas is not None else None
     sbpa = smem_bytes_per_attempt(kernel, mean_degree, accept_rate)
     smem_derived = sms * SMEM_BYTES_PER_SM * clk_mhz * 1e6
     smem_peak = probe["smem_bytes_per_s"] if probe else smem_derived
@@ -328,6 +362,8 @@ def sweep_roofline(stats, attempts_per_launch, probe, clk_mhz, kernel, mean_degr
             "smem_frac_vs_derived": aps * sbpa / smem_derived,
             "smem_target_met": aps * sbpa / smem_peak >= 0.5,
             "philox_frac": (aps * (0.25 if msc else 1.0) / probe["philox_words_per_s"]) if probe else None,
+            # The same rate against what the bit-plane form executes at least (the fraction to quote for this build).
+            "ops_per_attempt_planes": planes, "frac_planes": aps * planes / 1e12 / peak if planes else None,
             # The same rate against the count of the first formulation (plain carry-save adders, one table lookup
             # per replica: (4.5 d + 288)/32), which stays fixed across builds and so tracks the kernel's progress.
             "ops_per_attempt_first_formulation": (4.5 * mean_degree + 288.0) / 32.0 if msc else None,
@@ -429,7 +465,7 @@ def run_ours(args, rank, world, dist):
     clocks = clk.summary()
     clk_mhz = clocks.get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
     roof = sweep_roofline(stats_acc, g.n * R * S, probe, clk_mhz, kernel, 2.0 * g.m / g.n, acc_rate,
-                          sms=probe["sms"], max_degree=int(g.maxdeg))
+                          sms=probe["sms"], max_degree=int(g.maxdeg), betas=betas)
     ann.close()
 
     # end to end through the C-ABI with host buffers (pinned), copies inside the region
