@@ -1872,8 +1872,9 @@ const void *word_energy_kernel(int src) {
 
 cudaError_t launch_word_energy(int src, GraphDev g, const int8_t *in, const int32_t *pos, int8_t *rows, int32_t *E,
                                int32_t R, int32_t words, uint32_t key0, uint32_t key1, int32_t *bad, cudaStream_t st) {
-    const void *fn = g.wt ? (g.mbig ? word_energy_kernel<true, true>(src) : word_energy_kernel<true, false>(src))
-                          : (g.mbig ? word_energy_kernel<false, true>(src) : word_energy_kernel<false, false>(src));
+    // Unsigned graphs have 32-bit entries at every size.
+    const void *fn = !g.wt ? word_energy_kernel<false, true>(src)
+                     : g.mbig ? word_energy_kernel<true, true>(src) : word_energy_kernel<true, false>(src);
     const size_t smem = word_energy_smem(g);
     if (cudaError_t e = raise_smem(const_cast<void *>(fn), smem)) return e;
     void *args[] = {&g, &in, &pos, &rows, &E, &R, &key0, &key1, &bad};
@@ -1922,8 +1923,8 @@ void *kernel_ptr(bool queued) {
 
 void *select_kernel(int G, int fb, bool weighted, int threads, int mmax, bool big, bool small, bool queued) {
     if (fb == 1 || fb == 2) {
-        if (big) return weighted ? msc_kernel<true, true>(mmax, fb == 2) : msc_kernel<false, true>(mmax, fb == 2);
-        return weighted ? msc_kernel<true, false>(mmax, fb == 2) : msc_kernel<false, false>(mmax, fb == 2);
+        if (!weighted) return msc_kernel<false, true>(mmax, fb == 2);   // 32-bit entries at every size
+        return big ? msc_kernel<true, true>(mmax, fb == 2) : msc_kernel<true, false>(mmax, fb == 2);
     }
     if (small) {
         if (fb == 7) return weighted ? small_kernel<7, true>(threads) : small_kernel<7, false>(threads);
