@@ -164,6 +164,8 @@ typedef struct {
                                  each fit one round of a CTA */
     int32_t row_queue;        /* 1: accepted items of the int8/int16 kernel go
                                  through a queue of the block */
+    int32_t early;            /* 1: in a run of steps the sweep is launched
+                                 while the resampling before it ends */
     int32_t tail_blocks, tail_threads, tail_ctas;
 } pa_sweep_shape_t;
 

@@ -50,8 +50,8 @@ class pa_stats_t(C.Structure):
 
 class pa_sweep_shape_t(C.Structure):
     _fields_ = [(name, C.c_int32) for name in
-                ("variant", "replicas", "blocks", "threads", "ctas", "small_graph", "row_queue", "tail_blocks",
-                 "tail_threads", "tail_ctas")]
+                ("variant", "replicas", "blocks", "threads", "ctas", "small_graph", "row_queue", "early",
+                 "tail_blocks", "tail_threads", "tail_ctas")]
 
 
 class pa_step_arrays(C.Structure):

@@ -285,6 +285,8 @@ cudaError_t launch_rs_min(const ResampleArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+int rs_step_ctas(int32_t R) { return cluster_shape(R, RS_THREADS).ctas; }
+
 cudaError_t launch_rs_step(const ResampleArgs &a, cudaStream_t st, bool early) {
     const ClusterShape shape = cluster_shape(a.R, RS_THREADS);
     auto *kernel = shape.k == 1   ? &k_rs_step<1>

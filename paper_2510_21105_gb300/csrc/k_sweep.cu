@@ -2164,6 +2164,20 @@ cudaError_t launch_sweep(const SweepConfig &cfg, const SweepArgs &a, cudaStream_
     return cudaLaunchKernelExC(&lc, fn, args);
 }
 
+// SMs that hold a CTA of the resampling get none of the sweep's while others have
+// room, so a sweep of at most q blocks per SM is spread as evenly as ever if the other
+// SMs take it with q each, or have no room for more. Otherwise some SM runs q + 1
+// (us per step of 2 sweeps on 152 SMs beside 8 CTAs, early / not: torus N = 4900 144
+// words 42.9 / 44.8, 146 words 65.0 / 44.6, 288 words 71.2 / 72.8, 296 words 91.4 /
+// 72.9, 430 words 94.0 / 96.1, 440 words 115.7 / 96.7, 608 words, all slots, 124.8 /
+// 126.7; packed, 720 blocks 112.5 / 114.3, 740 blocks 127.4 / 114.2). Clusters need
+// free SMs side by side (of four CTAs: 34 words 29.3 / 30.9, 36 words 37.7 / 31.0).
+bool sweep_spreads_beside(const SweepConfig &cfg, int beside, int sms) {
+    const bool clusters = cfg.field_bits == 2;
+    const int q = (cfg.grid + sms - 1) / sms, taken = beside + (clusters ? 2 * cfg.cluster : 0);
+    return (!clusters && cfg.occ == q) || cfg.grid <= q * (sms - taken);
+}
+
 bool word_energy_fits(const GraphDev &g) {
     int dev = 0, limit = 0;
     cudaGetDevice(&dev);

@@ -128,6 +128,7 @@ struct RunState {
     double ad_delta = 0.0;
     int32_t ad_nmax = 0;
     int cur = 0;
+    bool early_sweep = false;            // the sweep may be placed while the resampling ends
     bool have_emin = false;              // rec_emin[k_done] holds the minimum of the population's energies
     pa::SweepConfig sweep{};
     int variant = PA_VARIANT_I8;
@@ -740,6 +741,7 @@ int pa_anneal_begin(pa_ctx *c, const double *betas, int32_t K, int32_t R, int32_
             r.blk_base2 = wm;
         }
     }
+    r.early_sweep = !r.split && pa::sweep_spreads_beside(r.sweep, pa::rs_step_ctas(R), sms);
     r.nch = (R + pa::RS_CHUNK - 1) / pa::RS_CHUNK;
     const int32_t mmax = c->maxdeg;
     // Host tables.
@@ -1008,7 +1010,7 @@ int enqueue_step(pa_ctx *c, int32_t k, cudaStream_t st, bool time_sweep, bool ch
         PA_CUDA(c, cudaEventRecord(r.ev_join, r.st2));
         r.launches += 1;
     }
-    PA_CUDA(c, pa::launch_sweep(r.sweep, sa, st, early));
+    PA_CUDA(c, pa::launch_sweep(r.sweep, sa, st, early && r.early_sweep));
     if (r.split) PA_CUDA(c, cudaStreamWaitEvent(st, r.ev_join, 0));
     if (time_sweep) PA_CUDA(c, cudaEventRecord(s1, st));
     r.launches += 1;
@@ -1487,6 +1489,7 @@ int pa_sweep_shape(pa_ctx *c, pa_sweep_shape_t *out) {
     out->threads = r.sweep.threads;
     out->ctas = r.sweep.field_bits == 2 ? r.sweep.cluster : 1;
     out->small_graph = r.sweep.small ? 1 : 0;
+    out->early = r.early_sweep ? 1 : 0;
     out->row_queue = r.variant == PA_VARIANT_I8 && r.sweep.qcap > 0 ? 1 : 0;
     if (r.split) {
         out->tail_blocks = r.nblk2;

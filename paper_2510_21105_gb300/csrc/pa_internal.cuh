@@ -214,6 +214,7 @@ cudaError_t launch_check(const int8_t *raw, size_t bytes, int32_t *bad, cudaStre
 // Minimum of the energies; the step's start stamp, weights and parents.
 cudaError_t launch_rs_min(const ResampleArgs &a, cudaStream_t st);
 cudaError_t launch_rs_step(const ResampleArgs &a, cudaStream_t st, bool early = false);
+int rs_step_ctas(int32_t R);   // CTAs of its one cluster
 cudaError_t launch_stamp(unsigned long long *stamp, cudaStream_t st);
 
 struct SweepConfig {
@@ -251,5 +252,8 @@ cudaError_t sweep_configure(const GraphDev &g, int R, int G, int field_bits, int
 // CTAs per word that the multi-spin-coded layout should use for `words` words (1: no cluster).
 int msc_cluster(const GraphDev &g, int words, int sms);
 cudaError_t launch_sweep(const SweepConfig &cfg, const SweepArgs &a, cudaStream_t st, bool early = false);
+// Whether a sweep placed while `beside` CTAs of the resampling still hold an SM
+// each is spread over the SMs as evenly as without them.
+bool sweep_spreads_beside(const SweepConfig &cfg, int beside, int sms);
 
 }  // namespace pa
