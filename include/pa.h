@@ -120,16 +120,17 @@ typedef struct {
                                  do not advance resample with q = 1 (identity).
                                  0 = off (default) */
     int32_t reheat_back;      /* entries a reheat steps back (>= 1) */
-    int32_t msc_no_split;     /* PA_VARIANT_MSC: 0 (default) = when the
-                                 32-replica words are more than, and not a
-                                 multiple of, the SMs, the first
-                                 (words / SMs) * SMs words run in one-CTA
-                                 blocks and the rest concurrently in CTA pairs
-                                 on a second stream, so that every SM carries
-                                 the same work; 1 = every word in one-CTA
-                                 blocks, for callers whose other work (a
-                                 batch, a loaded server) fills the SMs anyway.
-                                 Results do not depend on it. */
+    int32_t msc_no_split;     /* PA_VARIANT_MSC: 0 (default) = the 32-replica
+                                 words past the largest multiple of the SM
+                                 count run in CTA pairs on a second stream
+                                 beside the others, in one-CTA blocks, where
+                                 that evens out the last wave of blocks (by
+                                 the number of words left over, the blocks an
+                                 SM holds and the size of the colour classes);
+                                 1 = every word in one-CTA blocks, for callers
+                                 whose other work (a batch, a loaded server)
+                                 fills the SMs anyway. Results do not depend
+                                 on it. */
 } pa_anneal_opts;
 
 typedef struct {
@@ -269,8 +270,8 @@ int pa_set_state(pa_ctx *ctx, const int8_t *spins, int32_t steps_done);
 
 /* Energies E = sum over edges w_ij x_i x_j and cuts (W - E)/2 (Eq. 1 and
  * the sign convention of Sec. 2) of R host configurations int8[R][n] (+1/-1,
- * vertex order), evaluated on the device. Independent of any anneal: a verifier for configurations read
- * back from files (e.g. the hexadecimal format of Sec. 3). energies int32[R]
+ * vertex order), evaluated on the device. Independent of any anneal: a
+ * verifier for configurations read back from files (e.g. the hexadecimal format of Sec. 3). energies int32[R]
  * and cuts int64[R] are caller buffers; either may be NULL. R = 0 is a no-op.
  * Allocates R*(n + 4) bytes of device memory for the call, R*(4n + 4) on graphs
  * without multi-spin-coded layouts. Errors: PA_EINVAL

@@ -95,7 +95,7 @@ def _anneal(argv):
     p.add_argument("--replicas-per-cta", type=int, default=0)
     p.add_argument("--threads", type=int, default=0)
     p.add_argument("--variant", type=int, default=2,
-                   help="0 int8/int16 fields, 1 multi-spin coded, 2 automatic (default), 3 CTA pairs")
+                   help="0 int8/int16 fields, 1 multi-spin coded, 2 automatic (default), 3 clusters of CTAs")
     p.add_argument("--hex", action="store_true")
     p.add_argument("--save-hex", default=None)
     p.add_argument("--curve", default=None, help="write step,beta,t_ms,best_cut CSV")

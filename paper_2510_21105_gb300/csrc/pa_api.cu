@@ -4,8 +4,8 @@
 // renumbering by colour), the per-step host tables (acceptance thresholds
 // floor(2^32 exp(-beta_k 2m)) and the squarings of q_k = exp(-dbeta_k)), the
 // device population, and the launch sequence of one temperature step:
-//   resample (3 small kernels) -> sweep kernel (fused parent copy + S sweeps
-//   + best tracking) -> non-local move when due.
+//   resample (one cluster launch) -> sweep kernel (fused parent copy + S sweeps
+//   + best tracking + the next step's minimum energy) -> non-local move when due.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -312,7 +312,7 @@ int validate_opts(pa_ctx *c, const pa_anneal_opts &o) {
     if (msc && c->maxdeg > 127)
         return fail(c, PA_EINVAL, "the multi-spin-coded variant needs max degree <= 127");
     if (msc && o.threads_per_cta > 256)
-        return fail(c, PA_EINVAL, "the multi-spin-coded variant runs at most 256 threads per CTA");
+        return fail(c, PA_EINVAL, "the multi-spin-coded variant takes threads_per_cta up to 256 (and chooses 256 or 512 itself)");
     if (o.nlm_period < 0) return fail(c, PA_EINVAL, "nlm_period < 0");
     if (o.nlm_kind != 0 && o.nlm_kind != 1) return fail(c, PA_EINVAL, "nlm_kind must be 0 or 1");
     if (o.nlm_kind == 1 && (o.nlm_block < 1 || o.nlm_block > 1024))

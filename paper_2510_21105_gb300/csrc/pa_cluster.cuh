@@ -1,7 +1,7 @@
 // pa_cluster.cuh -- the weight arithmetic of one resampling over a population
-// (or one rank's shard of it) in a single thread-block cluster: used by the
-// resampling entry points on caller buffers, where a launch has to do all of
-// it by itself.
+// (or one rank's shard of it) in a single thread-block cluster: every step's
+// resampling (k_rs_step) and the resampling entry points on caller buffers,
+// where a launch does all of it by itself.
 //
 // n slots, padded with zero weights to L = NT K C: CTA c of the C <= 8 CTAs of
 // NT threads holds the aligned range of L / C slots, thread t of it K
