@@ -49,7 +49,7 @@ def shape_key(g, R, S) -> str:
 
 def candidates_for(g, context="alone", candidates=None):
     """The candidates a graph admits in a context. "saturated" drops the
-    CTA-pair kernel, which only gains by balancing one instance over the SMs
+    cluster kernel, which only gains by spreading one instance over the SMs
     (when other work fills the GPU that balance comes for free and its
     cluster barriers are pure cost), and for the same reason runs the
     multi-spin-coded layout with every word in one-CTA blocks (msc_no_split),

@@ -292,7 +292,8 @@ void collect_events(RunState &r) {
 // 470 words 341 / 376, 560 words 439 / 400, 1000 words 672 / 740, 1200 words 838 /
 // 791; torus N = 10000 200 words 168 / 207, 470 words 338 / 378, 1000 words 687 /
 // 750; n = 2000, degree 12 (14 slices) 200 words 115 / 101, 512 words 164 / 157;
-// 18,000-vertex planar 200 words 359 / 399, 270 words 631 / 451.
+// 18,000-vertex planar, two blocks of 512 threads in an SM, 200 words 335 / 401, 240
+// words 454 / 401.
 bool pair_tail(int32_t words, int sms, int occ, int32_t slices) {
     const int32_t cap = occ * sms, rem = words % cap, q = rem / sms, r = rem % sms;
     if (r == 0 || slices < 24 || words < sms) return false;
@@ -888,9 +889,9 @@ int enqueue_step(pa_ctx *c, int32_t k, cudaStream_t st, bool time_sweep, bool ch
     // 12 steps of a small graph 0.68 / 0.64. The resampling step lets the sweep
     // start only after its own wait: with the sweep's CTAs placed while the last
     // ones of the step before still ran, they stacked up on the SMs that were free
-    // (adaptive schedule 54 ms). Beside other anneals the waiting CTAs cost more than
-    // the gaps: batch of nine 48.7 ms without, 49.1 with; Poisson trace of 64 served
-    // requests 1.659 against 1.651e12 attempts/s (three runs each).
+    // (adaptive schedule 54 ms). Beside other anneals the waiting CTAs give nothing:
+    // batch of nine 48.7 ms without early launches, 49.1 with; Poisson trace of 64
+    // served requests 1.6515 against 1.6508e12 attempts/s (five runs each).
     const bool early = chained && !r.split && !time_sweep;
     pa::ResampleArgs ra{};
     ra.E = r.E[cur].as<int32_t>();
